@@ -305,6 +305,14 @@ int gbd_tc_rate(int32_t device, int32_t prec, int32_t M, int32_t N, int32_t K, i
  * |difference| and max |FP64 result|. */
 int gbd_gemm_tc_selftest(gbd_ctx *ctx, int32_t M, int32_t N, int32_t K, int32_t nterms, int32_t flags, int32_t prec,
                          uint64_t seed, double *max_err, double *max_ref);
+/* The FP64 grouped GEMM on host arrays: C (M x N) = beta C + alpha sum_t
+ * op(A_t) op(B_t), nterms terms of K columns, each block dense row-major and
+ * back to back; flags 1 = A_t stored transposed (K x M), 2 = B_t stored
+ * transposed (N x K), 4 = the product is a result (large ones run on the
+ * tensor cores with exactly split operands) and not the input of an iteration
+ * (one FMA per product, terms in order, k ascending); beta 0 or 1.  GBD_ERR_ARG for sizes below 1, other flags or beta, or NULL. */
+int gbd_gemm_f64(gbd_ctx *ctx, int32_t M, int32_t N, int32_t K, int32_t nterms, int32_t flags, double alpha,
+                 int32_t beta, const double *A, const double *B, double *C);
 /* Failure detection without a fault: one bounded mbarrier wait (the helper
  * every role of the tensor-core kernel uses).  arrive = 0: nothing completes
  * the barrier, the wait runs out after its poll limit (2^22 polls, a few

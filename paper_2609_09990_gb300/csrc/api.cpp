@@ -483,6 +483,18 @@ int gbd_gemm_tc_selftest(gbd_ctx* ctx, int32_t M, int32_t N, int32_t K, int32_t 
   });
 }
 
+int gbd_gemm_f64(gbd_ctx* ctx, int32_t M, int32_t N, int32_t K, int32_t nterms, int32_t flags, double alpha,
+                 int32_t beta, const double* A, const double* B, double* C) {
+  return guarded(ctx, [&]() {
+    if (M < 1 || N < 1 || K < 1 || nterms < 1 || flags < 0 || flags > 7 || (beta != 0 && beta != 1) || !A || !B || !C ||
+        (int64_t)M * N > (1 << 26) || (int64_t)K * std::max(M, N) > (1 << 27) / nterms)
+      return fail(ctx, GBD_ERR_ARG, "invalid grouped-GEMM arguments");
+    if (!ctx->eng) ctx->eng.reset(new gbd::Engine(ctx->device));
+    ctx->eng->gemm_f64_host(M, N, K, nterms, flags, alpha, beta, A, B, C);
+    return GBD_OK;
+  });
+}
+
 int gbd_set_tier_stop(gbd_ctx* ctx, double floor_mult, int32_t hard_stag) {
   return guarded(ctx, [&]() {
     if (!(floor_mult > 0) || !std::isfinite(floor_mult) || hard_stag < 0)

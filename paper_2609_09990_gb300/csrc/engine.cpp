@@ -502,14 +502,29 @@ void Engine::upload(GemmPlan& p) {
   // one thread per element.  GB300's FP64 pipe is slow enough that the
   // unblocked loop keeps it busy, and both kernels run the same FMA
   // sequence per element.
+  // A plan of results: the tensor-core kernel with split operands, except
+  // for small outputs.  A K step of it takes about as long for 8 x 8 outputs
+  // as for 32 x 64, so it needs work to pay: at least 4096 products per step,
+  // or a large output in all (CAS(16,16) M=512: H_eff product 79 -> 21 ms,
+  // RDMs 240 -> 142 ms; CAS(9,9) 3-RDM 352 -> 93 ms).
   p.tiles.clear();
+  p.split.clear();
   p.flat.clear();
+  std::vector<int64_t> steps(p.outs.size(), 0);   // K steps of the split kernel per output
   for (int o = 0; o < (int)p.outs.size(); ++o) {
     const GemmOut& g = p.outs[o];
     const int64_t elems = (int64_t)g.M * g.N;
     const int64_t padded = (int64_t)((g.M + 31) / 32 * 32) * ((g.N + 31) / 32 * 32);
     int64_t ksum = 0;
-    for (int t = g.t0; t < g.t1; ++t) ksum += p.terms[t].K;
+    for (int t = g.t0; t < g.t1; ++t) {
+      ksum += p.terms[t].K;
+      steps[o] += (p.terms[t].K + kSplitChunk - 1) / kSplitChunk;
+    }
+    if (p.result && elems * ksum >= std::min<int64_t>(4096 * std::max<int64_t>(steps[o], 1), 1 << 20)) {
+      for (int tm = 0; tm * kSplitTileM < g.M; ++tm)
+        for (int tn = 0; tn * kSplitTileN < g.N; ++tn) p.split.push_back({o, tm, tn, 0});
+      continue;
+    }
     if (elems > 0 && 4 * elems < 3 * padded && ksum <= 1024) {
       for (int64_t e0 = 0; e0 < elems; e0 += 256) p.flat.push_back({o, -1, (int32_t)e0, 0});
       continue;
@@ -518,32 +533,35 @@ void Engine::upload(GemmPlan& p) {
       for (int tn = 0; tn * 32 < g.N; ++tn) p.tiles.push_back({o, tm, tn, 0});
   }
   // longest term lists first for load balance
-  std::stable_sort(p.tiles.begin(), p.tiles.end(), [&](const GemmTile& a, const GemmTile& b) {
+  auto longer = [&](const GemmTile& a, const GemmTile& b) {
     const GemmOut& x = p.outs[a.out];
     const GemmOut& y = p.outs[b.out];
     return (x.t1 - x.t0) > (y.t1 - y.t0);
-  });
-  std::stable_sort(p.flat.begin(), p.flat.end(), [&](const GemmTile& a, const GemmTile& b) {
-    const GemmOut& x = p.outs[a.out];
-    const GemmOut& y = p.outs[b.out];
-    return (x.t1 - x.t0) > (y.t1 - y.t0);
-  });
+  };
+  std::stable_sort(p.tiles.begin(), p.tiles.end(), longer);
+  std::stable_sort(p.flat.begin(), p.flat.end(), longer);
+  std::stable_sort(p.split.begin(), p.split.end(),
+                   [&](const GemmTile& a, const GemmTile& b) { return steps[a.out] > steps[b.out]; });
   p.d_tiles = dalloc<GemmTile>(std::max<size_t>(p.tiles.size(), 1));
+  p.d_split = dalloc<GemmTile>(std::max<size_t>(p.split.size(), 1));
   p.d_flat = dalloc<GemmTile>(std::max<size_t>(p.flat.size(), 1));
   h2d(p.d_flat, p.flat.data(), p.flat.size() * sizeof(GemmTile));
   h2d(p.d_terms, p.terms.data(), p.terms.size() * sizeof(GemmTerm));
   h2d(p.d_outs, p.outs.data(), p.outs.size() * sizeof(GemmOut));
   h2d(p.d_tiles, p.tiles.data(), p.tiles.size() * sizeof(GemmTile));
+  h2d(p.d_split, p.split.data(), p.split.size() * sizeof(GemmTile));
 }
 
 void Engine::release(GemmPlan& p) {
   dfree(p.d_terms);
   dfree(p.d_outs);
   dfree(p.d_tiles);
+  dfree(p.d_split);
   dfree(p.d_flat);
   p.d_terms = nullptr;
   p.d_outs = nullptr;
   p.d_tiles = nullptr;
+  p.d_split = nullptr;
   p.d_flat = nullptr;
 }
 
@@ -575,9 +593,10 @@ void Engine::release(AxpyPlan& p) {
 }
 
 void Engine::run(GemmPlan& p) {
-  if (p.tiles.empty() && p.flat.empty()) return;
-  launch_gemm_f64(p, stream);
-  stats.launches += (!p.tiles.empty()) + (!p.flat.empty());
+  if (p.tiles.empty() && p.split.empty() && p.flat.empty()) return;
+  const int l = launch_gemm_f64(p, stream);
+  if (l < 0) throw Error(-3, "grouped GEMM: shared memory refused");
+  stats.launches += l;
   CK(cudaGetLastError());
 }
 
@@ -1271,7 +1290,7 @@ struct Engine::Sigma {
   GraphSeq graph;
 };
 
-void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg) {
+void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool result) {
   // Y_b(Qin) exists when both operators have sub-blocks for (b, Qin)
   std::map<std::pair<int, int>, std::vector<const EnlSub*>> rby, lby;
   for (const auto& s : renl.subs) rby[{s.b, s.qin}].push_back(&s);
@@ -1294,6 +1313,7 @@ void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg) {
   GemmPlan& B = sg.B;
   A.clear();
   B.clear();
+  A.result = B.result = result;
   // stage A: Y_b(Qin)[:, cols (sout, q_r')] = sum psi(Qin)[:, cols (sin, q_r)] Rsub^T
   for (auto& y : ys) {
     int b = std::get<0>(y), qin = std::get<1>(y), qout = std::get<2>(y);
@@ -1898,7 +1918,7 @@ void Engine::probe_step(int k, int precision, int refine, double tol, double* th
   bool planned = false;
   *theta = solve_tiers(sg, diag, tol, precision, refine, planned);
   if (!planned) {
-    plan_sigma(sg.lenl, sg.renl, sg);
+    plan_sigma(sg.lenl, sg.renl, sg, true);   // one product, for the reported energy
     planned = true;
   }
   double* y = dalloc<double>(psi_size);
@@ -2263,7 +2283,7 @@ double Engine::final_energy() {
   finish_enl(sg.lenl, ax);
   build_renl(1, Renv[2], ER, sg.renl, ax);
   finish_enl(sg.renl, ax);
-  plan_sigma(sg.lenl, sg.renl, sg);
+  plan_sigma(sg.lenl, sg.renl, sg, true);
   double* y = dalloc<double>(psi_size);
   sigma(sg, psi, y);
   int nblk = reduction_blocks(psi_size);
@@ -2418,7 +2438,7 @@ void Engine::apply_heff(int k, const double* in, double* out, double* diag_out, 
   finish_enl(sg.renl, ax);
   double* y = dalloc<double>(psi_size);
   if (prec == 0) {
-    plan_sigma(sg.lenl, sg.renl, sg);
+    plan_sigma(sg.lenl, sg.renl, sg, true);
     sigma(sg, psi, y);
   } else {
     TcPlan* P = tc_plan(sg.lenl, sg.renl, prec == 1 ? kTF32 : prec == 2 ? kBF16 : prec == 3 ? kTF32x3 : kBF16x3);

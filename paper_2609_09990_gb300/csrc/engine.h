@@ -402,7 +402,8 @@ class Engine {
   void setup_two_site(int k);
   void form_psi(int k, int pattern);
   struct Sigma;
-  void plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg);
+  // result: this H_eff product is itself returned, not iterated (GemmPlan::result)
+  void plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool result = false);
   void sigma(Sigma& sg, const double* x, double* y);
   void compute_diag(const EnlOp& lenl, const EnlOp& renl, double* diag);
   // stag_rel > 0: stop on stagnation (reduced-precision operators); see the definition
@@ -459,6 +460,8 @@ class Engine {
   void probe_step(int k, int precision, int refine, double tol, double* theta, double* e64, double* r64);
   void gemm_tc_selftest(int M, int N, int K, int nterms, int flags, int prec, uint64_t seed, double* max_err,
                         double* max_ref);
+  void gemm_f64_host(int M, int N, int K, int nterms, int flags, double alpha, int beta, const double* A,
+                     const double* B, double* C);
   // the inner-PCG correction of the Davidson solver at centre k with the
   // FP64 sigma and the step's own H_eff diagonal, from host x, r and theta
   void pcg_selftest(int k, const double* x_host, const double* r_host, double theta, double* t_host,

@@ -107,13 +107,21 @@ struct GemmPlan {       // host side lists plus their device copies
   std::vector<GemmTerm> terms;
   std::vector<GemmOut> outs;
   std::vector<GemmTile> tiles;   // 32 x 32 register-blocked tiles
+  std::vector<GemmTile> split;   // 32 x 64 tiles of the tensor-core kernel with split operands
   std::vector<GemmTile> flat;    // {out, -1, first element, 0}: 256 elements, one per thread
   GemmTerm* d_terms = nullptr;
   GemmOut* d_outs = nullptr;
   GemmTile* d_tiles = nullptr;
+  GemmTile* d_split = nullptr;
   GemmTile* d_flat = nullptr;
   double flops = 0.0;       // 2 m n k summed over terms
-  void clear() { terms.clear(); outs.clear(); tiles.clear(); flat.clear(); flops = 0.0; }
+  // The products are results, or are summed into one: large outputs may take
+  // the split kernel, whose sums are rounded elsewhere (and less) than the
+  // FMA loop's.  What feeds a Davidson iteration or the next step leaves it
+  // false: an unconverged iteration amplifies a change of rounding until
+  // its iterates have no digit in common.
+  bool result = false;
+  void clear() { terms.clear(); outs.clear(); tiles.clear(); split.clear(); flat.clear(); flops = 0.0; }
   int add_out(double* C, int ldc, int M, int N, int beta) {
     GemmOut o{C, ldc, M, N, (int)terms.size(), (int)terms.size(), beta, 0};
     outs.push_back(o);
@@ -144,8 +152,13 @@ struct AxpyPlan {
 };
 constexpr int kAxpyChunk = 1024;   // output elements per work chunk of the block axpy
 
+// tile of the split kernel: outputs, and K columns per step
+constexpr int kSplitTileM = 32, kSplitTileN = 64, kSplitChunk = 32;
+
 // ---------------------------------------------------------------- kernels (kernels.cu)
-void launch_gemm_f64(const GemmPlan& p, cudaStream_t s);
+// launches made, or -1 when the split kernel's shared memory was refused
+int launch_gemm_f64(const GemmPlan& p, cudaStream_t s);
+int launch_gemm_f64_split(const GemmPlan& p, cudaStream_t s);
 void launch_axpy(const AxpyPlan& p, cudaStream_t s);
 void launch_set_identity(double* d, int m, cudaStream_t s);
 // dst = sign * src^T for blocks src (rows x cols, row-major, dense); one

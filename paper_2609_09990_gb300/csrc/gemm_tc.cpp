@@ -266,4 +266,28 @@ void Engine::gemm_tc_selftest(int M, int N, int K, int nterms, int flags, int pr
   sync();
 }
 
+// C = beta C + alpha sum_t op(A_t) op(B_t) on host arrays, as one output of a
+// grouped FP64 plan (blocks dense and back to back; flags 4: a plan of results)
+void Engine::gemm_f64_host(int M, int N, int K, int nterms, int flags, double alpha, int beta, const double* A,
+                           const double* B, double* C) {
+  const size_t asz = (size_t)M * K, bsz = (size_t)K * N, csz = (size_t)M * N;
+  double* dA = dalloc<double>(asz * nterms);
+  double* dB = dalloc<double>(bsz * nterms);
+  double* dC = dalloc<double>(csz);
+  h2d(dA, A, asz * nterms * sizeof(double));
+  h2d(dB, B, bsz * nterms * sizeof(double));
+  h2d(dC, C, csz * sizeof(double));
+  GemmPlan p;
+  p.result = flags & 4;
+  p.add_out(dC, N, M, N, beta);
+  for (int t = 0; t < nterms; ++t)
+    p.add_term(dA + asz * t, flags & 1 ? M : K, dB + bsz * t, flags & 2 ? K : N, K, flags & 3, alpha);
+  upload(p);
+  run(p);
+  release(p);
+  CK(cudaMemcpyAsync(C, dC, csz * sizeof(double), cudaMemcpyDeviceToHost, stream));
+  sync();
+  for (double* q : {dA, dB, dC}) dfree(q);
+}
+
 }  // namespace gbd

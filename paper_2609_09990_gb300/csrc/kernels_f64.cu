@@ -4,7 +4,8 @@
 // and MPO entries) and the Davidson vector operations.
 //
 // GB300 executes FP64 on its CUDA cores only; these kernels are the plain
-// FP64 path.  The grouped GEMM keeps a 32x32 output tile per CTA in
+// FP64 path (products that are results themselves run on the tensor cores,
+// kernels_f64_split.cu).  The grouped GEMM keeps a 32x32 output tile per CTA in
 // registers and walks every (A,B) term that contributes to that tile, so each
 // output block is written once, deterministically, without atomics.
 #include <cuda_runtime.h>
@@ -322,11 +323,14 @@ int reduction_blocks(int64_t n) {
   return (int)(b < 1 ? 1 : b);
 }
 
-void launch_gemm_f64(const GemmPlan& p, cudaStream_t s) {
+int launch_gemm_f64(const GemmPlan& p, cudaStream_t s) {
+  const int ns = launch_gemm_f64_split(p, s);
+  if (ns < 0) return ns;
   const int nt = (int)p.tiles.size();
   if (nt > 0) gemm_f64_kernel<<<nt < 152 * 24 ? nt : 152 * 24, GEMM_THREADS, 0, s>>>(p.d_terms, p.d_outs, p.d_tiles, nt);
   const int nf = (int)p.flat.size();
   if (nf > 0) gemm_f64_flat_kernel<<<nf < 152 * 8 ? nf : 152 * 8, 256, 0, s>>>(p.d_terms, p.d_outs, p.d_flat, nf);
+  return ns + (nt > 0) + (nf > 0);
 }
 
 void launch_axpy(const AxpyPlan& p, cudaStream_t s) {

@@ -142,6 +142,7 @@ double* Engine::expand_ci(int64_t& Na_str, int64_t& Nb_str) {
     const Bond& br = bonds[i + 1];
     std::vector<Fix> nx(br.nsec());
     GemmPlan p;
+    p.result = true;
     for (int j = 0; j < br.nsec(); ++j) {
       Fix& f = nx[j];
       std::vector<std::pair<int, int>> parts;   // (parent sector, s)
@@ -189,6 +190,7 @@ double* Engine::expand_ci(int64_t& Na_str, int64_t& Nb_str) {
     const Bond& br = bonds[i + 1];
     std::vector<Fix> nx(bl.nsec());
     GemmPlan p;
+    p.result = true;
     for (int j = 0; j < bl.nsec(); ++j) {
       Fix& f = nx[j];
       std::vector<std::pair<int, int>> parts;   // (child sector, s)
@@ -231,6 +233,7 @@ double* Engine::expand_ci(int64_t& Na_str, int64_t& Nb_str) {
     int np = (int)pre[j].a.size(), ns = (int)suf[j].a.size(), m = bh.dim[j];
     double* A = dalloc<double>((size_t)np * ns);
     GemmPlan p;
+    p.result = true;
     p.add_out(A, ns, np, ns, 0);
     p.add_term(pre[j].d, m, suf[j].d, ns, m, 0, 1.0);
     upload(p);
@@ -310,6 +313,7 @@ void Engine::rdms_ci(double* rdm1, double* rdm2) {
     int parts = (int)std::min<int64_t>(SPLIT, std::max<int64_t>(1, K / 4096));
     int64_t step = (K + parts - 1) / parts;
     GemmPlan p;
+    p.result = true;
     const double* Cchunk = C + (int64_t)ja0 * Nb_str;
     for (int s = 0; s < SPLIT; ++s) {
       int64_t k0 = (int64_t)s * step, k1 = std::min<int64_t>(K, k0 + step);
@@ -403,6 +407,7 @@ void Engine::rdm3(double* out) {
   // in a fixed order into dst
   auto gram = [&](const double* W, int ldw_is_vec, double* dst, int ncols) {
     GemmPlan p;
+    p.result = true;
     for (int s = 0; s < parts; ++s) {
       const int64_t k0 = (int64_t)s * step, k1 = std::min<int64_t>(ndet, k0 + step);
       p.add_out(Mp + (size_t)s * n2 * ncols, ncols, n2, ncols, 0);

@@ -420,6 +420,7 @@ std::vector<double> Engine::eval_strings(StringSet& S) {
     live += tsz * (int64_t)sizeof(double);
     peak = std::max(peak, live);
     GemmPlan g1, g2;
+    g1.result = g2.result = true;
     for (size_t p = 0; p < Sp.ch.size(); ++p)
       for (int s = 0; s < 4; ++s)
         for (int q = 0; q < ns; ++q) {
@@ -497,6 +498,7 @@ std::vector<double> Engine::eval_strings(StringSet& S) {
     live += tsz * (int64_t)sizeof(double);
     peak = std::max(peak, live);
     GemmPlan g1, g2;
+    g1.result = g2.result = true;
     for (size_t p = 0; p < Sp.ch.size(); ++p)
       for (int s = 0; s < 4; ++s)
         for (int r = 0; r < ns; ++r) {
@@ -547,6 +549,7 @@ std::vector<double> Engine::eval_strings(StringSet& S) {
     const Bond& bd = bonds[b];
     const BondProd& P = prod[b];
     GemmPlan g;
+    g.result = true;
     for (size_t c = 0; c < P.shift.size(); ++c) {
       const int nl = (int)P.lrows[c].size(), nr = (int)P.rrows[c].size();
       std::vector<int> qs;

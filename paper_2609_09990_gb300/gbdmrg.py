@@ -104,6 +104,8 @@ def lib():
         "gbd_set_env_precision": (C.c_int, [vp, C.c_int32]),
         "gbd_gemm_tc_selftest": (C.c_int, [vp, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32,
                                            C.c_uint64, _dp, _dp]),
+        "gbd_gemm_f64": (C.c_int, [vp, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_double, C.c_int32,
+                                   _dp, _dp, _dp]),
         "gbd_set_preconditioner": (C.c_int, [vp, C.c_int32]),
         "gbd_set_tc_tile": (C.c_int, [vp, C.c_int32]),
         "gbd_set_tc_order": (C.c_int, [vp, C.c_int32]),
@@ -387,6 +389,18 @@ class Context:
         self._check(self.L.gbd_gemm_tc_selftest(self.ptr, M, N, K, nterms, flags, prec, seed, C.byref(e),
                                                 C.byref(r)), "gbd_gemm_tc_selftest")
         return e.value, r.value
+
+    def gemm_f64(self, A, B, flags=0, alpha=1.0, C0=None):
+        """C0 + alpha sum_t op(A[t]) op(B[t]) by the FP64 grouped GEMM (flags 1: A[t] is K x M, 2: B[t] is N x K,
+        4: the product is a result)."""
+        A = np.ascontiguousarray(A, dtype=np.float64)
+        B = np.ascontiguousarray(B, dtype=np.float64)
+        K, M = A.shape[1:] if flags & 1 else A.shape[:0:-1]
+        N = B.shape[1] if flags & 2 else B.shape[2]
+        out = np.zeros((M, N)) if C0 is None else np.array(C0, dtype=np.float64)
+        self._check(self.L.gbd_gemm_f64(self.ptr, M, N, K, A.shape[0], flags, alpha, 0 if C0 is None else 1, _d(A),
+                                        _d(B), _d(out)), "gbd_gemm_f64")
+        return out
 
     def set_tier_stop(self, floor_mult, hard_stag=0):
         self._check(self.L.gbd_set_tier_stop(self.ptr, float(floor_mult), int(hard_stag)), "gbd_set_tier_stop")
