@@ -491,17 +491,32 @@ void Engine::h2d(void* dst, const void* src, size_t bytes) {
   pin_pos = start + n;
 }
 
+namespace {
+// rows and columns of the tiles of an M x N block: at most cap outputs and
+// kFmaSide on a side, the fewest warps in all, then the fewest operands
+std::pair<int, int> cut_block(int M, int N, int cap) {
+  std::pair<int, int> best{1, 1};
+  double least = 1e300;
+  for (int gn = (N + kFmaSide - 1) / kFmaSide, tried = 0; gn <= N && tried < 6; ++gn, ++tried) {
+    const int tn = (N + gn - 1) / gn;
+    const int rows = std::min({M, kFmaSide, std::max(1, cap / tn)});
+    if (tn > cap) continue;
+    const int gm = (M + rows - 1) / rows, tm = (M + gm - 1) / gm;
+    const double warps = (double)gm * ((N + tn - 1) / tn) * ((tm * tn + 31) / 32);
+    const double cost = warps * (1.0 + 0.02 * (tm + tn));
+    if (cost < least) {
+      least = cost;
+      best = {tm, tn};
+    }
+  }
+  return best;
+}
+}  // namespace
+
 void Engine::upload(GemmPlan& p) {
   check(p);
   p.d_terms = dalloc<GemmTerm>(p.terms.size());
   p.d_outs = dalloc<GemmOut>(p.outs.size());
-  // tiles: 32 x 32 outputs, or, where 32 x 32 tiles would leave more than
-  // a quarter of their elements idle (sector blocks of a few tens) and the
-  // summed K is short (environment updates, not the sigma's long term
-  // lists, where register blocking pays), flat items of 256 elements with
-  // one thread per element.  GB300's FP64 pipe is slow enough that the
-  // unblocked loop keeps it busy, and both kernels run the same FMA
-  // sequence per element.
   // A plan of results: the tensor-core kernel with split operands, except
   // for small outputs.  A K step of it takes about as long for 8 x 8 outputs
   // as for 32 x 64, so it needs work to pay: at least 4096 products per step,
@@ -509,12 +524,13 @@ void Engine::upload(GemmPlan& p) {
   // RDMs 240 -> 142 ms; CAS(9,9) 3-RDM 352 -> 93 ms).
   p.tiles.clear();
   p.split.clear();
-  p.flat.clear();
+  std::vector<std::pair<int64_t, int>> fma;   // chain length and output
+  int64_t fma_elems = 0;
   std::vector<int64_t> steps(p.outs.size(), 0);   // K steps of the split kernel per output
   for (int o = 0; o < (int)p.outs.size(); ++o) {
     const GemmOut& g = p.outs[o];
     const int64_t elems = (int64_t)g.M * g.N;
-    const int64_t padded = (int64_t)((g.M + 31) / 32 * 32) * ((g.N + 31) / 32 * 32);
+    if (elems == 0) continue;
     int64_t ksum = 0;
     for (int t = g.t0; t < g.t1; ++t) {
       ksum += p.terms[t].K;
@@ -525,27 +541,34 @@ void Engine::upload(GemmPlan& p) {
         for (int tn = 0; tn * kSplitTileN < g.N; ++tn) p.split.push_back({o, tm, tn, 0});
       continue;
     }
-    if (elems > 0 && 4 * elems < 3 * padded && ksum <= 1024) {
-      for (int64_t e0 = 0; e0 < elems; e0 += 256) p.flat.push_back({o, -1, (int32_t)e0, 0});
-      continue;
-    }
-    for (int tm = 0; tm * 32 < g.M; ++tm)
-      for (int tn = 0; tn * 32 < g.N; ++tn) p.tiles.push_back({o, tm, tn, 0});
+    fma.push_back({ksum, o});
+    fma_elems += elems;
   }
-  // longest term lists first for load balance
-  auto longer = [&](const GemmTile& a, const GemmTile& b) {
-    const GemmOut& x = p.outs[a.out];
-    const GemmOut& y = p.outs[b.out];
-    return (x.t1 - x.t0) > (y.t1 - y.t0);
-  };
-  std::stable_sort(p.tiles.begin(), p.tiles.end(), longer);
-  std::stable_sort(p.flat.begin(), p.flat.end(), longer);
+  // The others: FMA tiles, the largest that still give every SM about eight
+  // (fewer outputs a tile read more operands per product, fewer tiles leave
+  // SMs with longer chains than others: CAS(12,12) M=256 FP64 Davidson solve
+  // 394 ms with this rule, 406 ms with tiles of 128, 457 ms with four 256-output
+  // tiles an SM allowed, 493 ms with tiles of 64).
+  int cap = 256;
+  while (cap > 32 && fma_elems < (int64_t)8 * num_sms * cap) cap /= 2;
+  p.per_lane = cap > 128 ? 2 : 1;
+  p.tile_span = 0;
+  // longest chains first
+  std::stable_sort(fma.begin(), fma.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  std::unordered_map<uint64_t, std::pair<int, int>> cuts;   // block sizes repeat
+  for (const auto& f : fma) {
+    const GemmOut& g = p.outs[f.second];
+    auto& c = cuts[(uint64_t)g.M << 32 | (uint32_t)g.N];
+    if (c.first == 0) c = cut_block(g.M, g.N, cap);
+    p.tile_span = std::max(p.tile_span, (c.first | 1) + (c.second | 1));
+    for (int m = 0; m < g.M; m += c.first)
+      for (int n = 0; n < g.N; n += c.second)
+        p.tiles.push_back({f.second, m, n, std::min(c.first, g.M - m) << 16 | std::min(c.second, g.N - n)});
+  }
   std::stable_sort(p.split.begin(), p.split.end(),
                    [&](const GemmTile& a, const GemmTile& b) { return steps[a.out] > steps[b.out]; });
   p.d_tiles = dalloc<GemmTile>(std::max<size_t>(p.tiles.size(), 1));
   p.d_split = dalloc<GemmTile>(std::max<size_t>(p.split.size(), 1));
-  p.d_flat = dalloc<GemmTile>(std::max<size_t>(p.flat.size(), 1));
-  h2d(p.d_flat, p.flat.data(), p.flat.size() * sizeof(GemmTile));
   h2d(p.d_terms, p.terms.data(), p.terms.size() * sizeof(GemmTerm));
   h2d(p.d_outs, p.outs.data(), p.outs.size() * sizeof(GemmOut));
   h2d(p.d_tiles, p.tiles.data(), p.tiles.size() * sizeof(GemmTile));
@@ -557,12 +580,10 @@ void Engine::release(GemmPlan& p) {
   dfree(p.d_outs);
   dfree(p.d_tiles);
   dfree(p.d_split);
-  dfree(p.d_flat);
   p.d_terms = nullptr;
   p.d_outs = nullptr;
   p.d_tiles = nullptr;
   p.d_split = nullptr;
-  p.d_flat = nullptr;
 }
 
 void Engine::upload(AxpyPlan& p) {
@@ -593,7 +614,7 @@ void Engine::release(AxpyPlan& p) {
 }
 
 void Engine::run(GemmPlan& p) {
-  if (p.tiles.empty() && p.split.empty() && p.flat.empty()) return;
+  if (p.tiles.empty() && p.split.empty()) return;
   const int l = launch_gemm_f64(p, stream);
   if (l < 0) throw Error(-3, "grouped GEMM: shared memory refused");
   stats.launches += l;

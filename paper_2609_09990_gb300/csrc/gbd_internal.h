@@ -106,14 +106,14 @@ struct GemmTile {
 struct GemmPlan {       // host side lists plus their device copies
   std::vector<GemmTerm> terms;
   std::vector<GemmOut> outs;
-  std::vector<GemmTile> tiles;   // 32 x 32 register-blocked tiles
+  std::vector<GemmTile> tiles;   // FMA kernel: {out, first row, first column, rows << 16 | columns}
   std::vector<GemmTile> split;   // 32 x 64 tiles of the tensor-core kernel with split operands
-  std::vector<GemmTile> flat;    // {out, -1, first element, 0}: 256 elements, one per thread
   GemmTerm* d_terms = nullptr;
   GemmOut* d_outs = nullptr;
   GemmTile* d_tiles = nullptr;
   GemmTile* d_split = nullptr;
-  GemmTile* d_flat = nullptr;
+  int tile_span = 0;             // largest rows + columns of a tile (odd pitches)
+  int per_lane = 2;              // outputs per lane: tiles of at most 128 per_lane outputs
   double flops = 0.0;       // 2 m n k summed over terms
   // The products are results, or are summed into one: large outputs may take
   // the split kernel, whose sums are rounded elsewhere (and less) than the
@@ -121,7 +121,7 @@ struct GemmPlan {       // host side lists plus their device copies
   // false: an unconverged iteration amplifies a change of rounding until
   // its iterates have no digit in common.
   bool result = false;
-  void clear() { terms.clear(); outs.clear(); tiles.clear(); split.clear(); flat.clear(); flops = 0.0; }
+  void clear() { terms.clear(); outs.clear(); tiles.clear(); split.clear(); flops = 0.0; }
   int add_out(double* C, int ldc, int M, int N, int beta) {
     GemmOut o{C, ldc, M, N, (int)terms.size(), (int)terms.size(), beta, 0};
     outs.push_back(o);
@@ -153,6 +153,8 @@ struct AxpyPlan {
 constexpr int kAxpyChunk = 1024;   // output elements per work chunk of the block axpy
 
 // tile of the split kernel: outputs, and K columns per step
+// largest side of an FMA tile (shared memory: 3 steps of 32 columns of both sides, at most 51 KB)
+constexpr int kFmaSide = 32;
 constexpr int kSplitTileM = 32, kSplitTileN = 64, kSplitChunk = 32;
 
 // ---------------------------------------------------------------- kernels (kernels.cu)

@@ -5,9 +5,10 @@
 //
 // GB300 executes FP64 on its CUDA cores only; these kernels are the plain
 // FP64 path (products that are results themselves run on the tensor cores,
-// kernels_f64_split.cu).  The grouped GEMM keeps a 32x32 output tile per CTA in
-// registers and walks every (A,B) term that contributes to that tile, so each
-// output block is written once, deterministically, without atomics.
+// kernels_f64_split.cu).  Every output element is written once,
+// deterministically, without atomics.
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "gbd_internal.h"
@@ -16,106 +17,183 @@ namespace gbd {
 
 namespace {
 
-constexpr int TM = 32, TN = 32, TK = 16, GEMM_THREADS = 64;
+// Grouped GEMM by FP64 FMAs.  An output element is one chain of FMAs over its
+// terms in order and k ascending, A scaled by its coefficient first, whatever
+// the tile: the result does not depend on how the plan is cut.
+//
+// Bound: the FP64 pipe, 2 FMAs per SM and clock -- so slow that a warp needs
+// no register blocking to fill it (an FMA of a warp occupies its sub-core for
+// 64 clocks, as long as its result takes; its two operand reads from shared
+// memory take 4 of the SM's), but every idle lane and every other FP64
+// instruction counts.  So a tile is a rectangle of at most 128 E outputs cut
+// to the sector block, one or two outputs a lane and nothing padded but the
+// last warp; coefficients of +-1 cost no FP64 operation, others one per
+// operand element.  A fifth warp prepares the operands: the columns of all
+// terms of the output, concatenated, are taken 32 at a time (one lane each,
+// whatever term it falls in, so that short terms fill a step too) and copied
+// asynchronously into a ring of three steps: one being multiplied, one
+// landing, one on its way.
+// CAS(12,12) M=256 H_eff product (3.41 GFLOP): 13.1 -> 3.5 ms (0.98 TFLOP/s of
+// the pipe's 1.19; 92 % of its cycles busy), against a kernel of 32 x 32
+// register tiles for the long chains and one with a lane per output that read
+// from global memory and multiplied by the coefficient at every FMA.
+constexpr int FT = 128, FK = 32, FR = 3;
 
-__global__ void __launch_bounds__(GEMM_THREADS)
+template <int E>
+__global__ void __launch_bounds__(FT + 32, 8)
 gemm_f64_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
-                const GemmTile* __restrict__ tiles, int ntiles) {
-  __shared__ double As[TK][TM + 1];
-  __shared__ double Bs[TK][TN + 1];
-  const int tid = threadIdx.x;
-  const int tx = tid & 7, ty = tid >> 3;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const GemmTile tl = tiles[tile];
-    const GemmOut o = outs[tl.out];
-    const int m0 = tl.tm * TM, n0 = tl.tn * TN;
-    double acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    for (int t = o.t0; t < o.t1; ++t) {
-      const GemmTerm T = terms[t];
-      const bool ta = T.flags & 1, tb = T.flags & 2;
-      for (int k0 = 0; k0 < T.K; k0 += TK) {
-        // A tile: TM x TK of op(A), scaled by alpha
-#pragma unroll
-        for (int r = 0; r < (TM * TK) / GEMM_THREADS; ++r) {
-          int idx = tid + r * GEMM_THREADS;
-          int i, kk;
-          if (!ta) { i = idx / TK; kk = idx % TK; } else { i = idx % TM; kk = idx / TM; }
-          int gm = m0 + i, gk = k0 + kk;
-          double v = 0.0;
-          if (gm < o.M && gk < T.K)
-            v = ta ? T.A[(int64_t)gk * T.lda + gm] : T.A[(int64_t)gm * T.lda + gk];
-          As[kk][i] = v * T.alpha;
+                const GemmTile* __restrict__ tiles) {
+  extern __shared__ double ring[];
+  __shared__ double coef[FR][FK];
+  __shared__ int how[FR][FK];   // coefficient of a column: 0 one, 1 minus one, 2 another
+  __shared__ int ncol[FR], scaled[FR];
+  const GemmTile tl = tiles[blockIdx.x];
+  const GemmOut o = outs[tl.out];
+  const int m0 = tl.tm, n0 = tl.tn, tm = tl.pad >> 16, tn = tl.pad & 0xFFFF;
+  const int pa = tm | 1, pb = tn | 1, step = FK * (pa + pb);   // odd pitches: the copies' lanes are K columns
+  if (threadIdx.x >= FT) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(ring));
+    int t = o.t0, k = 0, n = 0;   // next column: k of term t; columns of the prepared step
+    const double *a = nullptr, *b = nullptr;
+    int64_t sa = 0, sb = 0;
+    double al = 1.0;
+    // operand addresses of the next 32 columns, one per lane
+    auto prepare = [&]() {
+      n = 0;
+      while (t < o.t1) {
+        int kt = t + lane < o.t1 ? max(terms[t + lane].K, 0) : 0;
+        if (lane == 0) kt -= k;
+        int sum = kt;   // inclusive sums over the next 32 terms
+        for (int d = 1; d < 32; d <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, sum, d);
+          if (lane >= d) sum += v;
         }
-        // B tile: TK x TN of op(B)
-#pragma unroll
-        for (int r = 0; r < (TN * TK) / GEMM_THREADS; ++r) {
-          int idx = tid + r * GEMM_THREADS;
-          int j, kk;
-          if (!tb) { j = idx % TN; kk = idx / TN; } else { j = idx / TK; kk = idx % TK; }
-          int gn = n0 + j, gk = k0 + kk;
-          double v = 0.0;
-          if (gn < o.N && gk < T.K)
-            v = tb ? T.B[(int64_t)gn * T.ldb + gk] : T.B[(int64_t)gk * T.ldb + gn];
-          Bs[kk][j] = v;
+        const int total = __shfl_sync(0xffffffffu, sum, 31);
+        if (total == 0) {
+          t += 32;
+          k = 0;
+          continue;
         }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < TK; ++kk) {
-          double a[4], b[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 8 * i];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 8 * j];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        n = min(FK, total);
+        int lo = 0;   // the first term whose sum exceeds this lane's column
+        for (int d = 16; d > 0; d >>= 1)
+          if (__shfl_sync(0xffffffffu, sum, lo + d - 1) <= lane) lo += d;
+        const int before = __shfl_sync(0xffffffffu, sum - kt, lo);
+        if (lane < n) {
+          const GemmTerm T = terms[t + lo];
+          const int64_t kk = lane - before + (lo == 0 ? k : 0);
+          if (T.flags & 1) {
+            a = T.A + kk * T.lda + m0;
+            sa = 1;
+          } else {
+            a = T.A + (int64_t)m0 * T.lda + kk;
+            sa = T.lda;
+          }
+          if (T.flags & 2) {
+            b = T.B + (int64_t)n0 * T.ldb + kk;
+            sb = T.ldb;
+          } else {
+            b = T.B + kk * T.ldb + n0;
+            sb = 1;
+          }
+          al = T.alpha;
         }
-        __syncthreads();
+        const int adv = __popc(__ballot_sync(0xffffffffu, sum <= n));   // terms used up
+        const int used = __shfl_sync(0xffffffffu, sum, max(adv - 1, 0));
+        k = adv == 0 ? k + n : n - used;
+        t += adv;
+        break;
       }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int gm = m0 + ty + 8 * i;
-      if (gm >= o.M) continue;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        int gn = n0 + tx + 8 * j;
-        if (gn >= o.N) continue;
-        double* c = o.C + (int64_t)gm * o.ldc + gn;
-        *c = o.beta ? (*c + acc[i][j]) : acc[i][j];
+    };
+    auto issue = [&](int s) {
+      if (lane < n) {
+        uint32_t da = base + (s * step + lane * pa) * 8, db = base + (s * step + FK * pa + lane * pb) * 8;
+        const double *pa_ = a, *pb_ = b;
+        for (int i = 0; i < tm; ++i, da += 8, pa_ += sa)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(da), "l"(pa_) : "memory");
+        for (int j = 0; j < tn; ++j, db += 8, pb_ += sb)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(db), "l"(pb_) : "memory");
+        coef[s][lane] = al;
+        how[s][lane] = al == 1.0 ? 0 : al == -1.0 ? 1 : 2;
       }
+      const unsigned any = __ballot_sync(0xffffffffu, lane < n && al != 1.0);
+      if (lane == 0) {
+        ncol[s] = n;
+        scaled[s] = any != 0;
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    prepare();
+    issue(0);
+    prepare();
+    issue(1);
+    prepare();
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    for (int s = 0; ncol[s] > 0;) {
+      issue(s == 0 ? 2 : s - 1);
+      prepare();
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncthreads();
+      s = s == 2 ? 0 : s + 1;
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    return;
   }
-}
-
-// one output element per thread, 256 consecutive elements (row-major) of
-// one output per item; per element the same FMA sequence as gemm_f64_kernel
-// (terms in order, k ascending, A scaled by alpha first)
-__global__ void __launch_bounds__(256)
-gemm_f64_flat_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
-                     const GemmTile* __restrict__ items, int nitems) {
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-    const GemmTile w = items[it];
-    const GemmOut o = outs[w.out];
-    const int64_t e = (int64_t)w.tn + threadIdx.x;
-    if (e >= (int64_t)o.M * o.N) continue;
-    const int i = (int)(e / o.N), j = (int)(e - (int64_t)i * o.N);
-    double acc = 0.0;
-    for (int t = o.t0; t < o.t1; ++t) {
-      const GemmTerm T = terms[t];
-      const bool ta = T.flags & 1, tb = T.flags & 2;
-      const double* a = ta ? T.A + i : T.A + (int64_t)i * T.lda;
-      const double* b = tb ? T.B + (int64_t)j * T.ldb : T.B + j;
-      const int64_t sa = ta ? T.lda : 1, sb = tb ? 1 : T.ldb;
-      for (int k = 0; k < T.K; ++k) acc = fma(a[k * sa] * T.alpha, b[k * sb], acc);
+  const int ne = tm * tn;
+  int ia[E], jb[E];
+  double acc[E];
+#pragma unroll
+  for (int u = 0; u < E; ++u) {
+    const int e = min((int)threadIdx.x + u * FT, ne - 1);   // idle lanes repeat the last output
+    ia[u] = e / tn;
+    jb[u] = e - ia[u] * tn;
+    acc[u] = 0.0;
+  }
+  // outputs per lane of this warp
+  const int w0 = (int)threadIdx.x & ~31, on = (w0 < ne) + (E == 2 && w0 + FT < ne);
+  __syncthreads();
+  for (int s = 0;;) {
+    const int n = ncol[s];
+    if (n == 0) break;
+    double* A = ring + s * step;
+    const double* B = A + FK * pa;
+    if (scaled[s]) {
+      // columns with a coefficient other than 1: signs by their bit (no FP64
+      // operation), others multiplied; one column per lane
+      const int kk = threadIdx.x & (FK - 1), h = kk < n ? how[s][kk] : 0;
+      for (int i = threadIdx.x >> 5; i < tm; i += FT / 32) {
+        double& v = A[kk * pa + i];
+        if (h == 1) v = __longlong_as_double(__double_as_longlong(v) ^ (1ll << 63));
+        if (__any_sync(0xffffffffu, h == 2))
+          if (h == 2) v *= coef[s][kk];
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(FT) : "memory");
     }
-    double* c = o.C + (int64_t)i * o.ldc + j;
-    *c = o.beta ? (*c + acc) : acc;
+    auto products = [&](auto outputs) {
+      constexpr int O = decltype(outputs)::value;
+      if (n == FK) {
+#pragma unroll 8
+        for (int k = 0; k < FK; ++k)
+#pragma unroll
+          for (int u = 0; u < O; ++u) acc[u] = fma(A[k * pa + ia[u]], B[k * pb + jb[u]], acc[u]);
+      } else {
+        for (int k = 0; k < n; ++k)
+#pragma unroll
+          for (int u = 0; u < O; ++u) acc[u] = fma(A[k * pa + ia[u]], B[k * pb + jb[u]], acc[u]);
+      }
+    };
+    if (E == 2 && on == 2) products(std::integral_constant<int, E>());
+    else if (on > 0) products(std::integral_constant<int, 1>());
+    __syncthreads();
+    s = s == 2 ? 0 : s + 1;
+  }
+#pragma unroll
+  for (int u = 0; u < E; ++u) {
+    if ((int)threadIdx.x + u * FT >= ne) continue;
+    double* c = o.C + (int64_t)(m0 + ia[u]) * o.ldc + n0 + jb[u];
+    *c = o.beta ? (*c + acc[u]) : acc[u];
   }
 }
 
@@ -327,10 +405,10 @@ int launch_gemm_f64(const GemmPlan& p, cudaStream_t s) {
   const int ns = launch_gemm_f64_split(p, s);
   if (ns < 0) return ns;
   const int nt = (int)p.tiles.size();
-  if (nt > 0) gemm_f64_kernel<<<nt < 152 * 24 ? nt : 152 * 24, GEMM_THREADS, 0, s>>>(p.d_terms, p.d_outs, p.d_tiles, nt);
-  const int nf = (int)p.flat.size();
-  if (nf > 0) gemm_f64_flat_kernel<<<nf < 152 * 8 ? nf : 152 * 8, 256, 0, s>>>(p.d_terms, p.d_outs, p.d_flat, nf);
-  return ns + (nt > 0) + (nf > 0);
+  const int smem = FR * FK * p.tile_span * (int)sizeof(double);
+  if (nt > 0 && p.per_lane == 2) gemm_f64_kernel<2><<<nt, FT + 32, smem, s>>>(p.d_terms, p.d_outs, p.d_tiles);
+  if (nt > 0 && p.per_lane == 1) gemm_f64_kernel<1><<<nt, FT + 32, smem, s>>>(p.d_terms, p.d_outs, p.d_tiles);
+  return ns + (nt > 0);
 }
 
 void launch_axpy(const AxpyPlan& p, cudaStream_t s) {
