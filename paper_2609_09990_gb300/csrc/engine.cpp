@@ -391,25 +391,56 @@ bool Engine::in_allocation(const void* p, int64_t rows, int64_t cols, int64_t ld
   return true;
 }
 
-void Engine::check(const GemmPlan& p) const {
-  for (const auto& o : p.outs) {
-    check_range(o.C, o.M, o.N, o.ldc, "C");
+bool Engine::outputs_ok(const GemmPlan& p, int o0, int o1) const {
+  AllocCache ca, cb, cc;   // A, B and C mostly stay in one allocation each
+  for (int i = o0; i < o1; ++i) {
+    const GemmOut& o = p.outs[i];
+    if (!in_allocation(o.C, o.M, o.N, o.ldc, cc)) return false;
     for (int t = o.t0; t < o.t1; ++t) {
       const GemmTerm& g = p.terms[t];
       if (g.K <= 0) continue;
-      if (g.flags & 1) check_range(g.A, g.K, o.M, g.lda, "A^T");
-      else check_range(g.A, o.M, g.K, g.lda, "A");
-      if (g.flags & 2) check_range(g.B, o.N, g.K, g.ldb, "B^T");
-      else check_range(g.B, g.K, o.N, g.ldb, "B");
+      if (!(g.flags & 1 ? in_allocation(g.A, g.K, o.M, g.lda, ca) : in_allocation(g.A, o.M, g.K, g.lda, ca)) ||
+          !(g.flags & 2 ? in_allocation(g.B, o.N, g.K, g.ldb, cb) : in_allocation(g.B, g.K, o.N, g.ldb, cb)))
+        return false;
     }
   }
+  return true;
+}
+
+bool Engine::outputs_ok(const AxpyPlan& p, int o0, int o1) const {
+  AllocCache cs, cd;
+  for (int i = o0; i < o1; ++i) {
+    const AxpyOut& o = p.outs[i];
+    if (!in_allocation(o.dst, 1, o.len, o.len, cd)) return false;
+    for (int t = o.t0; t < o.t1; ++t)
+      if (!in_allocation(p.terms[t].src, 1, o.len, o.len, cs)) return false;
+  }
+  return true;
+}
+
+namespace {
+// outputs of a plan in blocks of about 4096 terms on the host pool (one block: here)
+template <class Plan, class F>
+bool all_blocks(const Plan& p, const F& ok) {
+  const int no = (int)p.outs.size();
+  const int nb = (int)std::min<size_t>(64, (p.terms.size() + p.outs.size()) / 4096 + 1);
+  if (nb == 1) return ok(0, no);
+  std::atomic<int> bad(0);
+  parallel_for(nb, [&](int b) {
+    if (!ok((int)((int64_t)no * b / nb), (int)((int64_t)no * (b + 1) / nb))) bad = 1;
+  });
+  return !bad;
+}
+}  // namespace
+
+void Engine::check(const GemmPlan& p) const {
+  if (!all_blocks(p, [&](int a, int b) { return outputs_ok(p, a, b); }))
+    throw Error(-6, "plan check: a block of a grouped GEMM exceeds its allocation");
 }
 
 void Engine::check(const AxpyPlan& p) const {
-  for (const auto& o : p.outs) {
-    check_range(o.dst, 1, o.len, o.len, "axpy dst");
-    for (int t = o.t0; t < o.t1; ++t) check_range(p.terms[t].src, 1, o.len, o.len, "axpy src");
-  }
+  if (!all_blocks(p, [&](int a, int b) { return outputs_ok(p, a, b); }))
+    throw Error(-6, "plan check: a block of an axpy exceeds its allocation");
 }
 
 void Engine::sync() {
@@ -446,6 +477,15 @@ cudaEvent_t Engine::pool_event() {
 }
 
 void Engine::h2d(void* dst, const void* src, size_t bytes) {
+  const Part p{src, bytes};
+  h2d(dst, &p, 1);
+}
+
+void Engine::h2d(void* dst, const Part* parts, int np) {
+  size_t bytes = 0;   // the last part's end is not padded
+  for (int i = 0; i < np; ++i)
+    if (parts[i].bytes) bytes = ((bytes + 15) & ~(size_t)15) + parts[i].bytes;
+    else bytes = (bytes + 15) & ~(size_t)15;
   if (bytes == 0) return;
   constexpr size_t kRingMax = (size_t)256 << 20;
   if (pin_ring && bytes > pin_cap / 4 && pin_cap < kRingMax) {
@@ -464,7 +504,12 @@ void Engine::h2d(void* dst, const void* src, size_t bytes) {
     pin_cap = cap;
   }
   if (!pin_ring || bytes > pin_cap / 4) {
-    CK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, stream));
+    size_t off = 0;
+    for (int i = 0; i < np; ++i) {
+      if (parts[i].bytes)
+        CK(cudaMemcpyAsync((uint8_t*)dst + off, parts[i].src, parts[i].bytes, cudaMemcpyHostToDevice, stream));
+      off += (parts[i].bytes + 15) & ~(size_t)15;
+    }
     return;
   }
   const uint64_t n = (bytes + 255) & ~(uint64_t)255;
@@ -483,7 +528,11 @@ void Engine::h2d(void* dst, const void* src, size_t bytes) {
     pin_inflight.pop_front();
   }
   uint8_t* slot = pin_ring + (start % pin_cap);
-  std::memcpy(slot, src, bytes);
+  size_t at = 0;
+  for (int i = 0; i < np; ++i) {
+    if (parts[i].bytes) std::memcpy(slot + at, parts[i].src, parts[i].bytes);
+    at += (parts[i].bytes + 15) & ~(size_t)15;
+  }
   CK(cudaMemcpyAsync(dst, slot, bytes, cudaMemcpyHostToDevice, stream));
   cudaEvent_t e = pool_event();
   CK(cudaEventRecord(e, stream));
@@ -515,8 +564,6 @@ std::pair<int, int> cut_block(int M, int N, int cap) {
 
 void Engine::upload(GemmPlan& p) {
   check(p);
-  p.d_terms = dalloc<GemmTerm>(p.terms.size());
-  p.d_outs = dalloc<GemmOut>(p.outs.size());
   // A plan of results: the tensor-core kernel with split operands, except
   // for small outputs.  A K step of it takes about as long for 8 x 8 outputs
   // as for 32 x 64, so it needs work to pay: at least 4096 products per step,
@@ -526,19 +573,18 @@ void Engine::upload(GemmPlan& p) {
   p.split.clear();
   std::vector<std::pair<int64_t, int>> fma;   // chain length and output
   int64_t fma_elems = 0;
-  std::vector<int64_t> steps(p.outs.size(), 0);   // K steps of the split kernel per output
+  std::vector<std::pair<int64_t, int>> split;   // K steps and output
   for (int o = 0; o < (int)p.outs.size(); ++o) {
     const GemmOut& g = p.outs[o];
     const int64_t elems = (int64_t)g.M * g.N;
     if (elems == 0) continue;
-    int64_t ksum = 0;
+    int64_t ksum = 0, steps = 0;
     for (int t = g.t0; t < g.t1; ++t) {
       ksum += p.terms[t].K;
-      steps[o] += (p.terms[t].K + kSplitChunk - 1) / kSplitChunk;
+      steps += (p.terms[t].K + kSplitChunk - 1) / kSplitChunk;
     }
-    if (p.result && elems * ksum >= std::min<int64_t>(4096 * std::max<int64_t>(steps[o], 1), 1 << 20)) {
-      for (int tm = 0; tm * kSplitTileM < g.M; ++tm)
-        for (int tn = 0; tn * kSplitTileN < g.N; ++tn) p.split.push_back({o, tm, tn, 0});
+    if (p.result && elems * ksum >= std::min<int64_t>(4096 * std::max<int64_t>(steps, 1), 1 << 20)) {
+      split.push_back({steps, o});
       continue;
     }
     fma.push_back({ksum, o});
@@ -553,33 +599,57 @@ void Engine::upload(GemmPlan& p) {
   while (cap > 32 && fma_elems < (int64_t)8 * num_sms * cap) cap /= 2;
   p.per_lane = cap > 128 ? 2 : 1;
   p.tile_span = 0;
-  // longest chains first
-  std::stable_sort(fma.begin(), fma.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  // longest chains first, to within a sixteenth of a power of two
+  auto longest_first = [](const std::vector<std::pair<int64_t, int>>& v, std::vector<int>& order) {
+    std::vector<int> bucket(v.size()), start(1026, 0);
+    for (size_t i = 0; i < v.size(); ++i) {
+      int e;
+      const double m = std::frexp((double)(v[i].first + 1), &e);   // 0.5 <= m < 1
+      bucket[i] = std::max(0, 1023 - (e * 16 + (int)((m - 0.5) * 32)));
+      start[bucket[i] + 1]++;
+    }
+    for (int b = 0; b < 1025; ++b) start[b + 1] += start[b];
+    order.resize(v.size());
+    for (size_t i = 0; i < v.size(); ++i) order[start[bucket[i]]++] = (int)i;
+  };
+  std::vector<int> order;
+  longest_first(fma, order);
   std::unordered_map<uint64_t, std::pair<int, int>> cuts;   // block sizes repeat
-  for (const auto& f : fma) {
-    const GemmOut& g = p.outs[f.second];
-    auto& c = cuts[(uint64_t)g.M << 32 | (uint32_t)g.N];
-    if (c.first == 0) c = cut_block(g.M, g.N, cap);
+  p.tiles.reserve(fma.size() + fma_elems / cap);
+  for (int i : order) {
+    const int out = fma[i].second;
+    const GemmOut& g = p.outs[out];
+    std::pair<int, int> c(g.M, g.N);
+    if (g.M > kFmaSide || g.N > kFmaSide || g.M * g.N > cap) {
+      auto& m = cuts[(uint64_t)g.M << 32 | (uint32_t)g.N];
+      if (m.first == 0) m = cut_block(g.M, g.N, cap);
+      c = m;
+    }
     p.tile_span = std::max(p.tile_span, (c.first | 1) + (c.second | 1));
     for (int m = 0; m < g.M; m += c.first)
       for (int n = 0; n < g.N; n += c.second)
-        p.tiles.push_back({f.second, m, n, std::min(c.first, g.M - m) << 16 | std::min(c.second, g.N - n)});
+        p.tiles.push_back({out, m, n, std::min(c.first, g.M - m) << 16 | std::min(c.second, g.N - n)});
   }
-  std::stable_sort(p.split.begin(), p.split.end(),
-                   [&](const GemmTile& a, const GemmTile& b) { return steps[a.out] > steps[b.out]; });
-  p.d_tiles = dalloc<GemmTile>(std::max<size_t>(p.tiles.size(), 1));
-  p.d_split = dalloc<GemmTile>(std::max<size_t>(p.split.size(), 1));
-  h2d(p.d_terms, p.terms.data(), p.terms.size() * sizeof(GemmTerm));
-  h2d(p.d_outs, p.outs.data(), p.outs.size() * sizeof(GemmOut));
-  h2d(p.d_tiles, p.tiles.data(), p.tiles.size() * sizeof(GemmTile));
-  h2d(p.d_split, p.split.data(), p.split.size() * sizeof(GemmTile));
+  longest_first(split, order);
+  for (int i : order) {
+    const int out = split[i].second;
+    for (int tm = 0; tm * kSplitTileM < p.outs[out].M; ++tm)
+      for (int tn = 0; tn * kSplitTileN < p.outs[out].N; ++tn) p.split.push_back({out, tm, tn, 0});
+  }
+  uint8_t* at[4];
+  p.d_lists = upload_lists<4>({{p.terms.data(), p.terms.size() * sizeof(GemmTerm)},
+                               {p.outs.data(), p.outs.size() * sizeof(GemmOut)},
+                               {p.tiles.data(), p.tiles.size() * sizeof(GemmTile)},
+                               {p.split.data(), p.split.size() * sizeof(GemmTile)}}, at);
+  p.d_terms = (GemmTerm*)at[0];
+  p.d_outs = (GemmOut*)at[1];
+  p.d_tiles = (GemmTile*)at[2];
+  p.d_split = (GemmTile*)at[3];
 }
 
 void Engine::release(GemmPlan& p) {
-  dfree(p.d_terms);
-  dfree(p.d_outs);
-  dfree(p.d_tiles);
-  dfree(p.d_split);
+  dfree(p.d_lists);
+  p.d_lists = nullptr;
   p.d_terms = nullptr;
   p.d_outs = nullptr;
   p.d_tiles = nullptr;
@@ -596,18 +666,18 @@ void Engine::upload(AxpyPlan& p) {
     p.nchunks += (p.outs[o].len + kAxpyChunk - 1) / kAxpyChunk;
     p.bytes += 8.0 * (p.outs[o].t1 - p.outs[o].t0 + 1) * (double)p.outs[o].len;
   }
-  p.d_terms = dalloc<AxpyTerm>(p.terms.size());
-  p.d_outs = dalloc<AxpyOut>(p.outs.size());
-  p.d_cstart = dalloc<int64_t>(p.cstart.size());
-  h2d(p.d_terms, p.terms.data(), p.terms.size() * sizeof(AxpyTerm));
-  h2d(p.d_outs, p.outs.data(), p.outs.size() * sizeof(AxpyOut));
-  h2d(p.d_cstart, p.cstart.data(), p.cstart.size() * sizeof(int64_t));
+  uint8_t* at[3];
+  p.d_lists = upload_lists<3>({{p.terms.data(), p.terms.size() * sizeof(AxpyTerm)},
+                               {p.outs.data(), p.outs.size() * sizeof(AxpyOut)},
+                               {p.cstart.data(), p.cstart.size() * sizeof(int64_t)}}, at);
+  p.d_terms = (AxpyTerm*)at[0];
+  p.d_outs = (AxpyOut*)at[1];
+  p.d_cstart = (int64_t*)at[2];
 }
 
 void Engine::release(AxpyPlan& p) {
-  dfree(p.d_terms);
-  dfree(p.d_outs);
-  dfree(p.d_cstart);
+  dfree(p.d_lists);
+  p.d_lists = nullptr;
   p.d_terms = nullptr;
   p.d_outs = nullptr;
   p.d_cstart = nullptr;
@@ -786,22 +856,39 @@ struct EnlPart {
   int64_t own = 0;
 };
 void merge_parts(std::vector<EnlPart>& parts, EnlOp& op, AxpyPlan& ax) {
-  for (EnlPart& P : parts) {
-    const int64_t ob = op.own_size;
-    const int tb = (int)ax.terms.size();
-    for (EnlSub s : P.subs) {
-      if (s.own_off >= 0) s.own_off += ob;
-      op.subs.push_back(s);
+  // where each share goes, then the copies on the host pool
+  struct At { size_t sub, out, term; int64_t own; };
+  std::vector<At> at(parts.size() + 1);
+  at[0] = {op.subs.size(), ax.outs.size(), ax.terms.size(), op.own_size};
+  for (size_t u = 0; u < parts.size(); ++u)
+    at[u + 1] = {at[u].sub + parts[u].subs.size(), at[u].out + parts[u].outs.size(),
+                 at[u].term + parts[u].terms.size(), at[u].own + parts[u].own};
+  op.subs.resize(at.back().sub);
+  ax.outs.resize(at.back().out);
+  ax.terms.resize(at.back().term);
+  op.own_size = at.back().own;
+  auto copy = [&](int u) {
+    EnlPart& P = parts[u];
+    EnlSub* s = op.subs.data() + at[u].sub;
+    for (const EnlSub& x : P.subs) {
+      *s = x;
+      if (s->own_off >= 0) s->own_off += at[u].own;
+      ++s;
     }
-    for (AxpyOut o : P.outs) {
-      o.dst = (double*)((intptr_t)o.dst + ob);   // element offsets until finish_enl
-      o.t0 += tb;
-      o.t1 += tb;
-      ax.outs.push_back(o);
+    AxpyOut* o = ax.outs.data() + at[u].out;
+    for (const AxpyOut& x : P.outs) {
+      *o = x;
+      o->dst = (double*)((intptr_t)x.dst + at[u].own);   // element offsets until finish_enl
+      o->t0 += (int)at[u].term;
+      o->t1 += (int)at[u].term;
+      ++o;
     }
-    ax.terms.insert(ax.terms.end(), P.terms.begin(), P.terms.end());
-    op.own_size += P.own;
-  }
+    std::copy(P.terms.begin(), P.terms.end(), ax.terms.begin() + at[u].term);
+  };
+  if (at.back().sub + at.back().term < 16384)
+    for (int u = 0; u < (int)parts.size(); ++u) copy(u);
+  else
+    parallel_for((int)parts.size(), copy);
 }
 }  // namespace
 
@@ -952,13 +1039,28 @@ void Engine::append_conjugates(EnlOp& op, int bond, bool left) const {
   const auto& sg = left ? sign_l : sign_r;
   if (bond >= (int)cj.size()) return;
   const int nch = (int)cj[bond].size();
-  std::vector<std::vector<size_t>> by((size_t)nch);
+  // sub-blocks of every channel (counting sort, order kept), then the place
+  // of every derived channel's copies
   const size_t n0 = op.subs.size();
-  for (size_t i = 0; i < n0; ++i) by[op.subs[i].b].push_back(i);
+  std::vector<size_t> start((size_t)nch + 1, 0), at((size_t)nch + 1, n0);
+  for (size_t i = 0; i < n0; ++i) start[op.subs[i].b + 1]++;
+  for (int c = 0; c < nch; ++c) start[c + 1] += start[c];
+  std::vector<int> idx(n0);
+  {
+    std::vector<size_t> fill(start.begin(), start.end() - 1);
+    for (size_t i = 0; i < n0; ++i) idx[fill[op.subs[i].b]++] = (int)i;
+  }
   for (int d = 0; d < nch; ++d) {
-    if (!env_derived(bond, d, left)) continue;
-    for (size_t i : by[cj[bond][d]]) {
-      const EnlSub s = op.subs[i];
+    const int c = cj[bond][d];
+    at[d + 1] = at[d] + (env_derived(bond, d, left) ? start[c + 1] - start[c] : 0);
+  }
+  op.subs.resize(at[nch]);
+  auto copy = [&](int d) {
+    size_t o = at[d];
+    if (at[d + 1] == o) return;
+    const int c = cj[bond][d];
+    for (size_t i = start[c]; i < start[c + 1]; ++i) {
+      const EnlSub s = op.subs[idx[i]];
       EnlSub t = s;
       t.b = d;
       t.qin = s.qout;
@@ -969,9 +1071,13 @@ void Engine::append_conjugates(EnlOp& op, int bond, bool left) const {
       t.cols = s.rows;
       t.sign = s.sign * sg[bond][d];
       t.trans = s.trans ^ 1;
-      op.subs.push_back(t);
+      op.subs[o++] = t;
     }
-  }
+  };
+  if (at[nch] - n0 < 16384)
+    for (int d = 0; d < nch; ++d) copy(d);
+  else
+    parallel_for(nch, copy);
 }
 
 void Engine::finish_enl(EnlOp& op, AxpyPlan& ax) {
@@ -1312,20 +1418,29 @@ struct Engine::Sigma {
 };
 
 void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool result) {
-  // Y_b(Qin) exists when both operators have sub-blocks for (b, Qin)
-  std::map<std::pair<int, int>, std::vector<const EnlSub*>> rby, lby;
-  for (const auto& s : renl.subs) rby[{s.b, s.qin}].push_back(&s);
-  for (const auto& s : lenl.subs) lby[{s.b, s.qin}].push_back(&s);
-  std::map<std::pair<int, int>, int64_t> yoff;
+  // Y_b(Qin) exists when both operators have sub-blocks for (b, Qin), key b nq + Qin
+  const int nq = EL.n();
+  const SubGroups rby(renl, nq);
+  std::vector<char> has_l((size_t)rby.nkeys, 0);
+  std::vector<int> lstart((size_t)nq * 4 + 1, 0), lout(lenl.subs.size());   // Lenl subs by (Qout, sout)
+  for (const auto& s : lenl.subs) {
+    const size_t key = (size_t)s.b * nq + s.qin;
+    if (key < has_l.size()) has_l[key] = 1;
+    lstart[s.qout * 4 + s.sout + 1]++;
+  }
+  for (int i = 0; i < nq * 4; ++i) lstart[i + 1] += lstart[i];
+  {
+    std::vector<int> fill(lstart.begin(), lstart.end() - 1);
+    for (size_t i = 0; i < lenl.subs.size(); ++i) lout[fill[lenl.subs[i].qout * 4 + lenl.subs[i].sout]++] = (int)i;
+  }
+  std::vector<int64_t> yoff((size_t)rby.nkeys, -1);
+  std::vector<int> ys;   // keys with a Y block
   int64_t ysize = 0;
-  std::vector<std::tuple<int, int, int>> ys;   // b, qin, qout
-  for (auto& kv : rby) {
-    if (!lby.count(kv.first)) continue;
-    int qin = kv.first.second;
-    int qout = kv.second[0]->qout;
-    yoff[kv.first] = ysize;
-    ys.push_back({kv.first.first, qin, qout});
-    ysize += (int64_t)EL.dim[qin] * ER.dim[qout];
+  for (int key = 0; key < rby.nkeys; ++key) {
+    if (rby.start[key] == rby.start[key + 1] || !has_l[key]) continue;
+    yoff[key] = ysize;
+    ys.push_back(key);
+    ysize += (int64_t)EL.dim[key % nq] * ER.dim[renl.subs[rby.idx[rby.start[key]]].qout];
   }
   sg.Y = dalloc<double>(ysize);
   sg.in = dalloc<double>(psi_size);
@@ -1335,16 +1450,21 @@ void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool re
   A.clear();
   B.clear();
   A.result = B.result = result;
+  A.outs.reserve(ys.size() * 4);
+  A.terms.reserve(renl.subs.size());
+  B.terms.reserve(lenl.subs.size());
   // stage A: Y_b(Qin)[:, cols (sout, q_r')] = sum psi(Qin)[:, cols (sin, q_r)] Rsub^T
-  for (auto& y : ys) {
-    int b = std::get<0>(y), qin = std::get<1>(y), qout = std::get<2>(y);
-    double* Yb = sg.Y + yoff[{b, qin}];
+  for (int key : ys) {
+    const int qin = key % nq;
+    const int i0 = rby.start[key], i1 = rby.start[key + 1];
+    const int qout = renl.subs[rby.idx[i0]].qout;
+    double* Yb = sg.Y + yoff[key];
     int ldy = ER.dim[qout];
-    const auto& subs = rby[{b, qin}];
     for (int so = 0; so < 4; ++so) {
       if (ER.soff[qout][so] < 0) continue;
       A.add_out(Yb + ER.soff[qout][so], ldy, EL.dim[qin], ER.sdim[qout][so], 0);
-      for (const EnlSub* s : subs) {
+      for (int i = i0; i < i1; ++i) {
+        const EnlSub* s = &renl.subs[rby.idx[i]];
         if (s->sout != so) continue;
         if (s->trans)   // Rsub^T = sign * (the block at ptr), cols x rows
           A.add_term(sg.in + psi_off[qin] + ER.soff[qin][s->sin], ER.dim[qin], s->ptr, s->rows, s->cols, 0, s->sign);
@@ -1354,19 +1474,16 @@ void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool re
     }
   }
   // stage B: sigma(Qout)[rows (q_l', sout), :] = sum Lsub Y_b(Qin)[rows (q_l, sin), :]
-  std::map<std::pair<int, int>, std::vector<const EnlSub*>> lout;
-  for (const auto& s : lenl.subs) lout[{s.qout, s.sout}].push_back(&s);
-  for (int q = 0; q < EL.n(); ++q)
+  for (int q = 0; q < nq; ++q)
     for (int so = 0; so < 4; ++so) {
       if (EL.soff[q][so] < 0) continue;
       int ld = ER.dim[q];
       B.add_out(sg.out + psi_off[q] + (int64_t)EL.soff[q][so] * ld, ld, EL.sdim[q][so], ld, 0);
-      auto it = lout.find({q, so});
-      if (it == lout.end()) continue;
-      for (const EnlSub* s : it->second) {
-        auto yo = yoff.find({s->b, s->qin});
-        if (yo == yoff.end()) continue;
-        B.add_term(s->ptr, s->trans ? s->rows : s->cols, sg.Y + yo->second + (int64_t)EL.soff[s->qin][s->sin] * ld, ld,
+      for (int i = lstart[q * 4 + so]; i < lstart[q * 4 + so + 1]; ++i) {
+        const EnlSub* s = &lenl.subs[lout[i]];
+        const size_t key = (size_t)s->b * nq + s->qin;
+        if (key >= yoff.size() || yoff[key] < 0) continue;
+        B.add_term(s->ptr, s->trans ? s->rows : s->cols, sg.Y + yoff[key] + (int64_t)EL.soff[s->qin][s->sin] * ld, ld,
                    s->cols, s->trans ? 1 : 0, s->sign);
       }
     }
@@ -1409,30 +1526,26 @@ void Engine::compute_diag(const EnlOp& lenl, const EnlOp& renl, double* diag) {
   double* DR = dalloc<double>(dr_off.back());
   CK(cudaMemsetAsync(DL, 0, dl_off.back() * sizeof(double), stream));
   CK(cudaMemsetAsync(DR, 0, dr_off.back() * sizeof(double), stream));
-  // gathers expressed as 1-wide GEMMs would be wasteful; use strided axpy:
-  // each diagonal element is one 1x1 output of a GEMM with K=1 (A = element,
-  // B = 1).  Cheaper: copy via the axpy kernel on strided views is not
-  // supported, so gather on the device with tiny GEMMs of shape m x 1.
-  GemmPlan g;
-  static const double one = 1.0;
-  double* d_one = dalloc<double>(1);
-  h2d(d_one, &one, sizeof(double));
-  for (const auto& s : lenl.subs) {
+  std::vector<GatherTask> g;
+  AllocCache cache;
+  auto gather = [&](const EnlSub& s, double* dst, int dstep) {
+    if (!in_allocation(s.ptr, s.rows, s.cols, s.cols, cache)) throw Error(-6, "plan check: diagonal outside its allocation");
+    g.push_back({s.ptr, dst, s.rows, s.cols + 1, dstep, 0, s.sign});
+  };
+  for (const auto& s : lenl.subs) {   // column col of DL(q), rows from the section's offset
     if (s.qin != s.qout || s.sin != s.sout || col[s.b] < 0 || s.rows != s.cols) continue;
-    // column vector of the diagonal: rows r -> DL(q)[soff + r, col]
-    // express as M=rows, N=1, K=1 with A = diag elements (lda = cols+1), B = one
-    g.add_out(DL + dl_off[s.qin] + (int64_t)EL.soff[s.qin][s.sin] * nz + col[s.b], nz, s.rows, 1, 0);
-    g.add_term(s.ptr, s.cols + 1, d_one, 1, 1, 0, s.sign);
+    gather(s, DL + dl_off[s.qin] + (int64_t)EL.soff[s.qin][s.sin] * nz + col[s.b], nz);
   }
-  for (const auto& s : renl.subs) {
+  for (const auto& s : renl.subs) {   // row col of DR(q), columns from the section's offset
     if (s.qin != s.qout || s.sin != s.sout || col[s.b] < 0 || s.rows != s.cols) continue;
-    // row vector: DR(q)[col, soff + r]: M=1, N=rows, K=1, A = one, B = diag (ldb = cols+1, transB)
-    g.add_out(DR + dr_off[s.qin] + (int64_t)col[s.b] * ER.dim[s.qin] + ER.soff[s.qin][s.sin], 1, 1, s.rows, 0);
-    g.add_term(d_one, 1, s.ptr, s.cols + 1, 1, 2, s.sign);
+    gather(s, DR + dr_off[s.qin] + (int64_t)col[s.b] * ER.dim[s.qin] + ER.soff[s.qin][s.sin], 1);
   }
-  upload(g);
-  run(g);
-  release(g);
+  uint8_t* at[1];
+  void* d_g = upload_lists<1>({{g.data(), g.size() * sizeof(GatherTask)}}, at);
+  launch_gather((GatherTask*)at[0], (int)g.size(), stream);
+  stats.launches++;
+  CK(cudaGetLastError());
+  dfree(d_g);
   GemmPlan p;
   for (int q = 0; q < EL.n(); ++q) {
     p.add_out(diag + psi_off[q], ER.dim[q], EL.dim[q], ER.dim[q], 0);
@@ -1443,7 +1556,6 @@ void Engine::compute_diag(const EnlOp& lenl, const EnlOp& renl, double* diag) {
   release(p);
   dfree(DL);
   dfree(DR);
-  dfree(d_one);
 }
 
 // Shift-and-invert inner PCG on the projected correction equation

@@ -343,6 +343,9 @@ class Engine {
   // live allocation
   struct AllocCache { uintptr_t base = 0; size_t size = 0; };
   bool in_allocation(const void* p, int64_t rows, int64_t cols, int64_t ld, AllocCache& c) const;
+  // the ranges of outputs [o0, o1) of a plan (no shared cache)
+  bool outputs_ok(const GemmPlan& p, int o0, int o1) const;
+  bool outputs_ok(const AxpyPlan& p, int o0, int o1) const;
   const double* site_block(int i, int qi, int s, int& ld) const;
   void check(const GemmPlan& p) const;
   void check(const AxpyPlan& p) const;
@@ -369,6 +372,24 @@ class Engine {
   std::vector<cudaEvent_t> ev_pool;        // timing-disabled events for the ring
   cudaEvent_t pool_event();
   void h2d(void* dst, const void* src, size_t bytes);
+  // several host lists into one device buffer, each from a multiple of 16
+  // bytes: one staged region, one copy
+  struct Part { const void* src; size_t bytes; };
+  void h2d(void* dst, const Part* parts, int n);
+  // device copies of several lists in one allocation; at[i] = list i there
+  template <int N>
+  void* upload_lists(const Part (&parts)[N], uint8_t* (&at)[N]) {
+    size_t total = 0;
+    size_t off[N];
+    for (int i = 0; i < N; ++i) {
+      off[i] = total;
+      total += (parts[i].bytes + 15) & ~(size_t)15;
+    }
+    uint8_t* d = dalloc<uint8_t>(total);
+    for (int i = 0; i < N; ++i) at[i] = d + off[i];
+    h2d(d, parts, N);
+    return d;
+  }
   // environment-update launches timed by event pairs, read after the next
   // stream synchronisation (no synchronisation of their own)
   struct EnvTimer { cudaEvent_t a, b; double* acc; };   // acc: the stats counter the time goes to

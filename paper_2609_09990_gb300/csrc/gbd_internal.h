@@ -108,6 +108,7 @@ struct GemmPlan {       // host side lists plus their device copies
   std::vector<GemmOut> outs;
   std::vector<GemmTile> tiles;   // FMA kernel: {out, first row, first column, rows << 16 | columns}
   std::vector<GemmTile> split;   // 32 x 64 tiles of the tensor-core kernel with split operands
+  void* d_lists = nullptr;       // the device copies, in one allocation
   GemmTerm* d_terms = nullptr;
   GemmOut* d_outs = nullptr;
   GemmTile* d_tiles = nullptr;
@@ -143,6 +144,7 @@ struct AxpyPlan {
   std::vector<AxpyTerm> terms;
   std::vector<AxpyOut> outs;
   std::vector<int64_t> cstart;   // first work chunk of every output (upload fills it)
+  void* d_lists = nullptr;       // the device copies, in one allocation
   AxpyTerm* d_terms = nullptr;
   AxpyOut* d_outs = nullptr;
   int64_t* d_cstart = nullptr;
@@ -162,6 +164,9 @@ constexpr int kSplitTileM = 32, kSplitTileN = 64, kSplitChunk = 32;
 int launch_gemm_f64(const GemmPlan& p, cudaStream_t s);
 int launch_gemm_f64_split(const GemmPlan& p, cudaStream_t s);
 void launch_axpy(const AxpyPlan& p, cudaStream_t s);
+// dst[i * dstep] = coef * src[i * sstep], i < len, for every task
+struct GatherTask { const double* src; double* dst; int32_t len, sstep, dstep, pad; double coef; };
+void launch_gather(const GatherTask* tasks, int ntasks, cudaStream_t s);
 void launch_set_identity(double* d, int m, cudaStream_t s);
 // dst = sign * src^T for blocks src (rows x cols, row-major, dense); one
 // 32 x 32 tile per item

@@ -257,6 +257,16 @@ __global__ void __launch_bounds__(kAxpyThreads) axpy_kernel(const AxpyTerm* __re
   }
 }
 
+// one warp per strided vector (the diagonals of the enlarged operators: a few
+// tens of elements each, thousands of them; latency is all there is to hide)
+__global__ void gather_kernel(const GatherTask* __restrict__ tasks, int ntasks) {
+  const int t = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+  if (t >= ntasks) return;
+  const GatherTask g = tasks[t];
+  for (int i = threadIdx.x & 31; i < g.len; i += 32)
+    g.dst[(int64_t)i * g.dstep] = fma(g.coef, g.src[(int64_t)i * g.sstep], 0.0);
+}
+
 __global__ void set_identity_kernel(double* d, int m) {
   int64_t n = (int64_t)m * m;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
@@ -409,6 +419,10 @@ int launch_gemm_f64(const GemmPlan& p, cudaStream_t s) {
   if (nt > 0 && p.per_lane == 2) gemm_f64_kernel<2><<<nt, FT + 32, smem, s>>>(p.d_terms, p.d_outs, p.d_tiles);
   if (nt > 0 && p.per_lane == 1) gemm_f64_kernel<1><<<nt, FT + 32, smem, s>>>(p.d_terms, p.d_outs, p.d_tiles);
   return ns + (nt > 0);
+}
+
+void launch_gather(const GatherTask* tasks, int ntasks, cudaStream_t s) {
+  if (ntasks > 0) gather_kernel<<<(ntasks + 7) / 8, 256, 0, s>>>(tasks, ntasks);
 }
 
 void launch_axpy(const AxpyPlan& p, cudaStream_t s) {
