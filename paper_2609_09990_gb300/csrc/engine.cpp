@@ -333,7 +333,7 @@ Engine::~Engine() {
   free_snapshot();
   clear_states();
   if (psi) dfree(psi);
-  if (d_env_err) dfree(d_env_err);
+  if (d_wait_err) dfree(d_wait_err);
   cudaStreamSynchronize(stream);
   for (auto& u : pin_inflight) cudaEventDestroy(u.ev);
   for (cudaEvent_t e : ev_pool) cudaEventDestroy(e);
@@ -449,11 +449,11 @@ void Engine::sync() {
 }
 
 void Engine::drain_timers() {
-  if (env_tc_pending) {
-    env_tc_pending = false;
+  if (wait_pending) {
+    wait_pending = false;
     int flag = 0;
-    CK(cudaMemcpy(&flag, d_env_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (flag) throw Error(-5, "tensor-core environment update: a bounded device wait ran out");
+    CK(cudaMemcpy(&flag, d_wait_err, sizeof(int), cudaMemcpyDeviceToHost));
+    if (flag) throw Error(-5, "grouped GEMM on the tensor cores: a bounded device wait ran out");
   }
   for (auto& t : env_timers) {
     float ms = 0;
@@ -560,17 +560,30 @@ std::pair<int, int> cut_block(int M, int N, int cap) {
   }
   return best;
 }
+
+// order of the entries, largest first to within a sixteenth of a power of two
+void longest_first(const std::vector<std::pair<int64_t, int>>& v, std::vector<int>& order) {
+  std::vector<int> bucket(v.size()), start(1026, 0);
+  for (size_t i = 0; i < v.size(); ++i) {
+    int e;
+    const double m = std::frexp((double)(v[i].first + 1), &e);   // 0.5 <= m < 1
+    bucket[i] = std::max(0, 1023 - (e * 16 + (int)((m - 0.5) * 32)));
+    start[bucket[i] + 1]++;
+  }
+  for (int b = 0; b < 1025; ++b) start[b + 1] += start[b];
+  order.resize(v.size());
+  for (size_t i = 0; i < v.size(); ++i) order[start[bucket[i]]++] = (int)i;
+}
 }  // namespace
 
 void Engine::upload(GemmPlan& p) {
   check(p);
   // A plan of results: the tensor-core kernel with split operands, except
   // for small outputs.  A K step of it takes about as long for 8 x 8 outputs
-  // as for 32 x 64, so it needs work to pay: at least 4096 products per step,
-  // or a large output in all (CAS(16,16) M=512: H_eff product 79 -> 21 ms,
-  // RDMs 240 -> 142 ms; CAS(9,9) 3-RDM 352 -> 93 ms).
+  // as for 64 x 64, so it needs work to pay: at least 4096 products per step,
+  // or a large output in all (everything on it: CAS(13,11) M=200 orbital RDMs
+  // 10.1 ms instead of 7.5 ms).
   p.tiles.clear();
-  p.split.clear();
   std::vector<std::pair<int64_t, int>> fma;   // chain length and output
   int64_t fma_elems = 0;
   std::vector<std::pair<int64_t, int>> split;   // K steps and output
@@ -599,19 +612,6 @@ void Engine::upload(GemmPlan& p) {
   while (cap > 32 && fma_elems < (int64_t)8 * num_sms * cap) cap /= 2;
   p.per_lane = cap > 128 ? 2 : 1;
   p.tile_span = 0;
-  // longest chains first, to within a sixteenth of a power of two
-  auto longest_first = [](const std::vector<std::pair<int64_t, int>>& v, std::vector<int>& order) {
-    std::vector<int> bucket(v.size()), start(1026, 0);
-    for (size_t i = 0; i < v.size(); ++i) {
-      int e;
-      const double m = std::frexp((double)(v[i].first + 1), &e);   // 0.5 <= m < 1
-      bucket[i] = std::max(0, 1023 - (e * 16 + (int)((m - 0.5) * 32)));
-      start[bucket[i] + 1]++;
-    }
-    for (int b = 0; b < 1025; ++b) start[b + 1] += start[b];
-    order.resize(v.size());
-    for (size_t i = 0; i < v.size(); ++i) order[start[bucket[i]]++] = (int)i;
-  };
   std::vector<int> order;
   longest_first(fma, order);
   std::unordered_map<uint64_t, std::pair<int, int>> cuts;   // block sizes repeat
@@ -630,30 +630,119 @@ void Engine::upload(GemmPlan& p) {
       for (int n = 0; n < g.N; n += c.second)
         p.tiles.push_back({out, m, n, std::min(c.first, g.M - m) << 16 | std::min(c.second, g.N - n)});
   }
-  longest_first(split, order);
-  for (int i : order) {
-    const int out = split[i].second;
-    for (int tm = 0; tm * kSplitTileM < p.outs[out].M; ++tm)
-      for (int tn = 0; tn * kSplitTileN < p.outs[out].N; ++tn) p.split.push_back({out, tm, tn, 0});
+  plan_split(p, split);
+  if (!p.swork.empty()) {
+    p.d_digits = dalloc<uint8_t>(p.digit_bytes);
+    p.d_part = dalloc<double>(p.part_slots * kSplitTile * kSplitTile);
   }
-  uint8_t* at[4];
-  p.d_lists = upload_lists<4>({{p.terms.data(), p.terms.size() * sizeof(GemmTerm)},
+  uint8_t* at[7];
+  p.d_lists = upload_lists<7>({{p.terms.data(), p.terms.size() * sizeof(GemmTerm)},
                                {p.outs.data(), p.outs.size() * sizeof(GemmOut)},
                                {p.tiles.data(), p.tiles.size() * sizeof(GemmTile)},
-                               {p.split.data(), p.split.size() * sizeof(GemmTile)}}, at);
+                               {p.operands.data(), p.operands.size() * sizeof(SplitOperand)},
+                               {p.sterms.data(), p.sterms.size() * sizeof(SplitTerm)},
+                               {p.swork.data(), p.swork.size() * sizeof(SplitWork)},
+                               {p.ssums.data(), p.ssums.size() * sizeof(SplitSum)}}, at);
   p.d_terms = (GemmTerm*)at[0];
   p.d_outs = (GemmOut*)at[1];
   p.d_tiles = (GemmTile*)at[2];
-  p.d_split = (GemmTile*)at[3];
+  p.d_operands = (SplitOperand*)at[3];
+  p.d_sterms = (SplitTerm*)at[4];
+  p.d_swork = (SplitWork*)at[5];
+  p.d_ssums = (SplitSum*)at[6];
+}
+
+// The split kernel's lists for the outputs `list` (chunks per tile, output):
+// every distinct operand block once, the chunks of every 64 x 64 tile, long
+// chains cut into pieces of about a sixth of an SM's share of all chunks (at
+// least 16: a piece costs a partial tile written and read).  The cuts depend
+// on the plan alone, so results do not depend on the device's load.
+void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>& list) const {
+  p.operands.clear();
+  p.sterms.clear();
+  p.swork.clear();
+  p.ssums.clear();
+  p.split_items = p.digit_bytes = p.part_slots = 0;
+  if (list.empty()) return;
+  size_t nterms = 0;
+  int64_t all = 0;
+  for (const auto& l : list) {
+    const GemmOut& o = p.outs[l.second];
+    nterms += o.t1 - o.t0;
+    all += l.first * ((o.M + kSplitTile - 1) / kSplitTile) * ((o.N + kSplitTile - 1) / kSplitTile);
+  }
+  size_t cap = 64;
+  while (cap < 4 * nterms) cap *= 2;
+  std::vector<int> table(cap, -1);   // open addressing
+  auto operand = [&](const double* src, int ld, int rows, int K, bool kstrided) -> int {
+    uint64_t x = (uint64_t)(uintptr_t)src >> 3;
+    x = (x ^ ((uint64_t)rows << 40) ^ ((uint64_t)K << 52) ^ (uint64_t)kstrided) * 0x9E3779B97F4A7C15ull;
+    for (size_t i = (x >> 20) & (cap - 1);; i = (i + 1) & (cap - 1)) {
+      const int e = table[i];
+      if (e < 0) {
+        table[i] = (int)p.operands.size();
+        const int64_t rp = (rows + 7) / 8 * 8, chunks = (K + kSplitChunk - 1) / kSplitChunk;
+        const int last = K - (int)(chunks - 1) * kSplitChunk;
+        p.operands.push_back({src, ld, rows, K, kstrided, p.digit_bytes, p.split_items});
+        // 7 digit planes of FP16 and an exponent per row and chunk; the last chunk may be 16 wide
+        const int64_t bytes = (chunks - 1) * rp * (7 * 64 + 4) + rp * (7 * (last > 16 ? 64 : 32) + 4);
+        p.digit_bytes += (bytes + 127) / 128 * 128;
+        p.split_items += rp / 8 * chunks;
+        return table[i];
+      }
+      const SplitOperand& o = p.operands[e];
+      if (o.src == src && o.ld == ld && o.rows == rows && o.K == K && o.kstrided == (int)kstrided) return e;
+    }
+  };
+  const int64_t piece = std::max<int64_t>(16, all / (6 * num_sms) + 1);
+  p.sterms.reserve(nterms);
+  std::vector<std::pair<int64_t, int>> work;   // steps, index
+  std::vector<SplitWork> w;
+  std::vector<int64_t> kstep;                  // steps up to every term of the output
+  for (const auto& l : list) {
+    const GemmOut& o = p.outs[l.second];
+    const int t0 = (int)p.sterms.size();
+    kstep.assign(1, 0);
+    for (int t = o.t0; t < o.t1; ++t) {
+      const GemmTerm& g = p.terms[t];
+      if (g.K <= 0) continue;
+      const int a = operand(g.A, g.lda, o.M, g.K, g.flags & 1), b = operand(g.B, g.ldb, o.N, g.K, !(g.flags & 2));
+      p.sterms.push_back({p.operands[a].off, p.operands[b].off, (o.M + 7) / 8 * 8, (o.N + 7) / 8 * 8, g.K, t, g.alpha});
+      kstep.push_back(kstep.back() + (g.K + kSplitChunk - 1) / kSplitChunk);
+    }
+    const int64_t steps = kstep.back();
+    const int pieces = 2 * steps > 3 * piece ? (int)((steps + piece - 1) / piece) : 1;
+    for (int tm = 0; tm * kSplitTile < o.M; ++tm)
+      for (int tn = 0; tn * kSplitTile < o.N; ++tn) {
+        if (pieces > 1) {
+          p.ssums.push_back({l.second, tm, tn, (int)p.part_slots, pieces});
+          p.part_slots += pieces;
+        }
+        for (int i = 0; i < pieces; ++i) {
+          const int64_t s0 = steps * i / pieces, s1 = steps * (i + 1) / pieces;
+          const int t = (int)(std::upper_bound(kstep.begin(), kstep.end(), s0) - kstep.begin()) - 1;
+          work.push_back({s1 - s0, (int)w.size()});
+          w.push_back({l.second, tm, tn, t0 + t, (int)(s0 - kstep[t]) * kSplitChunk, (int)(s1 - s0),
+                       pieces > 1 ? (int)p.part_slots - pieces + i : -1, 0});
+        }
+      }
+  }
+  std::vector<int> order;
+  longest_first(work, order);
+  p.swork.reserve(w.size());
+  for (int i : order) p.swork.push_back(w[i]);
 }
 
 void Engine::release(GemmPlan& p) {
   dfree(p.d_lists);
+  dfree(p.d_digits);
+  dfree(p.d_part);
   p.d_lists = nullptr;
+  p.d_digits = nullptr;
+  p.d_part = nullptr;
   p.d_terms = nullptr;
   p.d_outs = nullptr;
   p.d_tiles = nullptr;
-  p.d_split = nullptr;
 }
 
 void Engine::upload(AxpyPlan& p) {
@@ -684,8 +773,13 @@ void Engine::release(AxpyPlan& p) {
 }
 
 void Engine::run(GemmPlan& p) {
-  if (p.tiles.empty() && p.split.empty()) return;
-  const int l = launch_gemm_f64(p, stream);
+  if (p.tiles.empty() && p.swork.empty()) return;
+  int* err = nullptr;
+  if (!p.swork.empty()) {
+    err = wait_flag();
+    wait_pending = true;
+  }
+  const int l = launch_gemm_f64(p, num_sms, err, stream);
   if (l < 0) throw Error(-3, "grouped GEMM: shared memory refused");
   stats.launches += l;
   CK(cudaGetLastError());

@@ -351,6 +351,7 @@ class Engine {
   void check(const AxpyPlan& p) const;
   void dfree(void* p);
   void upload(GemmPlan& p);
+  void plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>& list) const;
   void release(GemmPlan& p);
   void upload(AxpyPlan& p);
   void release(AxpyPlan& p);
@@ -400,8 +401,17 @@ class Engine {
   // a GemmPlan (every output overwritten) on the tensor cores, operands in
   // precision prec (TcPrec), split-K FP64 sums (gemm_tc.cpp)
   void run_tc(GemmPlan& p, int prec);
-  int* d_env_err = nullptr;      // bounded-wait flag of the tensor-core environment updates
-  bool env_tc_pending = false;   // such launches since the last check of the flag
+  // bounded-wait flag of the tensor-core environment updates and the split
+  // kernel, and whether any was launched since the last check of it
+  int* d_wait_err = nullptr;
+  bool wait_pending = false;
+  int* wait_flag() {
+    if (!d_wait_err) {
+      d_wait_err = dalloc<int>(2);   // [1]: the split kernel's work counter
+      CK(cudaMemsetAsync(d_wait_err, 0, 2 * sizeof(int), stream));
+    }
+    return d_wait_err;
+  }
   EnvTimer timer_begin(double* acc);
   void timer_end(EnvTimer t);
   int sigma_pending = 0;          // 1: FP64 sigma, 2: tensor-core sigma awaiting accounting

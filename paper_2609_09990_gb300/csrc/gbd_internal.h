@@ -103,16 +103,45 @@ struct GemmTile {
   int32_t out, tm, tn, pad;
 };
 
+// Operand block of the split kernel: rows of op(A) or columns of op(B), K long.
+// off: its records in the digit buffer; first: its first group of 8 rows x 32
+// columns in the list of all of them.
+struct SplitOperand {
+  const double* src;
+  int32_t ld, rows, K, kstrided;   // kstrided: consecutive k are ld apart, else consecutive rows
+  int64_t off, first;
+};
+struct SplitTerm {
+  int64_t a, b;          // records of its operands
+  int32_t ra, rb, K;     // rows of the operands rounded up to 8, columns
+  int32_t term;          // its GemmTerm
+  double alpha;
+};
+struct SplitWork {       // `steps` chunks of 32 columns of one tile, from column k0 of sterm t0
+  int32_t out, tm, tn, t0, k0, steps, slot, pad;   // slot: partial sum, -1 = the output itself
+};
+struct SplitSum { int32_t out, tm, tn, slot, count; };
+
 struct GemmPlan {       // host side lists plus their device copies
   std::vector<GemmTerm> terms;
   std::vector<GemmOut> outs;
   std::vector<GemmTile> tiles;   // FMA kernel: {out, first row, first column, rows << 16 | columns}
-  std::vector<GemmTile> split;   // 32 x 64 tiles of the tensor-core kernel with split operands
+  // the tensor-core kernel with split operands (kernels_f64_split.cu)
+  std::vector<SplitOperand> operands;   // the distinct operand blocks
+  std::vector<SplitTerm> sterms;        // the terms of its outputs
+  std::vector<SplitWork> swork;         // 64 x 64 tiles, or pieces of their chains
+  std::vector<SplitSum> ssums;          // tiles cut into pieces
+  int64_t split_items = 0, digit_bytes = 0, part_slots = 0;
   void* d_lists = nullptr;       // the device copies, in one allocation
   GemmTerm* d_terms = nullptr;
   GemmOut* d_outs = nullptr;
   GemmTile* d_tiles = nullptr;
-  GemmTile* d_split = nullptr;
+  SplitOperand* d_operands = nullptr;
+  SplitTerm* d_sterms = nullptr;
+  SplitWork* d_swork = nullptr;
+  SplitSum* d_ssums = nullptr;
+  uint8_t* d_digits = nullptr;   // records of the operands
+  double* d_part = nullptr;      // partial sums
   int tile_span = 0;             // largest rows + columns of a tile (odd pitches)
   int per_lane = 2;              // outputs per lane: tiles of at most 128 per_lane outputs
   double flops = 0.0;       // 2 m n k summed over terms
@@ -122,7 +151,7 @@ struct GemmPlan {       // host side lists plus their device copies
   // false: an unconverged iteration amplifies a change of rounding until
   // its iterates have no digit in common.
   bool result = false;
-  void clear() { terms.clear(); outs.clear(); tiles.clear(); split.clear(); flops = 0.0; }
+  void clear() { terms.clear(); outs.clear(); tiles.clear(); swork.clear(); flops = 0.0; }
   int add_out(double* C, int ldc, int M, int N, int beta) {
     GemmOut o{C, ldc, M, N, (int)terms.size(), (int)terms.size(), beta, 0};
     outs.push_back(o);
@@ -154,15 +183,17 @@ struct AxpyPlan {
 };
 constexpr int kAxpyChunk = 1024;   // output elements per work chunk of the block axpy
 
-// tile of the split kernel: outputs, and K columns per step
+// side of an output tile of the split kernel, and K columns per step
 // largest side of an FMA tile (shared memory: 3 steps of 32 columns of both sides, at most 51 KB)
 constexpr int kFmaSide = 32;
-constexpr int kSplitTileM = 32, kSplitTileN = 64, kSplitChunk = 32;
+constexpr int kSplitTile = 64, kSplitChunk = 32;
 
 // ---------------------------------------------------------------- kernels (kernels.cu)
 // launches made, or -1 when the split kernel's shared memory was refused
-int launch_gemm_f64(const GemmPlan& p, cudaStream_t s);
-int launch_gemm_f64_split(const GemmPlan& p, cudaStream_t s);
+// (num_sms: multiprocessors; err[0]: the flag raised when a bounded wait runs
+// out, err[1]: scratch, may be shared by launches of one stream)
+int launch_gemm_f64(const GemmPlan& p, int num_sms, int* err, cudaStream_t s);
+int launch_gemm_f64_split(const GemmPlan& p, int num_sms, int* err, cudaStream_t s);
 void launch_axpy(const AxpyPlan& p, cudaStream_t s);
 // dst[i * dstep] = coef * src[i * sstep], i < len, for every task
 struct GatherTask { const double* src; double* dst; int32_t len, sstep, dstep, pad; double coef; };

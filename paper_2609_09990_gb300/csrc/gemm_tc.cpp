@@ -174,11 +174,7 @@ void Engine::run_tc(GemmPlan& p, int prec) {
   float* part = slot ? dalloc<float>((size_t)slot) : nullptr;
   TcRed* dr = red.empty() ? nullptr : dalloc<TcRed>(red.size());
   if (dr) h2d(dr, red.data(), red.size() * sizeof(TcRed));
-  if (!d_env_err) {
-    d_env_err = dalloc<int>(1);
-    CK(cudaMemsetAsync(d_env_err, 0, sizeof(int), stream));
-  }
-  TcLaunch L{dt, dm, (int)tiles.size(), prec, nullptr, nullptr, base, d_env_err, part, nullptr, nullptr, ncap,
+  TcLaunch L{dt, dm, (int)tiles.size(), prec, nullptr, nullptr, base, wait_flag(), part, nullptr, nullptr, ncap,
              tc_stages(prec, ncap)};
   if (!launch_tc_gemm(maps, L, num_sms, stream)) throw Error(-3, "invalid tensor-core launch configuration");
   stats.launches++;
@@ -187,7 +183,7 @@ void Engine::run_tc(GemmPlan& p, int prec) {
     stats.launches++;
   }
   CK(cudaGetLastError());
-  env_tc_pending = true;   // the bounded-wait flag is read after the next synchronisation
+  wait_pending = true;   // the bounded-wait flag is read after the next synchronisation
   for (int h = 0; h < nh; ++h) {
     dfree(pa[h]);
     dfree(pb[h]);

@@ -411,8 +411,8 @@ int reduction_blocks(int64_t n) {
   return (int)(b < 1 ? 1 : b);
 }
 
-int launch_gemm_f64(const GemmPlan& p, cudaStream_t s) {
-  const int ns = launch_gemm_f64_split(p, s);
+int launch_gemm_f64(const GemmPlan& p, int num_sms, int* err, cudaStream_t s) {
+  const int ns = launch_gemm_f64_split(p, num_sms, err, s);
   if (ns < 0) return ns;
   const int nt = (int)p.tiles.size();
   const int smem = FR * FK * p.tile_span * (int)sizeof(double);

@@ -7,9 +7,9 @@
 // largest element below 2^55) and rounded once to an integer of 56 bits,
 // which is cut into seven signed base-256 digits -128..128 (FP16 holds them
 // exactly).  The digit products of equal weight are summed by the tensor
-// cores in FP32.  A sum over a chunk is an integer below 2^22 (at most 7 pairs x 32 x
-// 2^14), and its accumulator starts at 1.5 x 2^23, so that every step is
-// exact and the accumulator's bits are the integer.  The eight weights
+// cores in FP32.  A sum over a chunk is an integer below 2^22 (at most 7
+// pairs x 32 x 2^14), and its accumulator starts at 1.5 x 2^23, so that every
+// step is exact and the accumulator's bits are the integer.  The eight weights
 // (34 digit pairs; pairs of weight 8 and more are below the rounding of the
 // operands) are put together as one 64-bit integer, converted once and
 // added to the FP64 sum of the output with one FMA.
@@ -25,16 +25,23 @@
 // their chunk through plain FMAs instead, so infinities, NaN and extreme
 // scales give what the FMA loop gives.
 //
-// What bounds it: the three units that a chunk needs are about balanced --
-// mma.sync 34 x 32 x 8 clocks over four sub-cores, two FP64 operations per
-// output element, and the digit extraction (about 36 integer instructions
-// per operand element) -- and none is full: with three CTAs an SM their
-// latencies show (1.6 instructions a clock, tensor pipe 25 %, FP64 pipe 24 %
-// in stage A of the CAS(16,16) M=512 H_eff product).  The 32 x 64 tile keeps
-// the extraction at 3/64 of an element per product while sector blocks of a
-// few tens waste little of it; K chunks of 32 are what the exact FP32 sums
-// allow.  That H_eff product (39 GFLOP): 79 ms with FP64 FMAs, 21 ms here,
-// 1.9 TFLOP/s against the FP64 pipe's 1.2.
+// Two kernels.  split_operands cuts every operand block of a plan once (a
+// block of the sigma build serves up to hundreds of products) into records
+// that the second one copies as they are: per 32-column chunk and 64 rows, the
+// seven digit planes, swizzled for ldmatrix, and the rows' exponents, all
+// contiguous.  gemm_f64_split multiplies 64 x 64 output tiles: one thread
+// streams the records of all chunks of all terms of all tiles of its CTA
+// through a ring of three stages by bulk copies, twelve warps multiply.  Long
+// chains are cut into pieces with partial sums, added in a fixed order.
+// What bounds it: per 64 x 64 x 32 chunk 4350 clocks of mma.sync (34 pairs)
+// and 4096 clocks of the FP64 pipe (conversion and FMA of every output
+// element), which overlap between the three warps of a sub-core; both pipes
+// are 41 to 47 % busy in the H_eff product of CAS(16,16) M=512 (39 GFLOP):
+// 79 ms with FP64 FMAs, 21 ms with a first kernel that split its operands
+// itself, tile by tile, 9.9 ms here (operands 0.8, products 5.2 + 2.9),
+// 4.0 TFLOP/s against the FP64 pipe's 1.2.  Eight warps that kept all A digits
+// in registers: 7.8 + 3.6 ms for the products, with the work dealt out in
+// turn instead of by a counter.
 #include <cuda_runtime.h>
 
 #include <cuda_fp16.h>
@@ -45,30 +52,63 @@ namespace gbd {
 
 namespace {
 
-constexpr int XM = kSplitTileM, XN = kSplitTileN, XK = kSplitChunk, XT = 128;
-constexpr int NS = 7;                      // digits
-constexpr int PK = 40;                     // raw pitch, K contiguous (doubles): 320 B, conflict-free 16 B reads
-constexpr int PA = XM + 2, PB = XN + 2;    // raw pitch, K strided: rows of 272 / 528 B
-constexpr int kRawA = XM * PK, kRawB = XN * PK;                  // doubles (both layouts fit)
-static_assert(XK * PA <= kRawA && XK * PB <= kRawB, "raw tiles");
-constexpr int kSlA = XM * 64, kSlB = XN * 64;                    // bytes of one digit plane (32 halves a row)
-constexpr int kOffB = kRawA * 8, kOffSa = kOffB + kRawB * 8, kOffSb = kOffSa + NS * kSlA;
-constexpr int kOffE = kOffSb + NS * kSlB;
-constexpr int kSmem = kOffE + (XM + XN + 2) * 4;
-constexpr float kMagic = 12582912.0f;      // 1.5 x 2^23: integers in +-2^22 added to it are its low mantissa bits
+constexpr int XM = kSplitTile, XK = kSplitChunk;
+constexpr int NS = 7;                           // digits
+constexpr int kWarps = 12, XT = 32 * kWarps + 32;   // 13 warps: at most 4 on a sub-core, 128 registers
+constexpr int kStages = 3;
+constexpr int kRec = XM * (NS * 64 + 4);        // bytes of a full record: 64 rows x (7 x 32 halves + exponent)
+constexpr int kHead = 64;                       // bytes of a stage's header
+constexpr int kSmem = kStages * (2 * kRec + kHead) + 2 * kStages * 8 + 16;
+constexpr float kMagic = 12582912.0f;           // 1.5 x 2^23: integers in +-2^22 added to it are its low mantissa bits
 constexpr uint32_t kMagicBits = 0x4B400000u;
+constexpr int kBadExp = 1 << 28;                // exponent of a row that the digits cannot hold
+constexpr uint32_t kWaitLimit = 1u << 22;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
-// 8-byte asynchronous copy; zero fill when !in
-__device__ __forceinline__ void copy8(uint32_t dst, const double* src, bool in) {
-  const int n = in ? 8 : 0;
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t* b, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(b)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(b)) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_addr(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// bounded wait; false (and *err raised) when the limit runs out or another role already failed
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err) {
+  for (uint32_t it = 0; it < kWaitLimit; ++it) {
+    if (mbar_try(b, parity)) return true;
+    if ((it & 1023u) == 1023u && *(volatile int*)err) return false;
+  }
+  atomicExch(err, 1);
+  return false;
+}
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(dst)),
+               "l"(src), "r"(bytes), "r"(smem_addr(bar))
+               : "memory");
 }
 __device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void ldsm2(uint32_t addr, uint32_t (&r)[2]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r[0]), "=r"(r[1])
                : "r"(addr)
                : "memory");
 }
@@ -78,315 +118,353 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], u
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// 16-byte chunk c (0..3) of a digit row: rows two apart use different halves
-// of a 128-byte line for the 8-byte digit stores, and the eight rows of an
-// ldmatrix use eight different 16-byte bank groups
-__device__ __forceinline__ int swz(int row, int c) { return c ^ (((row >> 1) & 1) << 1 | ((row >> 2) & 1)); }
-
-// element (row, k) of a raw operand tile: K contiguous or K strided
-template <int P>
-__device__ __forceinline__ double raw_at(const double* raw, bool kcontig, int row, int k) {
-  return kcontig ? raw[row * PK + k] : raw[k * P + row];
+// Byte offset of 16-byte piece c of a digit row: rows of 64 bytes (32 columns,
+// c 0..3) or 32 bytes (chunks of at most 16 columns, c 0..1).  The eight rows
+// of an ldmatrix use eight different 16-byte bank groups.
+__device__ __forceinline__ int piece(int row, int c, int nh) {
+  return nh == 2 ? row * 64 + (c ^ (((row >> 1) & 1) << 1 | ((row >> 2) & 1))) * 16
+                 : row * 32 + (c ^ ((row >> 2) & 1)) * 16;
 }
+__device__ __forceinline__ int pad8(int rows) { return (rows + 7) & ~7; }
 
-// Digit planes of one operand row, by four threads (kq = 0..3) with elements
-// k = 16 h + 8 j + 2 kq + u of it each (h < nh, the 16-blocks in use).  The
-// digits of element (h, j, u) go to position 16 h + 4 kq + 2 j + u: the same
-// permutation of K for both operands.  Returns the row's scale exponent E
-// (all |x| < 2^(E - 1023); 1023 for a zero row); bad = 1 when E is not usable.
-template <int P>
-__device__ __forceinline__ int split_row(const double* raw, bool kcontig, int row, int kq, int nh, uint8_t* planes,
-                                         int plane, int& bad) {
-  uint32_t lo[8], hi[8];
+// ---------------------------------------------------------------- operand records
+// One warp per 8 rows of one chunk: four threads (kq = 0..3) per row, each
+// with the elements k = 16 h + 8 j + 2 kq + u; the digits of element (h, j, u)
+// go to position 16 h + 4 kq + 2 j + u, the same permutation of K for every
+// operand.  Bound by its integer work (about 36 instructions an element) and
+// by HBM (8 bytes read, 14 written).
+__global__ void __launch_bounds__(256) split_operands_kernel(const SplitOperand* __restrict__ ops, int nops,
+                                                             int64_t nitems, uint8_t* __restrict__ digits,
+                                                             int* __restrict__ next) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0;   // the product kernel's work counter
+  const int lane = threadIdx.x & 31, kq = lane & 3;
+  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  int64_t it = nitems * w / nw;
+  const int64_t end = nitems * (w + 1) / nw;
+  if (it >= end) return;
+  int lo_o = 0, hi_o = nops - 1;
+  while (lo_o < hi_o) {
+    const int mid = (lo_o + hi_o + 1) >> 1;
+    if (ops[mid].first <= it) lo_o = mid; else hi_o = mid - 1;
+  }
+  SplitOperand O = ops[lo_o];
+  for (; it < end; ++it) {
+    const int rp = pad8(O.rows), groups = rp >> 3, chunks = (O.K + XK - 1) / XK;
+    if (it - O.first >= (int64_t)groups * chunks) {   // items of an operand are never empty
+      O = ops[++lo_o];
+      --it;
+      continue;
+    }
+    const int loc = (int)(it - O.first), chunk = loc / groups, row = (loc - chunk * groups) * 8 + (lane >> 2);
+    const int k0 = chunk * XK, kc = min(XK, O.K - k0), nh = (kc + 15) >> 4;
+    uint32_t lo[8], hi[8];
 #pragma unroll
-  for (int h = 0; h < 2; ++h)
+    for (int i = 0; i < 8; ++i) {
+      const int k = 16 * (i >> 2) + 8 * ((i >> 1) & 1) + 2 * kq + (i & 1);
+      double v = 0.0;
+      if (row < O.rows && k < kc)
+        v = O.kstrided ? O.src[(int64_t)(k0 + k) * O.ld + row] : O.src[(int64_t)row * O.ld + k0 + k];
+      lo[i] = (uint32_t)__double2loint(v);
+      hi[i] = (uint32_t)__double2hiint(v);
+    }
+    uint32_t mx = 0, any = 0;
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      double2 v = make_double2(0.0, 0.0);
-      const int k = 16 * h + 8 * j + 2 * kq;
-      if (h < nh) {
-        if (kcontig) {
-          v = *reinterpret_cast<const double2*>(raw + row * PK + k);
-        } else {
-          v.x = raw[k * P + row];
-          v.y = raw[(k + 1) * P + row];
+    for (int i = 0; i < 8; ++i) {
+      mx = max(mx, hi[i] & 0x7FFFFFFFu);
+      any |= lo[i];
+    }
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    any |= __shfl_xor_sync(0xffffffffu, any, 1);
+    any |= __shfl_xor_sync(0xffffffffu, any, 2);
+    const bool zero = mx == 0;
+    int E = zero ? 1023 : (int)(mx >> 20) + 1;   // all |x| < 2^(E - 1023)
+    if (mx < (700u << 20) ? (mx != 0 || any != 0) : mx >= (1300u << 20)) E = kBadExp;
+    const int sh0 = zero ? 5000 : (int)(mx >> 20) + 8;   // right shift of the left-aligned mantissa: sh0 - exponent
+    const uint64_t bias = 2 * 0x0080808080808080ull + 1;
+    const int tile = row / XM, trow = row - tile * XM, rt = min(XM, rp - tile * XM);
+    const int plane = rt * nh * 32;
+    // chunks before this one are full: rp rows of 7 x 64 + 4 bytes
+    uint8_t* rec = digits + O.off + (int64_t)chunk * rp * (NS * 64 + 4) + (int64_t)tile * XM * (NS * nh * 32 + 4);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (h >= nh) break;
+      uint32_t pk[2][NS];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        uint32_t wl[2], wh[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const uint32_t xh = hi[4 * h + 2 * j + u], xl = lo[4 * h + 2 * j + u];
+          const uint32_t mh = __funnelshift_l(xl, xh, 11) | 0x80000000u;
+          const uint64_t m = ((uint64_t)mh << 32) | (uint32_t)(xl << 11);
+          const uint32_t s = (uint32_t)(sh0 - (int)((xh >> 20) & 0x7FFu));
+          uint64_t t;   // 2 |x| in units of the last digit; 0 for shifts of 64 and more
+          asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(m), "r"(s));
+          const int64_t sg = (int64_t)((int32_t)xh >> 31);
+          const uint64_t q = (uint64_t)((int64_t)((t ^ (uint64_t)sg) - (uint64_t)sg + bias)) >> 1;
+          wl[u] = (uint32_t)q;
+          wh[u] = (uint32_t)(q >> 32);
+        }
+        // half2 of digit i of the two elements: byte + 1024 as FP16, less 1152
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+          uint32_t b;
+          if (i == 0) {
+            b = __byte_perm(wh[0], wh[1], 0x7632) | 0x64006400u;
+          } else {
+            const int byte = NS - 1 - i;
+            const uint32_t x0 = byte < 4 ? wl[0] : wh[0], x1 = byte < 4 ? wl[1] : wh[1];
+            const uint32_t c = byte & 3;
+            b = (__byte_perm(x0, x1, c | (c << 4) | ((c + 4) << 8) | ((c + 4) << 12)) & 0x00FF00FFu) | 0x64006400u;
+          }
+          const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&b), __half2half2(__ushort_as_half(0x6480)));
+          pk[j][i] = *reinterpret_cast<const uint32_t*>(&d);
         }
       }
-      const int i = 4 * h + 2 * j;
-      lo[i] = (uint32_t)__double2loint(v.x);
-      hi[i] = (uint32_t)__double2hiint(v.x);
-      lo[i + 1] = (uint32_t)__double2loint(v.y);
-      hi[i + 1] = (uint32_t)__double2hiint(v.y);
+      uint8_t* dst = rec + piece(trow, 2 * h + (kq >> 1), nh) + (kq & 1) * 8;
+#pragma unroll
+      for (int i = 0; i < NS; ++i) *reinterpret_cast<uint2*>(dst + i * plane) = make_uint2(pk[0][i], pk[1][i]);
     }
-  uint32_t mx = 0, any = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    mx = max(mx, hi[i] & 0x7FFFFFFFu);
-    any |= lo[i];
+    if (kq == 0) *reinterpret_cast<int*>(rec + NS * plane + trow * 4) = E;
   }
-  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-  int E = (int)(mx >> 20) + 1;
-  const bool zero = mx == 0;
-  bad = 0;
-  if (mx < (700u << 20)) bad = (mx != 0 || any != 0);
-  if (mx >= (1300u << 20)) bad = 1;
-  const int sh0 = zero ? 5000 : E + 7;   // right shift of the left-aligned mantissa: sh0 - exponent
-  const uint64_t bias = 2 * 0x0080808080808080ull + 1;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    if (h >= nh) break;
-    uint32_t pk[2][NS];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      uint32_t wl[2], wh[2];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const uint32_t xh = hi[4 * h + 2 * j + u], xl = lo[4 * h + 2 * j + u];
-        const uint32_t mh = __funnelshift_l(xl, xh, 11) | 0x80000000u;
-        const uint64_t m = ((uint64_t)mh << 32) | (uint32_t)(xl << 11);
-        const uint32_t s = (uint32_t)(sh0 - (int)((xh >> 20) & 0x7FFu));
-        uint64_t t;   // 2 |x| in units of the last digit; 0 for shifts of 64 and more
-        asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(m), "r"(s));
-        const int64_t sg = (int64_t)((int32_t)xh >> 31);
-        const uint64_t w = (uint64_t)((int64_t)((t ^ (uint64_t)sg) - (uint64_t)sg + bias)) >> 1;
-        wl[u] = (uint32_t)w;
-        wh[u] = (uint32_t)(w >> 32);
-      }
-      // half2 of digit i of the two elements: byte + 1024 as FP16, less 1152
-#pragma unroll
-      for (int i = 0; i < NS; ++i) {
-        uint32_t b;
-        if (i == 0) {
-          b = __byte_perm(wh[0], wh[1], 0x7632) | 0x64006400u;
-        } else {
-          const int byte = NS - 1 - i;
-          const uint32_t x0 = byte < 4 ? wl[0] : wh[0], x1 = byte < 4 ? wl[1] : wh[1];
-          const uint32_t c = byte & 3;
-          b = (__byte_perm(x0, x1, c | (c << 4) | ((c + 4) << 8) | ((c + 4) << 12)) & 0x00FF00FFu) | 0x64006400u;
-        }
-        const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&b), __half2half2(__ushort_as_half(0x6480)));
-        pk[j][i] = *reinterpret_cast<const uint32_t*>(&d);
-      }
-    }
-    uint8_t* dst = planes + row * 64 + swz(row, 2 * h + (kq >> 1)) * 16 + (kq & 1) * 8;
-#pragma unroll
-    for (int i = 0; i < NS; ++i) *reinterpret_cast<uint2*>(dst + i * plane) = make_uint2(pk[0][i], pk[1][i]);
-  }
-  return zero ? 1023 : E;
 }
 
-__global__ void __launch_bounds__(XT, 3)
+// ---------------------------------------------------------------- products
+struct Head {          // what the consumers need of one chunk, 64 bytes
+  double* C;           // output tile (or partial slot), written after the last chunk
+  double alpha;
+  int32_t ldc, mr, nr, flags;   // kFirst | kLast | kBeta | kEnd
+  int32_t nh, kc, term, k0;     // 16-column halves; columns, GemmTerm and first column of the chunk
+  int32_t m0, n0, pad0, pad1;
+};
+static_assert(sizeof(Head) == kHead, "stage header");
+enum { kFirst = 1, kLast = 2, kBeta = 4, kEnd = 8 };
+
+__global__ void __launch_bounds__(XT, 1)
 gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
-                      const GemmTile* __restrict__ tiles, int ntiles) {
+                      const SplitTerm* __restrict__ sterms, const SplitWork* __restrict__ work, int nwork,
+                      const uint8_t* __restrict__ digits, double* __restrict__ part, int* err, int* next) {
   extern __shared__ __align__(128) uint8_t sm[];
-  double* rawA = reinterpret_cast<double*>(sm);
-  double* rawB = reinterpret_cast<double*>(sm + kOffB);
-  uint8_t* slA = sm + kOffSa;
-  uint8_t* slB = sm + kOffSb;
-  int* expA = reinterpret_cast<int*>(sm + kOffE);
-  int* expB = expA + XM;
-  int* flag = expB + XN;   // [2]: a chunk needs plain FMAs
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wm = warp & 1, wn = warp >> 1;
-  const uint32_t rawA_a = smem_addr(rawA), rawB_a = smem_addr(rawB);
-  if (tid < 2) flag[tid] = 0;
-  int par = 0;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const GemmTile tl = tiles[tile];
-    const GemmOut o = outs[tl.out];
-    const int m0 = tl.tm * XM, n0 = tl.tn * XN;
-    const int mr = min(XM, o.M - m0), nr = min(XN, o.N - n0);
-    double acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-
-    // raw tiles of chunk k0 of term T: kc columns, zeros up to a multiple of 16
-    auto fetch = [&](const GemmTerm& T, int k0) {
-      const int kc = min(XK, T.K - k0), kz = (kc + 15) & ~15;
-      if (!(T.flags & 1)) {
-        const double* s = T.A + (int64_t)m0 * T.lda + k0;
-        if (lane < kz)
-          for (int r = warp; r < mr; r += 4)
-            copy8(rawA_a + (r * PK + lane) * 8, s + (int64_t)r * T.lda + (lane < kc ? lane : 0), lane < kc);
-      } else {
-        const double* s = T.A + (int64_t)k0 * T.lda + m0;
-        if (lane < mr)
-          for (int k = warp; k < kz; k += 4)
-            copy8(rawA_a + (k * PA + lane) * 8, s + (int64_t)(k < kc ? k : 0) * T.lda + lane, k < kc);
-      }
-      if (T.flags & 2) {
-        const double* s = T.B + (int64_t)n0 * T.ldb + k0;
-        if (lane < kz)
-          for (int r = warp; r < nr; r += 4)
-            copy8(rawB_a + (r * PK + lane) * 8, s + (int64_t)r * T.ldb + (lane < kc ? lane : 0), lane < kc);
-      } else {
-        const double* s = T.B + (int64_t)k0 * T.ldb + n0;
-        for (int k = warp; k < kz; k += 4)
-          for (int n = lane; n < nr; n += 32)
-            copy8(rawB_a + (k * PB + n) * 8, s + (int64_t)(k < kc ? k : 0) * T.ldb + n, k < kc);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-
-    // the chunk in work is (T, k0); (Tn) is the next term with columns
-    int t = o.t0, k0 = 0;
-    GemmTerm T{}, Tn{};
-    auto skip_empty = [&](int& i, GemmTerm& X) {
-      while (i < o.t1) {
-        X = terms[i];
-        if (X.K > 0) break;
-        ++i;
-      }
-    };
-    skip_empty(t, T);
-    int tn = t + 1;
-    if (t < o.t1) {
-      skip_empty(tn, Tn);
-      fetch(T, 0);
+  // stage s: record of A, record of B; the headers and barriers behind them
+  Head* heads = reinterpret_cast<Head*>(sm + kStages * 2 * kRec);
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + kStages * (2 * kRec + kHead));
+  uint64_t* empty = full + kStages;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], kWarps);
     }
-    while (t < o.t1) {
-      const int kc = min(XK, T.K - k0), nh = (kc + 15) >> 4;
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncthreads();   // raw tiles landed; every warp is done with the digit planes
-      const bool ka = !(T.flags & 1), kb = T.flags & 2;
-      const int ahi = __double2hiint(T.alpha);
-      const int aexp = (ahi >> 20) & 0x7FF;
-      const bool abad = aexp < 950 || aexp > 1100;
-      {
-        const int row = tid >> 2, kq = tid & 3;
-        int bad;
-        if ((row & ~7) < mr) {   // whole warps
-          const int E = split_row<PA>(rawA, ka, row, kq, nh, slA, kSlA, bad);
-          if (row < mr) {
-            if (kq == 0) expA[row] = E;
-            if (bad || abad) flag[par] = 1;
-          }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  if (warp == kWarps) {
+    if (lane != 0) return;
+    // ---------------- producer
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    // the first piece of work by block, the others as they are free: pieces
+    // differ by an order of magnitude in length (dealt out in turn, the
+    // busiest SM of a CAS(16,16) stage A worked 1.3 times as long as the mean)
+    int wnext = 0;
+    for (int w = blockIdx.x; w < nwork && ok; w = wnext) {
+      wnext = (int)gridDim.x + atomicAdd(next, 1);   // needed after this piece
+      const SplitWork W = work[w];
+      const GemmOut o = outs[W.out];
+      Head h;
+      h.m0 = W.tm * XM;
+      h.n0 = W.tn * XM;
+      h.mr = min(XM, o.M - h.m0);
+      h.nr = min(XM, o.N - h.n0);
+      h.C = W.slot >= 0 ? part + (int64_t)W.slot * XM * XM : o.C + (int64_t)h.m0 * o.ldc + h.n0;
+      h.ldc = W.slot >= 0 ? XM : o.ldc;
+      const int beta = W.slot < 0 && o.beta ? kBeta : 0;
+      const int ra = pad8(h.mr), rb = pad8(h.nr);
+      int t = W.t0, k0 = W.k0;
+      SplitTerm T = sterms[t];
+      for (int i = 0; i < W.steps; ++i) {
+        while (k0 >= T.K) {   // also past terms without columns
+          T = sterms[++t];
+          k0 = 0;
         }
-#pragma unroll 1
-        for (int p = 0; p < XN; p += 32) {
-          if (((p + row) & ~7) >= nr) break;
-          const int E = split_row<PB>(rawB, kb, p + row, kq, nh, slB, kSlB, bad);
-          if (p + row < nr) {
-            if (kq == 0) expB[p + row] = E;
-            if (bad) flag[par] = 1;
-          }
-        }
+        h.kc = min(XK, T.K - k0);
+        h.nh = (h.kc + 15) >> 4;
+        h.flags = (i == 0 ? kFirst : 0) | (i == W.steps - 1 ? kLast | beta : 0);
+        h.term = T.term;
+        h.alpha = T.alpha;
+        h.k0 = k0;
+        const int row_bytes = NS * h.nh * 32 + 4, chunk = k0 / XK;
+        if (!mbar_wait(&empty[s], ph ^ 1, err)) { ok = false; break; }
+        heads[s] = h;
+        uint8_t* st = sm + s * 2 * kRec;
+        mbar_expect(&full[s], (uint32_t)((ra + rb) * row_bytes));
+        bulk_copy(st, digits + T.a + (int64_t)chunk * T.ra * (NS * 64 + 4) + (int64_t)h.m0 * row_bytes, ra * row_bytes,
+                  &full[s]);
+        bulk_copy(st + kRec, digits + T.b + (int64_t)chunk * T.rb * (NS * 64 + 4) + (int64_t)h.n0 * row_bytes,
+                  rb * row_bytes, &full[s]);
+        if (++s == kStages) { s = 0; ph ^= 1; }
+        k0 += XK;
       }
-      __syncthreads();
-      const bool plain = flag[par] != 0;
-      if (plain) {
-        // the chunk by FP64 FMAs from the raw tiles
+    }
+    if (ok && mbar_wait(&empty[s], ph ^ 1, err)) {
+      heads[s].flags = kEnd;
+      mbar_arrive(&full[s]);
+    } else {
+      // stages armed but never consumed: let their copies land before the CTA exits
+      for (int i = 0; i < kStages; ++i)
+        for (uint32_t it = 0; it < (1u << 20) && !mbar_try(&full[i], i < s ? ph : ph ^ 1); ++it) {
+        }
+    }
+    return;
+  }
+  // ---------------- consumers
+  constexpr int kN8 = 3;   // 8-column groups of a warp: 8 of a tile over 12 / 4 warps
+  double acc[kN8][4];
+  int s = 0;
+  uint32_t ph = 0;
+  for (;;) {
+    if (!mbar_wait(&full[s], ph, err)) break;
+    const Head h = heads[s];
+    if (h.flags & kEnd) break;
+    const uint8_t* ra = sm + s * 2 * kRec;
+    const uint8_t* rb = ra + kRec;
+    const int nh = h.nh;
+    // warps: row groups of 16, and the 8-column groups dealt out among the
+    // warps of a row group, so that small tiles keep most warps at work
+    const int nm = (h.mr + 15) >> 4, per = kWarps / nm, g = warp % nm, nb = warp / nm;
+    const int n8 = (h.nr + 7) >> 3;
+    const bool on = nb < per && nb < n8;
+    if (h.flags & kFirst) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int c8 = (wn + 2 * i) * 8;
+      for (int i = 0; i < kN8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    }
+    if (on) {
+      const int pa = pad8(h.mr) * nh * 32, pb = pad8(h.nr) * nh * 32;   // plane bytes
+      const int* expA = reinterpret_cast<const int*>(ra + NS * pa);
+      const int* expB = reinterpret_cast<const int*>(rb + NS * pb);
+      const int r0 = 16 * g + (lane >> 2);
+      // rows and columns outside the tile hold whatever the stage held before: never stored
+      const bool ok0 = r0 < h.mr, ok1 = r0 + 8 < h.mr;
+      const int x0 = ok0 ? expA[r0] : 1023, x1 = ok1 ? expA[r0 + 8] : 1023;
+      const int ahi = __double2hiint(h.alpha), alo = __double2loint(h.alpha), aexp = (ahi >> 20) & 0x7FF;
+      const bool badA = x0 == kBadExp || x1 == kBadExp || aexp < 950 || aexp > 1100;
+      const int arow = 16 * g + (lane & 15);
+      const uint32_t ad0 = smem_addr(ra + piece(arow, lane >> 4, nh));
+      const uint32_t ad1 = smem_addr(ra + piece(arow, 2 + (lane >> 4), 2));   // second half, full chunks only
+#pragma unroll
+      for (int i = 0; i < kN8; ++i) {
+        const int c8 = (nb + i * per) * 8;
+        if (c8 >= h.nr) break;
+        const int c = c8 + 2 * (lane & 3);
+        const int y0 = c < h.nr ? expB[c] : 1023, y1 = c + 1 < h.nr ? expB[c + 1] : 1023;
+        if (__any_sync(0xffffffffu, badA || y0 == kBadExp || y1 == kBadExp)) {
+          // the chunk of these 16 x 8 outputs by FP64 FMAs from the operands themselves
+          const GemmTerm T = terms[h.term];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const int r = 16 * wm + (lane >> 2) + 8 * (j >> 1), c = c8 + 2 * (lane & 3) + (j & 1);
-            if (r < mr && c < nr)
-              for (int k = 0; k < kc; ++k)
-                acc[i][j] = fma(raw_at<PA>(rawA, ka, r, k) * T.alpha, raw_at<PB>(rawB, kb, c, k), acc[i][j]);
+            const int r = r0 + 8 * (j >> 1), cc = c + (j & 1);
+            if (r >= h.mr || cc >= h.nr) continue;
+            const int64_t m = h.m0 + r, n = h.n0 + cc;
+            for (int k = h.k0; k < h.k0 + h.kc; ++k) {
+              const double av = T.flags & 1 ? T.A[(int64_t)k * T.lda + m] : T.A[m * T.lda + k];
+              const double bv = T.flags & 2 ? T.B[n * T.ldb + k] : T.B[(int64_t)k * T.ldb + n];
+              acc[i][j] = fma(av * T.alpha, bv, acc[i][j]);
+            }
           }
+          continue;
         }
-        __syncthreads();
-      }
-      if (tid == 0) flag[par ^ 1] = 0;
-      par ^= 1;
-      // the next chunk's raw tiles arrive while this one multiplies
-      const int ahi_cur = ahi, alo_cur = __double2loint(T.alpha);
-      k0 += XK;
-      if (k0 < T.K) {
-        fetch(T, k0);
-      } else {
-        t = tn;
-        k0 = 0;
-        T = Tn;
-        if (t < o.t1) {
-          fetch(T, 0);
-          ++tn;
-          skip_empty(tn, Tn);
-        }
-      }
-      if (plain || 16 * wm >= mr) continue;
-      uint32_t a[2][NS][4];
-      {
-        const int row = 16 * wm + (lane & 15);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (h < nh) {
-            const uint32_t ad = smem_addr(slA + row * 64 + swz(row, 2 * h + (lane >> 4)) * 16);
-#pragma unroll
-            for (int i = 0; i < NS; ++i) ldsm4(ad + i * kSlA, a[h][i]);
-          }
-        }
-      }
-      const int r0 = 16 * wm + (lane >> 2);
-      const int e0 = expA[r0] - 2100, e1 = expA[r0 + 8] - 2100;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int c8 = (wn + 2 * i) * 8;
-        if (c8 >= nr) break;
-        float s[8][4];
+        float f[8][4];
 #pragma unroll
         for (int d = 0; d < 8; ++d)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) s[d][j] = kMagic;
-        const int row = c8 + (lane & 7);
-        const uint32_t bd = smem_addr(slB + row * 64 + swz(row, lane >> 3) * 16);
+          for (int j = 0; j < 4; ++j) f[d][j] = kMagic;
+        // one half of the columns at a time: 28 registers of A digits, read
+        // again for every 8 columns, leave room for three warps a sub-core
+        const int brow = c8 + (lane & 7);
+        for (int hh = 0; hh < nh; ++hh) {
+          uint32_t a[NS][4];
+          const uint32_t ad = hh ? ad1 : ad0;
 #pragma unroll
-        for (int jb = 0; jb < NS; ++jb) {
-          uint32_t b[4];
-          ldsm4(bd + jb * kSlB, b);
+          for (int x = 0; x < NS; ++x) ldsm4(ad + x * pa, a[x]);
+          const uint32_t bd = smem_addr(rb + piece(brow, 2 * hh + ((lane >> 3) & 1), nh));
 #pragma unroll
-          for (int ia = 0; ia < NS; ++ia)
-            if (ia + jb < 8) mma_f16(s[ia + jb], a[0][ia], b[0], b[1]);
-          if (nh > 1) {
+          for (int jb = 0; jb < NS; ++jb) {
+            uint32_t b[2];
+            ldsm2(bd + jb * pb, b);
 #pragma unroll
             for (int ia = 0; ia < NS; ++ia)
-              if (ia + jb < 8) mma_f16(s[ia + jb], a[1][ia], b[2], b[3]);
+              if (ia + jb < 8) mma_f16(f[ia + jb], a[ia], b[0], b[1]);
           }
         }
-        const int2 eb = *reinterpret_cast<const int2*>(expB + c8 + 2 * (lane & 3));
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          auto bits = [&](int d) { return (int)(__float_as_uint(s[d][j]) - kMagicBits); };
+          auto bits = [&](int d) { return (int)(__float_as_uint(f[d][j]) - kMagicBits); };
           // weights 2^40 .. 2^0, and the last two rounded to units
           const int q = bits(0) * 256 + bits(1);
           const int p = bits(2) * 256 + bits(3);
           const int l = bits(4) * 256 + bits(5) + ((bits(6) * 256 + bits(7) + 32768) >> 16);
           const int64_t v = ((int64_t)q << 32) + (int64_t)p * 65536 + l;
-          const int e = (j < 2 ? e0 : e1) + ((j & 1) ? eb.y : eb.x);
-          acc[i][j] = fma(__ll2double_rn(v), __hiloint2double(ahi_cur + (e << 20), alo_cur), acc[i][j]);
+          const int e = (j < 2 ? x0 : x1) + ((j & 1) ? y1 : y0) - 2100;
+          acc[i][j] = fma(__ll2double_rn(v), __hiloint2double(ahi + (int)((uint32_t)e << 20), alo), acc[i][j]);
         }
       }
     }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
+    if (++s == kStages) { s = 0; ph ^= 1; }
+    if ((h.flags & kLast) && on) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int c = (wn + 2 * i) * 8 + 2 * (lane & 3);
+      for (int i = 0; i < kN8; ++i) {
+        const int c = (nb + i * per) * 8 + 2 * (lane & 3);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int r = 16 * wm + (lane >> 2) + 8 * (j >> 1), cc = c + (j & 1);
-        if (r >= mr || cc >= nr) continue;
-        double* d = o.C + (int64_t)(m0 + r) * o.ldc + n0 + cc;
-        *d = o.beta ? (*d + acc[i][j]) : acc[i][j];
+        for (int j = 0; j < 4; ++j) {
+          const int r = 16 * g + (lane >> 2) + 8 * (j >> 1), cc = c + (j & 1);
+          if (r >= h.mr || cc >= h.nr) continue;
+          double* d = h.C + (int64_t)r * h.ldc + cc;
+          *d = h.flags & kBeta ? (*d + acc[i][j]) : acc[i][j];
+        }
       }
     }
   }
 }
 
+// tiles whose chain was cut: the pieces' partial sums in their order
+__global__ void __launch_bounds__(256)
+split_sum_kernel(const GemmOut* __restrict__ outs, const SplitSum* __restrict__ sums, const double* __restrict__ part) {
+  const SplitSum S = sums[blockIdx.x];
+  const GemmOut o = outs[S.out];
+  const int m0 = S.tm * XM, n0 = S.tn * XM, mr = min(XM, o.M - m0), nr = min(XM, o.N - n0);
+  for (int x = threadIdx.x; x < mr * XM; x += 256) {
+    const int r = x / XM, c = x - r * XM;
+    if (c >= nr) continue;
+    const double* p = part + (int64_t)S.slot * XM * XM + x;
+    double v = 0.0;
+    for (int i = 0; i < S.count; ++i) v += p[(int64_t)i * XM * XM];
+    double* d = o.C + (int64_t)(m0 + r) * o.ldc + n0 + c;
+    *d = o.beta ? *d + v : v;
+  }
+}
+
 }  // namespace
 
-int launch_gemm_f64_split(const GemmPlan& p, cudaStream_t s) {
-  const int n = (int)p.split.size();
+int launch_gemm_f64_split(const GemmPlan& p, int num_sms, int* err, cudaStream_t s) {
+  const int n = (int)p.swork.size();
   if (n == 0) return 0;
   static const cudaError_t attr =
       cudaFuncSetAttribute(gemm_f64_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (attr != cudaSuccess) return -1;
-  const int grid = n < 152 * 3 ? n : 152 * 3;
-  gemm_f64_split_kernel<<<grid, XT, kSmem, s>>>(p.d_terms, p.d_outs, p.d_split, n);
-  return 1;
+  const int64_t blocks = (p.split_items + 7) / 8;
+  split_operands_kernel<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, s>>>(
+      p.d_operands, (int)p.operands.size(), p.split_items, p.d_digits, err + 1);
+  gemm_f64_split_kernel<<<n < num_sms ? n : num_sms, XT, kSmem, s>>>(p.d_terms, p.d_outs, p.d_sterms, p.d_swork, n,
+                                                                     p.d_digits, p.d_part, err, err + 1);
+  if (!p.ssums.empty()) split_sum_kernel<<<(int)p.ssums.size(), 256, 0, s>>>(p.d_outs, p.d_ssums, p.d_part);
+  return 2 + !p.ssums.empty();
 }
 
 }  // namespace gbd
