@@ -376,8 +376,14 @@ void Engine::rdms_ci(double* rdm1, double* rdm2) {
 // from products of excitation operators,
 //   <E_pq E_rs E_tu> = Gamma3_pqrstu + d_qt Gamma_purs + d_st Gamma_pqru
 //                      + d_qr Gamma_pstu + d_qr d_st gamma_pu,
-// and <E_pq E_rs E_tu> = D[qp] . (E_rs D[tu]) with D[tu] = E_tu C: for each
-// rs, the n^2 vectors E_rs D[tu] and one split-K Gram GEMM against D.  FP64.
+// and <E_pq E_rs E_tu> = D[qp] . (E_rs D[tu]) with D[tu] = E_tu C.  Gamma3
+// does not change when its index pairs (pq), (rs), (tu) change places, so one
+// order of each triple is computed, tu <= rs <= pq as numbers: for each rs the
+// rs + 1 vectors E_rs D[tu] and a Gram GEMM against the n^2 - rs vectors D[qp],
+// a sixth of all products.  The GEMMs of as many rs as fit 1 GiB of vectors
+// are one launch, each split over K until the launch has a few tiles for
+// every SM (CAS(9,9) M=96: 88 ms with one launch of a dozen tiles per rs and
+// all triples, 4.1 ms).
 void Engine::rdm3(double* out) {
   int64_t NaS = 0, NbS = 0;
   double* C = expand_ci(NaS, NbS);
@@ -393,59 +399,93 @@ void Engine::rdm3(double* out) {
   CK(cudaMemcpyAsync(d_excA, excA.data(), excA.size() * sizeof(int), cudaMemcpyHostToDevice, stream));
   CK(cudaMemcpyAsync(d_excB, excB.data(), excB.size() * sizeof(int), cudaMemcpyHostToDevice, stream));
   double* D = dalloc<double>((size_t)n2 * ndet);
-  double* F = dalloc<double>((size_t)n2 * ndet);
   launch_apply_e_chunk(C, NbS, d_excA, d_excB, n2, 0, (int)NaS, D, stream);
   stats.launches++;
   CK(cudaGetLastError());
-  const int SPLIT = 32;
-  const int parts = (int)std::min<int64_t>(SPLIT, std::max<int64_t>(1, ndet / 4096));
-  const int64_t step = (ndet + parts - 1) / parts;
-  double* Mp = dalloc<double>((size_t)parts * n2 * n2);
-  double* M3 = dalloc<double>((size_t)n2 * n2 * n2);
+  double* Dt = dalloc<double>((size_t)n2 * ndet);   // Dt[pq] = D[qp]
+  for (int i = 0; i < n2; ++i)
+    CK(cudaMemcpyAsync(Dt + (size_t)i * ndet, D + (size_t)(i % n * n + i / n) * ndet, ndet * sizeof(double),
+                       cudaMemcpyDeviceToDevice, stream));
+  // batches of rs: [first, last), their vectors in F
+  std::vector<int> first{0};
+  int64_t fvec = 0, fmax = 0;
+  for (int rs = 0; rs < n2; ++rs) {
+    if (fvec > 0 && (fvec + rs + 1) * ndet > ((int64_t)1 << 27)) {
+      first.push_back(rs);
+      fvec = 0;
+    }
+    fvec += rs + 1;
+    fmax = std::max(fmax, fvec);
+  }
+  first.push_back(n2);
+  double* F = dalloc<double>((size_t)fmax * ndet);
+  std::vector<int64_t> off3(n2 + 1, 0);   // M3: (n2 - rs) x (rs + 1) per rs
+  for (int rs = 0; rs < n2; ++rs) off3[rs + 1] = off3[rs] + (int64_t)(n2 - rs) * (rs + 1);
+  double* M3 = dalloc<double>((size_t)off3[n2]);
   double* M2 = dalloc<double>((size_t)n2 * n2 + n2);
-  // Gram of D against a set of n2 vectors W (D . W^T), split over K and summed
-  // in a fixed order into dst
-  auto gram = [&](const double* W, int ldw_is_vec, double* dst, int ncols) {
+  // products of rows of X with rows of Y (or one vector Y), all of a list in
+  // one launch: K split into equal parts, summed in a fixed order
+  struct Gram { const double* X; const double* Y; double* dst; int rows, cols; bool vec; };
+  auto grams = [&](const std::vector<Gram>& list) {
+    int64_t tiles = 0, elems = 0;
+    for (const Gram& g : list) {
+      tiles += (int64_t)((g.rows + kSplitTile - 1) / kSplitTile) * ((g.cols + kSplitTile - 1) / kSplitTile);
+      elems += (int64_t)g.rows * g.cols;
+    }
+    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>((8 * num_sms + tiles - 1) / tiles, ndet / 1024));
+    const int64_t step = (ndet + parts - 1) / parts;
+    double* Mp = dalloc<double>((size_t)parts * elems);
     GemmPlan p;
     p.result = true;
-    for (int s = 0; s < parts; ++s) {
-      const int64_t k0 = (int64_t)s * step, k1 = std::min<int64_t>(ndet, k0 + step);
-      p.add_out(Mp + (size_t)s * n2 * ncols, ncols, n2, ncols, 0);
-      if (k1 > k0) p.add_term(D + k0, (int)ndet, W + k0, ldw_is_vec ? 1 : (int)ndet, (int)(k1 - k0),
-                              ldw_is_vec ? 0 : 2, 1.0);
+    AxpyPlan ax;
+    int64_t at = 0;
+    for (const Gram& g : list) {
+      const int64_t len = (int64_t)g.rows * g.cols;
+      ax.outs.push_back({g.dst, len, (int)ax.terms.size(), 0});
+      for (int s = 0; s < parts; ++s, at += len) {
+        const int64_t k0 = (int64_t)s * step, k1 = std::min<int64_t>(ndet, k0 + step);
+        p.add_out(Mp + at, g.cols, g.rows, g.cols, 0);
+        if (k1 > k0)
+          p.add_term(g.X + k0, (int)ndet, g.Y + k0, g.vec ? 1 : (int)ndet, (int)(k1 - k0), g.vec ? 0 : 2, 1.0);
+        ax.terms.push_back({Mp + at, 1.0});
+      }
+      ax.outs.back().t1 = (int)ax.terms.size();
     }
     upload(p);
     run(p);
     release(p);
-    AxpyPlan ax;
-    ax.outs.push_back({dst, (int64_t)n2 * ncols, 0, 0});
-    for (int s = 0; s < parts; ++s) ax.terms.push_back({Mp + (size_t)s * n2 * ncols, 1.0});
-    ax.outs.back().t1 = (int)ax.terms.size();
     upload(ax);
     run(ax);
     release(ax);
+    dfree(Mp);
   };
-  gram(D, 0, M2, n2);            // <E_qp C | E_rs C>
-  gram(C, 1, M2 + (size_t)n2 * n2, 1);   // <E_qp C | C>
-  for (int rs = 0; rs < n2; ++rs) {
-    launch_apply_e_vecs(D, n2, NaS, NbS, d_excA, d_excB, n2, rs, F, stream);
-    stats.launches++;
+  // <E_qp C | E_rs C> and <E_qp C | C>
+  grams({{D, D, M2, n2, n2, false}, {D, C, M2 + (size_t)n2 * n2, n2, 1, true}});
+  for (size_t u = 0; u + 1 < first.size(); ++u) {
+    std::vector<Gram> list;
+    double* f = F;
+    for (int rs = first[u]; rs < first[u + 1]; ++rs) {
+      launch_apply_e_vecs(D, rs + 1, NaS, NbS, d_excA, d_excB, n2, rs, f, stream);
+      stats.launches++;
+      list.push_back({Dt + (size_t)rs * ndet, f, M3 + off3[rs], n2 - rs, rs + 1, false});
+      f += (size_t)(rs + 1) * ndet;
+    }
     CK(cudaGetLastError());
-    gram(F, 0, M3 + (size_t)rs * n2 * n2, n2);
+    grams(list);
   }
   int nblk = reduction_blocks(ndet);
   double* partial = dalloc<double>(nblk);
   double* nrm_d = dalloc<double>(1);
   launch_multi_dot(C, ndet, 1, C, ndet, nrm_d, partial, nblk, stream);
   stats.launches += 2;
-  std::vector<double> h3((size_t)n2 * n2 * n2), h2((size_t)n2 * n2 + n2);
+  std::vector<double> h3((size_t)off3[n2]), h2((size_t)n2 * n2 + n2);
   double nrm2 = 0;
   CK(cudaMemcpyAsync(h3.data(), M3, h3.size() * sizeof(double), cudaMemcpyDeviceToHost, stream));
   CK(cudaMemcpyAsync(h2.data(), M2, h2.size() * sizeof(double), cudaMemcpyDeviceToHost, stream));
   CK(cudaMemcpyAsync(&nrm2, nrm_d, sizeof(double), cudaMemcpyDeviceToHost, stream));
   sync();
   stats.d2h += (h3.size() + h2.size() + 1) * sizeof(double);
-  for (void* q : {(void*)C, (void*)d_excA, (void*)d_excB, (void*)D, (void*)F, (void*)Mp, (void*)M3, (void*)M2,
+  for (void* q : {(void*)C, (void*)d_excA, (void*)d_excB, (void*)D, (void*)Dt, (void*)F, (void*)M3, (void*)M2,
                   (void*)partial, (void*)nrm_d})
     dfree(q);
   if (!(nrm2 > 0)) throw Error(-4, "MPS has zero norm in the determinant expansion");
@@ -462,19 +502,23 @@ void Engine::rdm3(double* out) {
           g2[(size_t)(p * n + q) * n2 + r * n + s2] = v;
         }
   auto G2 = [&](int p, int q, int r, int s2) { return g2[(size_t)(p * n + q) * n2 + r * n + s2]; };
-  for (int p = 0; p < n; ++p)
-    for (int q = 0; q < n; ++q)
-      for (int r = 0; r < n; ++r)
-        for (int s2 = 0; s2 < n; ++s2)
-          for (int t = 0; t < n; ++t)
-            for (int u = 0; u < n; ++u) {
-              double v = h3[((size_t)(r * n + s2) * n2 + q * n + p) * n2 + t * n + u] / nrm2;
-              if (q == t) v -= G2(p, u, r, s2);
-              if (s2 == t) v -= G2(p, q, r, u);
-              if (q == r) v -= G2(p, s2, t, u);
-              if (q == r && s2 == t) v -= g1[p * n + u];
-              out[((((size_t)(p * n + q) * n + r) * n + s2) * n + t) * n + u] = v;
-            }
+  auto put = [&](int x, int y, int z, double v) { out[((size_t)x * n2 + y) * n2 + z] = v; };
+  for (int rs = 0; rs < n2; ++rs)
+    for (int pq = rs; pq < n2; ++pq)
+      for (int tu = 0; tu <= rs; ++tu) {
+        const int p = pq / n, q = pq % n, r = rs / n, s2 = rs % n, t = tu / n, u = tu % n;
+        double v = h3[off3[rs] + (int64_t)(pq - rs) * (rs + 1) + tu] / nrm2;
+        if (q == t) v -= G2(p, u, r, s2);
+        if (s2 == t) v -= G2(p, q, r, u);
+        if (q == r) v -= G2(p, s2, t, u);
+        if (q == r && s2 == t) v -= g1[p * n + u];
+        put(pq, rs, tu, v);
+        put(pq, tu, rs, v);
+        put(rs, pq, tu, v);
+        put(rs, tu, pq, v);
+        put(tu, pq, rs, v);
+        put(tu, rs, pq, v);
+      }
 }
 
 // ---------------------------------------------------------------- orbital RDMs
