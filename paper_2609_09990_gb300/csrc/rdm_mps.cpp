@@ -646,17 +646,25 @@ void Engine::rdms(double* rdm1, double* rdm2) {
         const Mat4 m[2] = {lad[sg], lad[2 + sg]};
         S.add(pos, m, odd, 2, (int64_t)p * n + q);
       }
+  // Gamma_pqrs = Gamma_rspq (the pairs change places) = Gamma_qpsr (real state):
+  // one of the four is contracted, the others are copies
+  auto at = [&](int p, int q, int r, int s) { return (((int64_t)p * n + q) * n + r) * n + s; };
+  auto first = [&](int p, int q, int r, int s) {
+    return std::min(std::min(at(p, q, r, s), at(r, s, p, q)), std::min(at(q, p, s, r), at(s, r, q, p)));
+  };
   if (rdm2)
     for (int p = 0; p < n; ++p)
       for (int q = 0; q < n; ++q)
         for (int r = 0; r < n; ++r)
-          for (int s = 0; s < n; ++s)
+          for (int s = 0; s < n; ++s) {
+            if (first(p, q, r, s) != at(p, q, r, s)) continue;
             for (int sg = 0; sg < 2; ++sg)
               for (int tu = 0; tu < 2; ++tu) {
                 const int pos[4] = {p, r, s, q};
                 const Mat4 m[4] = {lad[sg], lad[tu], lad[2 + tu], lad[2 + sg]};
-                S.add(pos, m, odd, 4, n2 + (((int64_t)p * n + q) * n + r) * n + s);
+                S.add(pos, m, odd, 4, n2 + at(p, q, r, s));
               }
+          }
   const std::vector<double> v = eval_strings(S);
   std::vector<double> g1(n2, 0.0);
   if (rdm2) std::fill(rdm2, rdm2 + (size_t)n2 * n2, 0.0);
@@ -665,6 +673,11 @@ void Engine::rdms(double* rdm1, double* rdm2) {
     if (o < n2) g1[o] += v[i];
     else rdm2[o - n2] += v[i];
   }
+  if (rdm2)
+    for (int p = 0; p < n; ++p)
+      for (int q = 0; q < n; ++q)
+        for (int r = 0; r < n; ++r)
+          for (int s = 0; s < n; ++s) rdm2[at(p, q, r, s)] = rdm2[first(p, q, r, s)];
   if (rdm1) std::memcpy(rdm1, g1.data(), n2 * sizeof(double));
 }
 
