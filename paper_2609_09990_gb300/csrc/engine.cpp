@@ -316,6 +316,7 @@ Engine::Engine(int dev) : device(dev) {
   CK(cudaEventCreate(&evgm));
   CK(cudaMallocHost(&tc_err_host, sizeof(int)));
   *tc_err_host = 0;
+  CK(cudaMallocHost(&dav_host, (kDavMax + 2) * sizeof(double)));
   pin_cap = (size_t)16 << 20;
   CK(cudaMallocHost(&pin_ring, pin_cap));
   cudaMemPool_t pool;
@@ -327,6 +328,7 @@ Engine::Engine(int dev) : device(dev) {
 Engine::~Engine() {
   cudaSetDevice(device);
   if (tc_err_host) cudaFreeHost(tc_err_host);
+  if (dav_host) cudaFreeHost(dav_host);
   for (auto& e : Lenv) free_env(e);
   for (auto& e : Renv) free_env(e);
   for (auto& s : sites) free_site(s);
@@ -1588,13 +1590,19 @@ void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool re
 void Engine::sigma(Sigma& sg, const double* x, double* y) {
   settle();
   CK(cudaMemcpyAsync(sg.in, x, psi_size * sizeof(double), cudaMemcpyDeviceToDevice, stream));
+  sigma_run(sg);
+  CK(cudaMemcpyAsync(y, sg.out, psi_size * sizeof(double), cudaMemcpyDeviceToDevice, stream));
+}
+
+// sg.out = H_eff sg.in
+void Engine::sigma_run(Sigma& sg) {
+  settle();
   CK(cudaEventRecord(ev0, stream));
   replay(sg.graph, [&]() {
     run(sg.A);
     run(sg.B);
   });
   CK(cudaEventRecord(ev1, stream));
-  CK(cudaMemcpyAsync(y, sg.out, psi_size * sizeof(double), cudaMemcpyDeviceToDevice, stream));
   sigma_pending = 1;
   stats.sigma_flops += sg.A.flops + sg.B.flops;
   stats.n_sigma++;
@@ -1713,8 +1721,8 @@ void Engine::inner_pcg(const std::function<void(const double*, double*)>& op, co
 // the host, vectors on the device; preconditioner t = -r / (diag - theta)
 // with |diag - theta| clamped to 1e-8; two classical Gram-Schmidt passes;
 // restart from the 4 lowest Ritz vectors when the space is full.
-double Engine::davidson(const std::function<void(const double*, double*)>& op, const double* diag, double tol,
-                        int max_iter, int max_space, double stag_rel) {
+double Engine::davidson(const SigmaOp& op, const double* diag, double tol, int max_iter, int max_space,
+                        double stag_rel) {
   // Two host synchronisations per iteration: the residual norm (convergence
   // test) and the new row of the projected matrix.  Gram-Schmidt
   // coefficients and the normalisation never leave the device.
@@ -1757,7 +1765,7 @@ double Engine::davidson(const std::function<void(const double*, double*)>& op, c
   const int nphi = defl_phi ? (int)defl.size() : 0;
   double* dpen = nphi ? dalloc<double>(nphi) : nullptr;
   auto opp = [&](const double* a, double* b) {
-    op(a, b);
+    op.apply(a, b);
     if (nphi) {
       dots(defl_phi, nphi, a, dpen);
       launch_lincomb(b, defl_phi, n, dpen, nphi, n, 1, stream, defl_w);
@@ -1804,6 +1812,14 @@ double Engine::davidson(const std::function<void(const double*, double*)>& op, c
     double var = (sum_dd - 2.0 * th * sum_d) / (double)n + th * th;
     return MlpScalars{th, rn + 1e-300, std::sqrt(std::max(var, 0.0)) + 1e-300, (double)it};
   };
+  // Jacobi corrections of vectors up to kDavLongest: four kernels an iteration
+  // besides the sigma, which reads and writes its own buffers, and results
+  // in pinned memory instead of copies
+  const bool fused = pk == 0 && !recording && nphi == 0 && max_space <= kDavMax && n <= kDavLongest;
+  double* wpart = fused ? dalloc<double>((size_t)(max_space + 1) * 8 * nblk) : nullptr;
+  int* count = fused ? dalloc<int>(1) : nullptr;
+  double* dorth2 = fused ? dalloc<double>(max_space) : nullptr;
+  if (fused) CK(cudaMemsetAsync(count, 0, sizeof(int), stream));
   std::vector<double> w(max_space), Z((size_t)max_space * max_space), hk((size_t)max_space * max_space);
   for (int it = 0;; ++it) {
     for (int i = 0; i < k; ++i)
@@ -1812,13 +1828,24 @@ double Engine::davidson(const std::function<void(const double*, double*)>& op, c
     theta = w[0];
     std::vector<double> c(k);
     for (int i = 0; i < k; ++i) c[i] = Z[(size_t)i * k + 0];
-    h2d(coef, c.data(), k);
-    launch_lincomb(x, V, n, coef, k, n, 0, stream);
-    launch_lincomb(sx, S, n, coef, k, n, 0, stream);
-    launch_residual_precond(x, sx, diag, theta, n, r, t, partial, nblk, dres, stream);
-    stats.launches += 4;
     double rr;
-    d2h(&rr, dres, 1);
+    if (fused) {
+      DavCoef dc;
+      for (int i = 0; i < k; ++i) dc.c[i] = c[i];
+      stats.launches += launch_davidson_residual(V, S, diag, dc, theta, n, k, nblk, x, t, wpart, dorth,
+                                                 dav_host + kDavMax + 1, count, stream);
+      sync();
+      settle();
+      stats.d2h += sizeof(double);
+      rr = dav_host[kDavMax + 1];
+    } else {
+      h2d(coef, c.data(), k);
+      launch_lincomb(x, V, n, coef, k, n, 0, stream);
+      launch_lincomb(sx, S, n, coef, k, n, 0, stream);
+      launch_residual_precond(x, sx, diag, theta, n, r, t, partial, nblk, dres, stream);
+      stats.launches += 4;
+      d2h(&rr, dres, 1);
+    }
     double rn = std::sqrt(std::max(rr, 0.0));
     stats.last_residual = rn;
     if (rn < tol || it >= max_iter) break;
@@ -1868,6 +1895,29 @@ double Engine::davidson(const std::function<void(const double*, double*)>& op, c
       std::fill(Hs.begin(), Hs.end(), 0.0);
       for (int j = 0; j < kk; ++j) Hs[(size_t)j * max_space + j] = w[j];
       k = kk;
+      if (fused) dots(V, k, t, dorth);   // the overlaps with the new vectors
+    }
+    if (fused) {
+      // t <- t - V (V^T t), twice; v_k = t / |t|, into the sigma's input too; s_k = H v_k
+      stats.launches += launch_davidson_project(V, dorth, n, k, nblk, t, wpart, dorth2, nullptr, count, stream);
+      stats.launches += launch_davidson_project(V, dorth2, n, k, nblk, t, wpart, drow + max_space + 1,
+                                                dav_host + kDavMax, count, stream);
+      launch_normalize2(t, drow + max_space + 1, n, V + (size_t)k * n, *op.in, stream);
+      stats.launches++;
+      op.run();
+      stats.launches += launch_davidson_row(V, *op.out, n, k + 1, nblk, S + (size_t)k * n, wpart, drow, dav_host, count,
+                                            stream);
+      CK(cudaGetLastError());
+      sync();
+      settle();
+      stats.d2h += (k + 2) * sizeof(double);
+      if (!(dav_host[kDavMax] > 1e-28)) break;   // breakdown: t had no new direction
+      for (int i = 0; i <= k; ++i) {
+        Hs[(size_t)i * max_space + k] = dav_host[i];
+        Hs[(size_t)k * max_space + i] = dav_host[i];
+      }
+      ++k;
+      continue;
     }
     // t <- t - V (V^T t), twice; v_k = t / |t|; s_k = H v_k
     for (int pass = 0; pass < 2; ++pass) {
@@ -1908,6 +1958,7 @@ double Engine::davidson(const std::function<void(const double*, double*)>& op, c
     record_converged(psi);
   }
   if (dbad) dfree(dbad);
+  for (void* p : {(void*)wpart, (void*)count, (void*)dorth2}) dfree(p);
   for (void* p : {(void*)V, (void*)S, (void*)Vt, (void*)St, (void*)x, (void*)sx, (void*)r, (void*)t, (void*)partial,
                   (void*)dres, (void*)dorth, (void*)drow, (void*)coef})
     dfree(p);
@@ -2065,12 +2116,19 @@ void Engine::truncate(int k, int dir, int M, double* tau_out, std::vector<double
 // FP64 iterations.  Each tier restarts from the previous tier's Ritz vector.
 double Engine::solve_tiers(Sigma& sg, const double* diag, double tol, int precision, int refine, bool& planned) {
   double theta = 0;
-  auto fp64op = [&](const double* x, double* y) {
-    if (!planned) {
-      plan_sigma(sg.lenl, sg.renl, sg);
-      planned = true;
-    }
-    sigma(sg, x, y);
+  const SigmaOp fp64op{[&](const double* x, double* y) {
+                         if (!planned) {
+                           plan_sigma(sg.lenl, sg.renl, sg);
+                           planned = true;
+                         }
+                         sigma(sg, x, y);
+                       },
+                       [&]() { sigma_run(sg); }, &sg.in, &sg.out};
+  // the tensor-core sigma of a plan
+  auto tcop = [&](TcPlan* P) {
+    double **in, **out;
+    tc_buffers(P, in, out);
+    return SigmaOp{[this, P](const double* x, double* y) { tc_apply(P, x, y); }, [this, P]() { tc_run(P); }, in, out};
   };
   int64_t it0 = stats.davidson_iters;
   auto tier_done = [&](int t) {
@@ -2092,7 +2150,7 @@ double Engine::solve_tiers(Sigma& sg, const double* diag, double tol, int precis
     stats.last_residual = 1e300;
     if (!skip_tier1) {
       P = tc_plan(sg.lenl, sg.renl, p1);
-      theta = davidson([&](const double* x, double* y) { tc_apply(P, x, y); }, diag, std::max(tol, floor1),
+      theta = davidson(tcop(P), diag, std::max(tol, floor1),
                        sched.max_iter, sched.max_space, 10.0 * u1);
       tc_free(P);
       t1_iters_cur += stats.davidson_iters - it0;
@@ -2101,7 +2159,7 @@ double Engine::solve_tiers(Sigma& sg, const double* diag, double tol, int precis
     }
     if (stats.last_residual >= tol) {
       P = tc_plan(sg.lenl, sg.renl, tier2);
-      theta = davidson([&](const double* x, double* y) { tc_apply(P, x, y); }, diag, tol, sched.max_iter,
+      theta = davidson(tcop(P), diag, tol, sched.max_iter,
                        sched.max_space, tier2_floor_mult * u2);
       tc_free(P);
       tier_done(1);

@@ -437,9 +437,18 @@ class Engine {
   void plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool result = false);
   void sigma(Sigma& sg, const double* x, double* y);
   void compute_diag(const EnlOp& lenl, const EnlOp& renl, double* diag);
+  void sigma_run(Sigma& sg);
+  // the operator of a Davidson solve: b = H a, or `run` for *out = H *in on
+  // its own buffers (there after the first apply)
+  struct SigmaOp {
+    std::function<void(const double*, double*)> apply;
+    std::function<void()> run;
+    double* const* in;
+    double* const* out;
+  };
+  double* dav_host = nullptr;     // pinned: sums of a Davidson iteration
   // stag_rel > 0: stop on stagnation (reduced-precision operators); see the definition
-  double davidson(const std::function<void(const double*, double*)>& op, const double* diag, double tol,
-                  int max_iter, int max_space, double stag_rel);
+  double davidson(const SigmaOp& op, const double* diag, double tol, int max_iter, int max_space, double stag_rel);
   // the Davidson solve of one step in schedule precision `precision` with at
   // most `refine` FP64 iterations; the Ritz vector is left in psi
   double solve_tiers(Sigma& sg, const double* diag, double tol, int precision, int refine, bool& planned);
@@ -455,6 +464,8 @@ class Engine {
   TcPlan* tc_plan_impl(const EnlOp& lenl, const EnlOp& renl, int prec);
   std::map<int64_t, TcTune> tuned;
   void tc_apply(TcPlan* p, const double* x, double* y);
+  void tc_run(TcPlan* p);
+  static void tc_buffers(TcPlan* p, double**& in, double**& out);
   void tc_free(TcPlan* p);
   void truncate(int k, int dir, int M, double* tau, std::vector<double>* kept);
   // A fixed launch sequence on `stream`: run directly on its first use,

@@ -221,6 +221,25 @@ void launch_scale(double* x, double a, int64_t n, cudaStream_t s);
 // partial holds 2 * nblk doubles, sums_dev 2.
 void launch_projected_precond(const double* v, const double* x, const double* diag, double theta, double scale,
                               int64_t n, double* out, double* partial, int nblk, double* sums_dev, cudaStream_t s);
+// Vector work of one Davidson iteration with the Jacobi correction: the same
+// sums, rounded in the same order, as lincomb + residual_precond + multi_dot.
+// For n <= kDavLongest and k <= kDavMax; nblk = reduction_blocks(n); part
+// holds (k + 1) * 8 nblk doubles; count is an int that is 0 between launches;
+// host pointers are pinned memory, valid after the stream is synchronised.
+// Each returns its launches.
+constexpr int kDavMax = 32;
+constexpr int64_t kDavLongest = (int64_t)608 * 1024;   // four elements per lane and reduction block
+struct DavCoef { double c[kDavMax]; };
+int launch_davidson_residual(const double* V, const double* S, const double* diag, const DavCoef& c, double theta,
+                             int64_t n, int k, int nblk, double* x, double* t, double* part, double* overlaps,
+                             double* host_rr, int* count, cudaStream_t s);
+// t -= V d, then the overlaps V_j . t, or (host_norm given) t . t, to out
+int launch_davidson_project(const double* V, const double* d, int64_t n, int k, int nblk, double* t, double* part,
+                            double* out, double* host_norm, int* count, cudaStream_t s);
+// sk = y and the row V_j . sk, j < k
+int launch_davidson_row(const double* V, const double* y, int64_t n, int k, int nblk, double* sk, double* part,
+                        double* out, double* host, int* count, cudaStream_t s);
+void launch_normalize2(const double* t, const double* nrm2_dev, int64_t n, double* out, double* out2, cudaStream_t s);
 // y = a x + b y
 void launch_axpby(double* y, double a, const double* x, double b, int64_t n, cudaStream_t s);
 // d[i] += w sum_j phi[j * n + i]^2 (j < k)

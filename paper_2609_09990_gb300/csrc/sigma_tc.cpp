@@ -841,6 +841,23 @@ void Engine::tc_free(TcPlan* P) {
 // folded into its converted panel rows, so no term carries a sign) (x, y: FP64 two-site vectors)
 void Engine::tc_apply(TcPlan* P, const double* x, double* y) {
   settle();
+  if (!P->xin) {
+    P->xin = dalloc<double>(psi_size);
+    P->yout = dalloc<double>(psi_size);
+  }
+  CK(cudaMemcpyAsync(P->xin, x, psi_size * sizeof(double), cudaMemcpyDeviceToDevice, stream));
+  tc_run(P);
+  CK(cudaMemcpyAsync(y, P->yout, psi_size * sizeof(double), cudaMemcpyDeviceToDevice, stream));
+}
+
+void Engine::tc_buffers(TcPlan* P, double**& in, double**& out) {
+  in = &P->xin;
+  out = &P->yout;
+}
+
+// P->yout = H_eff P->xin: the launches (and their graph) read and write these buffers
+void Engine::tc_run(TcPlan* P) {
+  settle();
   CK(cudaEventRecord(ev0, stream));
   auto launches = [&](const double* xi, double* yo) {
     launch_tc_convert_psi(xi, P->d_sec, P->nsec, psi_size, P->prec, P->psi[0], P->psi[1], P->psi_pitch, stream);
@@ -861,18 +878,7 @@ void Engine::tc_apply(TcPlan* P, const double* x, double* y) {
     CK(cudaEventRecordWithFlags(evg1, stream, evf));
     launch_tc_reduce(P->d_red, P->nred, P->red_total, P->part, yo, stream);
   };
-  if (use_graphs) {
-    // the graph reads and writes fixed buffers
-    if (!P->xin) {
-      P->xin = dalloc<double>(psi_size);
-      P->yout = dalloc<double>(psi_size);
-    }
-    CK(cudaMemcpyAsync(P->xin, x, psi_size * sizeof(double), cudaMemcpyDeviceToDevice, stream));
-    replay(P->graph, [&]() { launches(P->xin, P->yout); });
-    CK(cudaMemcpyAsync(y, P->yout, psi_size * sizeof(double), cudaMemcpyDeviceToDevice, stream));
-  } else {
-    launches(x, y);
-  }
+  replay(P->graph, [&]() { launches(P->xin, P->yout); });
   CK(cudaEventRecord(ev1, stream));
   CK(cudaMemcpyAsync(tc_err_host, P->d_err, sizeof(int), cudaMemcpyDeviceToHost, stream));
   stats.launches += P->nred ? 4 : 3;
