@@ -56,7 +56,8 @@ constexpr int XM = kSplitTile, XK = kSplitChunk;
 constexpr int NS = 7;                           // digits
 constexpr int kWarps = 12, XT = 32 * kWarps + 32;   // 13 warps: at most 4 on a sub-core, 128 registers
 constexpr int kStages = 3;
-constexpr int kRec = XM * (NS * 64 + 4);        // bytes of a full record: 64 rows x (7 x 32 halves + exponent)
+constexpr int kPlane = XM * 64;                 // bytes of a digit plane in a stage: 64 rows of 32 halves
+constexpr int kRec = NS * kPlane + XM * 4;      // a stage's operand: 7 planes and the exponents
 constexpr int kHead = 64;                       // bytes of a stage's header
 constexpr int kSmem = kStages * (2 * kRec + kHead) + 2 * kStages * 8 + 16;
 constexpr float kMagic = 12582912.0f;           // 1.5 x 2^23: integers in +-2^22 added to it are its low mantissa bits
@@ -117,6 +118,31 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], u
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// the first product of a sum: the accumulator's start is the constant operand
+__device__ __forceinline__ void mma_f16_first(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(kMagic));
+}
+// digit products of 16 columns into the sums of the eight weights (FIRST: their first)
+template <bool FIRST>
+__device__ __forceinline__ void weights(float (&f)[8][4], uint32_t ad, uint32_t bd) {
+  uint32_t a[NS][4];
+#pragma unroll
+  for (int x = 0; x < NS; ++x) ldsm4(ad + x * kPlane, a[x]);
+#pragma unroll
+  for (int jb = 0; jb < NS; ++jb) {
+    uint32_t b[2];
+    ldsm2(bd + jb * kPlane, b);
+#pragma unroll
+    for (int ia = 0; ia < NS; ++ia) {
+      if (ia + jb >= 8) continue;
+      if (FIRST && (jb == 0 || (jb == 1 && ia == 6))) mma_f16_first(f[ia + jb], a[ia], b[0], b[1]);
+      else mma_f16(f[ia + jb], a[ia], b[0], b[1]);
+    }
+  }
 }
 // Byte offset of 16-byte piece c of a digit row: rows of 64 bytes (32 columns,
 // c 0..3) or 32 bytes (chunks of at most 16 columns, c 0..1).  The eight rows
@@ -261,8 +287,9 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
   }
   __syncthreads();
   if (warp == kWarps) {
-    if (lane != 0) return;
-    // ---------------- producer
+    // ---------------- producer: lane 0 keeps the books, lanes 0-15 copy the
+    // seven planes and the exponents of both operands (planes keep one pitch in
+    // the stage, so that the consumers' addresses are constants apart)
     int s = 0;
     uint32_t ph = 0;
     bool ok = true;
@@ -270,8 +297,8 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
     // differ by an order of magnitude in length (dealt out in turn, the
     // busiest SM of a CAS(16,16) stage A worked 1.3 times as long as the mean)
     int wnext = 0;
-    for (int w = blockIdx.x; w < nwork && ok; w = wnext) {
-      wnext = (int)gridDim.x + atomicAdd(next, 1);   // needed after this piece
+    for (int w = blockIdx.x; w < nwork && ok; w = __shfl_sync(0xffffffffu, wnext, 0)) {
+      if (lane == 0) wnext = (int)gridDim.x + atomicAdd(next, 1);   // needed after this piece
       const SplitWork W = work[w];
       const GemmOut o = outs[W.out];
       Head h;
@@ -283,6 +310,8 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
       h.ldc = W.slot >= 0 ? XM : o.ldc;
       const int beta = W.slot < 0 && o.beta ? kBeta : 0;
       const int ra = pad8(h.mr), rb = pad8(h.nr);
+      const int side = lane >> 3, x = lane & 7;   // this lane's copy: operand (0, 1) and plane (7: exponents)
+      const int rows = side ? rb : ra, row0 = side ? h.n0 : h.m0;
       int t = W.t0, k0 = W.k0;
       SplitTerm T = sterms[t];
       for (int i = 0; i < W.steps; ++i) {
@@ -296,22 +325,30 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         h.term = T.term;
         h.alpha = T.alpha;
         h.k0 = k0;
-        const int row_bytes = NS * h.nh * 32 + 4, chunk = k0 / XK;
-        if (!mbar_wait(&empty[s], ph ^ 1, err)) { ok = false; break; }
-        heads[s] = h;
+        const int chunk = k0 / XK, row_bytes = NS * h.nh * 32 + 4;
+        ok = mbar_wait(&empty[s], ph ^ 1, err);
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         uint8_t* st = sm + s * 2 * kRec;
-        mbar_expect(&full[s], (uint32_t)((ra + rb) * row_bytes));
-        bulk_copy(st, digits + T.a + (int64_t)chunk * T.ra * (NS * 64 + 4) + (int64_t)h.m0 * row_bytes, ra * row_bytes,
-                  &full[s]);
-        bulk_copy(st + kRec, digits + T.b + (int64_t)chunk * T.rb * (NS * 64 + 4) + (int64_t)h.n0 * row_bytes,
-                  rb * row_bytes, &full[s]);
+        if (lane == 0) {
+          heads[s] = h;
+          mbar_expect(&full[s], (uint32_t)((ra + rb) * row_bytes));
+        }
+        __syncwarp();
+        if (lane < 16) {
+          const uint8_t* rec = digits + (side ? T.b : T.a) + (int64_t)chunk * (side ? T.rb : T.ra) * (NS * 64 + 4) +
+                               (int64_t)row0 * row_bytes;
+          const int plane = rows * h.nh * 32;
+          bulk_copy(st + side * kRec + x * kPlane, rec + x * plane, x < NS ? plane : rows * 4, &full[s]);
+        }
         if (++s == kStages) { s = 0; ph ^= 1; }
         k0 += XK;
       }
     }
     if (ok && mbar_wait(&empty[s], ph ^ 1, err)) {
-      heads[s].flags = kEnd;
-      mbar_arrive(&full[s]);
+      if (lane == 0) {
+        heads[s].flags = kEnd;
+        mbar_arrive(&full[s]);
+      }
     } else {
       // stages armed but never consumed: let their copies land before the CTA exits
       for (int i = 0; i < kStages; ++i)
@@ -344,9 +381,8 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
     }
     if (on) {
-      const int pa = pad8(h.mr) * nh * 32, pb = pad8(h.nr) * nh * 32;   // plane bytes
-      const int* expA = reinterpret_cast<const int*>(ra + NS * pa);
-      const int* expB = reinterpret_cast<const int*>(rb + NS * pb);
+      const int* expA = reinterpret_cast<const int*>(ra + NS * kPlane);
+      const int* expB = reinterpret_cast<const int*>(rb + NS * kPlane);
       const int r0 = 16 * g + (lane >> 2);
       // rows and columns outside the tile hold whatever the stage held before: never stored
       const bool ok0 = r0 < h.mr, ok1 = r0 + 8 < h.mr;
@@ -378,37 +414,21 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
           }
           continue;
         }
-        float f[8][4];
-#pragma unroll
-        for (int d = 0; d < 8; ++d)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) f[d][j] = kMagic;
         // one half of the columns at a time: 28 registers of A digits, read
         // again for every 8 columns, leave room for three warps a sub-core
-        const int brow = c8 + (lane & 7);
-        for (int hh = 0; hh < nh; ++hh) {
-          uint32_t a[NS][4];
-          const uint32_t ad = hh ? ad1 : ad0;
-#pragma unroll
-          for (int x = 0; x < NS; ++x) ldsm4(ad + x * pa, a[x]);
-          const uint32_t bd = smem_addr(rb + piece(brow, 2 * hh + ((lane >> 3) & 1), nh));
-#pragma unroll
-          for (int jb = 0; jb < NS; ++jb) {
-            uint32_t b[2];
-            ldsm2(bd + jb * pb, b);
-#pragma unroll
-            for (int ia = 0; ia < NS; ++ia)
-              if (ia + jb < 8) mma_f16(f[ia + jb], a[ia], b[0], b[1]);
-          }
-        }
+        float f[8][4];
+        const int brow = c8 + (lane & 7), bc = (lane >> 3) & 1;
+        weights<true>(f, ad0, smem_addr(rb + piece(brow, bc, nh)));
+        if (nh == 2) weights<false>(f, ad1, smem_addr(rb + piece(brow, 2 + bc, 2)));
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          auto bits = [&](int d) { return (int)(__float_as_uint(f[d][j]) - kMagicBits); };
-          // weights 2^40 .. 2^0, and the last two rounded to units
-          const int q = bits(0) * 256 + bits(1);
-          const int p = bits(2) * 256 + bits(3);
-          const int l = bits(4) * 256 + bits(5) + ((bits(6) * 256 + bits(7) + 32768) >> 16);
-          const int64_t v = ((int64_t)q << 32) + (int64_t)p * 65536 + l;
+          // the sums are the accumulators' bits less kMagicBits, 2^8 apart from
+          // 2^40 down to 2^0, the last two rounded to units; the constants of
+          // two weights are taken off together (all of it modulo 2^32)
+          auto two = [&](int d) { return __float_as_uint(f[d][j]) * 256u + __float_as_uint(f[d + 1][j]); };
+          const int p = (int)(two(2) - kMagicBits * 257u);
+          const int l = (int)(two(4) - kMagicBits * 257u) + ((int)(two(6) - (kMagicBits * 257u - 32768u)) >> 16);
+          const int64_t v = (int64_t)p * 65536 + l + (int64_t)((uint64_t)(two(0) - kMagicBits * 257u) << 32);
           const int e = (j < 2 ? x0 : x1) + ((j & 1) ? y1 : y0) - 2100;
           acc[i][j] = fma(__ll2double_rn(v), __hiloint2double(ahi + (int)((uint32_t)e << 20), alo), acc[i][j]);
         }
