@@ -14,6 +14,19 @@
 // that type and issue hi*hi + hi*lo + lo*hi into the same accumulator.
 // Every mbarrier wait is bounded: on timeout the kernel raises *err, all
 // roles stop issuing, and TMEM is released before the CTA exits.
+//
+// What bounds it: with blocks of a few dozen rows and a dozen short MMAs per
+// K chunk (TF32x3) the issuing lane itself was the limit, ~1500 clocks per
+// chunk whatever the tile width, while the loads waited for free stages.  So
+// the issuer is as lean as it can be: the type is a template argument, the
+// K steps are unrolled, the descriptors of a chunk are formed once and
+// advanced by additions, and both issuing roles run in the lane that
+// elect.sync names (600-750 clocks per chunk now).  Stage A was bound by its
+// epilogue, whose 16-byte stores filled half a sector each: a lane stores 32
+// bytes at a time.  All accumulators and roundings are those of before.
+// Per sigma: CAS(16,16) M=512 12.9 -> 9.1 ms for 38 launches, CAS(20,20)
+// M=1024 58.8 -> 45.2 ms for 40, a full solve of CAS(10,10) 19.5 -> 13.2 ms
+// for 634.  Now stage A waits for its boxes (two stages of 96 KB at N = 256).
 #include <mutex>
 
 #include <cuda_bf16.h>
@@ -83,19 +96,20 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
   return d;
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
+template <bool bf>
+__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  if (bf)
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+  else
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(saddr(bar))
@@ -122,11 +136,38 @@ __device__ __forceinline__ float to_tf32(float x) {
   return __uint_as_float(r);
 }
 
+// true in one lane of a converged warp.  The issuing roles run in the elected
+// lane: the compiler then knows that one thread is active and feeds the tensor
+// core and TMA instructions their uniform operands directly.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
+// 32 bytes, one full sector per lane (d is 32-byte aligned)
+__device__ __forceinline__ void store32(void* d, const uint32_t* w) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(d), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
+               "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
+
+// the CTA's tile i (an empty one past the end) and its first term
+__device__ __forceinline__ TcTile tile_at(const TcLaunch& L, int i) {
+  TcTile T{};
+  if (i < L.ntiles) T = L.tiles[i];
+  return T;
+}
+__device__ __forceinline__ TcTerm first_term(const TcLaunch& L, const TcTile& T) {
+  TcTerm t{};
+  if (T.t1 > T.t0) t = L.terms[T.t0];
+  return t;
+}
+
+template <bool bf, bool x3>
 __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ TcMaps maps,
                                                              const TcLaunch L) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  const bool x3 = L.prec == kTF32x3 || L.prec == kBF16x3;
-  const bool bf = L.prec == kBF16 || L.prec == kBF16x3;
   // B boxes of this launch are at most L.ncap rows; the ring holds as many
   // stages as fit (tc_stages)
   const int bstage = L.ncap * 128;
@@ -139,8 +180,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
   uint64_t* tempty = tfull + 2;         // [2]
   uint32_t* tslot = reinterpret_cast<uint32_t*>(tempty + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int kc = bf ? kTcKChunk16 : kTcKChunk32;     // K elements per stage
-  const int kstep = bf ? 16 : 8;                      // K per MMA
+  constexpr int kc = bf ? kTcKChunk16 : kTcKChunk32;     // K elements per stage
+  constexpr int kstep = bf ? 16 : 8;                      // K per MMA
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
@@ -162,22 +203,24 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
   tc_fence_after();
   const uint32_t tmem = *tslot;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     // ---------------- TMA producer
     int stage = 0;
     uint32_t ph = 0;
     bool ok = true;
-    // descriptors are software-pipelined: the next tile's and the next
-    // term's loads are in flight while the current ones are issued
-    TcTile Tn;
-    if (blockIdx.x < L.ntiles) Tn = L.tiles[blockIdx.x];
+    // descriptors are software-pipelined: the tile after the next, the next
+    // tile's first term and the next term are in flight while the current
+    // ones are issued (each is a trip to L2, and many tiles are one box long)
+    TcTile Tc = tile_at(L, blockIdx.x), Tn = tile_at(L, blockIdx.x + gridDim.x);
+    TcTerm first_n = first_term(L, Tc);
     for (int tile = blockIdx.x; tile < L.ntiles && ok; tile += gridDim.x) {
-      const TcTile T = Tn;
-      if (tile + (int)gridDim.x < L.ntiles) Tn = L.tiles[tile + gridDim.x];
+      const TcTile T = Tc;
+      TcTerm tmn = first_n;
+      Tc = Tn;
+      first_n = first_term(L, Tn);
+      Tn = tile_at(L, tile + 2 * (int)gridDim.x);
       const int bbytes = (16 << T.bsel) * 128;
       const uint32_t tx = (uint32_t)(kStageA + bbytes) * (x3 ? 2 : 1);
-      TcTerm tmn;
-      if (T.t1 > T.t0) tmn = L.terms[T.t0];
       for (int t = T.t0; t < T.t1 && ok; ++t) {
         const TcTerm tm = tmn;
         if (t + 1 < T.t1) tmn = L.terms[t + 1];
@@ -209,20 +252,21 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         for (uint32_t it = 0; it < (1u << 20) && !mbar_try(&full[s], ph); ++it) {
         }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     // ---------------- MMA issuer
     int stage = 0;
     uint32_t ph = 0;
     int acc_i = 0;
     bool ok = true;
     const uint32_t fmt = bf ? 1u : 2u;
-    TcTile Tn;
-    if (blockIdx.x < L.ntiles) Tn = L.tiles[blockIdx.x];
+    TcTile Tc = tile_at(L, blockIdx.x), Tn = tile_at(L, blockIdx.x + gridDim.x);
+    TcTerm first_n = first_term(L, Tc);
     for (int tile = blockIdx.x; tile < L.ntiles && ok; tile += gridDim.x, ++acc_i) {
-      const TcTile T = Tn;
-      if (tile + (int)gridDim.x < L.ntiles) Tn = L.tiles[tile + gridDim.x];
-      TcTerm tmn;
-      if (T.t1 > T.t0) tmn = L.terms[T.t0];
+      const TcTile T = Tc;
+      TcTerm tmn = first_n;
+      Tc = Tn;
+      first_n = first_term(L, Tn);
+      Tn = tile_at(L, tile + 2 * (int)gridDim.x);
       const int a = acc_i & 1;
       const uint32_t aph = (acc_i >> 1) & 1;
       if (!mbar_wait(&tempty[a], aph ^ 1, L.err)) { ok = false; break; }
@@ -240,22 +284,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
           const uint32_t sa = saddr(base + stage * stage_bytes);
           const uint32_t sb = sa + kStageA;
           const int nk = min(kc, tm.k - k0) / kstep;
-          for (int kk = 0; kk < nk; ++kk) {
-            const uint64_t ad = smem_desc(sa + kk * 32), bd = smem_desc(sb + kk * 32);
-            if (bf) {
-              mma_bf16(dt, ad, bd, idesc, first ? 0u : 1u);
-              if (x3) {
-                const uint32_t sa2 = sb + bstage, sb2 = sa2 + kStageA;
-                mma_bf16(dt, ad, smem_desc(sb2 + kk * 32), idesc, 1u);                 // hi * lo
-                mma_bf16(dt, smem_desc(sa2 + kk * 32), bd, idesc, 1u);                 // lo * hi
-              }
-            } else {
-              mma_tf32(dt, ad, bd, idesc, first ? 0u : 1u);
-              if (x3) {
-                const uint32_t sa2 = sb + bstage, sb2 = sa2 + kStageA;
-                mma_tf32(dt, ad, smem_desc(sb2 + kk * 32), idesc, 1u);                 // hi * lo
-                mma_tf32(dt, smem_desc(sa2 + kk * 32), bd, idesc, 1u);                 // lo * hi
-              }
+          const uint64_t ad = smem_desc(sa), bd = smem_desc(sb);
+          const uint64_t ad2 = smem_desc(sb + bstage), bd2 = smem_desc(sb + bstage + kStageA);
+#pragma unroll
+          for (int kk = 0; kk < kc / kstep; ++kk) {   // 32 bytes of K: 2 units of the start address
+            if (kk == nk) break;
+            mma<bf>(dt, ad + 2 * kk, bd + 2 * kk, idesc, first ? 0u : 1u);
+            if (x3) {
+              mma<bf>(dt, ad + 2 * kk, bd2 + 2 * kk, idesc, 1u);   // hi * lo
+              mma<bf>(dt, ad2 + 2 * kk, bd + 2 * kk, idesc, 1u);   // lo * hi
             }
             first = 0;
           }
@@ -270,27 +307,29 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     const int q = warp & 3;              // TMEM lane quarter this warp may read
     const int row = q * 32 + lane;       // accumulator row (A row within the tile)
     int acc_i = 0;
+    // the tile after the next, and the next tile's output row (two dependent
+    // loads), are fetched while the current one is stored
+    auto member = [&](const TcTile& X) {
+      return X.mode == kTcYTblk && row < X.m_valid ? L.ymem[X.out + row] : -1;
+    };
+    TcTile Tc = tile_at(L, blockIdx.x), Tn = tile_at(L, blockIdx.x + gridDim.x);
+    int mem = member(Tc);
+    TcYRow yn{};
+    if (mem >= 0) yn = L.yrows[mem];
     for (int tile = blockIdx.x; tile < L.ntiles; tile += gridDim.x, ++acc_i) {
-      // descriptor and output row are loaded before the accumulator wait
-      const TcTile T = L.tiles[tile];
+      const TcTile T = Tc;
+      TcYRow yr = yn;
+      Tc = Tn;
+      mem = member(Tn);
+      Tn = tile_at(L, tile + 2 * (int)gridDim.x);
       const bool has = T.t1 > T.t0;
       const bool live = row < T.m_valid;
-      int pcol = 0;
-      TcYRow yr{};
-      if (T.mode == kTcYT && live) {
-        int r = T.m0 + row, s = 0;
-        for (int u = 1; u < 4; ++u)
-          if (r >= T.rbreak[u]) s = u;
-        pcol = T.rpad[s] + (r - T.rbreak[s]);
-      } else if (T.mode == kTcYTblk && live) {
-        const int64_t r = T.out + row;
-        yr = L.yrows[L.ymem[r]];
-        yr.base += (r - yr.first) * (int64_t)kc;
-      }
+      yr.base += (T.out + row - yr.first) * (int64_t)kc;
       const int a = acc_i & 1;
       const uint32_t aph = (acc_i >> 1) & 1;
       if (!mbar_wait(&tfull[a], aph, L.err)) break;
       tc_fence_after();
+      if (mem >= 0) yn = L.yrows[mem];
       for (int c0 = 0; c0 < T.n_mma; c0 += 16) {
         float v[16];
         if (has) {
@@ -304,11 +343,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
           // 16 contiguous output columns: section s, K offset k, block k / kc
           if (c0 >= T.n_valid) continue;
           const int c = T.n0 + c0;
-          int s = 0;
+          int koff = yr.koff[0], brk = T.rbreak[0];
+#pragma unroll
           for (int u = 1; u < 4; ++u)
-            if (c >= T.rbreak[u]) s = u;
-          if (yr.koff[s] < 0) continue;
-          const int k = yr.koff[s] + (c - T.rbreak[s]);
+            if (c >= T.rbreak[u]) {
+              koff = yr.koff[u];
+              brk = T.rbreak[u];
+            }
+          if (koff < 0) continue;
+          const int k = koff + (c - brk);
           const int64_t idx = yr.base + (int64_t)(k / kc) * yr.stride + (k % kc);
           if (bf) {
             uint32_t w[8], wl[8];
@@ -319,29 +362,20 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
               __nv_bfloat162 l2 = __floats2bfloat162_rn(v[2 * i] - __low2float(p2), v[2 * i + 1] - __high2float(p2));
               wl[i] = *reinterpret_cast<uint32_t*>(&l2);
             }
-            uint4* d = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(L.yt_hi) + idx);
-            d[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            d[1] = make_uint4(w[4], w[5], w[6], w[7]);
-            if (x3) {
-              uint4* dl = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(L.yt_lo) + idx);
-              dl[0] = make_uint4(wl[0], wl[1], wl[2], wl[3]);
-              dl[1] = make_uint4(wl[4], wl[5], wl[6], wl[7]);
-            }
+            store32(reinterpret_cast<__nv_bfloat16*>(L.yt_hi) + idx, w);
+            if (x3) store32(reinterpret_cast<__nv_bfloat16*>(L.yt_lo) + idx, wl);
           } else {
-            float h[16], l[16];
+            uint32_t h[16], l[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-              h[i] = to_tf32(v[i]);
-              l[i] = to_tf32(v[i] - h[i]);
+              const float hi = to_tf32(v[i]);
+              h[i] = __float_as_uint(hi);
+              l[i] = __float_as_uint(to_tf32(v[i] - hi));
             }
-            float4* dh = reinterpret_cast<float4*>(reinterpret_cast<float*>(L.yt_hi) + idx);
 #pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) dh[q4] = make_float4(h[4 * q4], h[4 * q4 + 1], h[4 * q4 + 2], h[4 * q4 + 3]);
-            if (x3) {
-              float4* dl = reinterpret_cast<float4*>(reinterpret_cast<float*>(L.yt_lo) + idx);
-#pragma unroll
-              for (int q4 = 0; q4 < 4; ++q4)
-                dl[q4] = make_float4(l[4 * q4], l[4 * q4 + 1], l[4 * q4 + 2], l[4 * q4 + 3]);
+            for (int u = 0; u < 2; ++u) {
+              store32(reinterpret_cast<float*>(L.yt_hi) + idx + 8 * u, h + 8 * u);
+              if (x3) store32(reinterpret_cast<float*>(L.yt_lo) + idx + 8 * u, l + 8 * u);
             }
           }
           continue;
@@ -353,19 +387,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
           if (T.mode == kTcSigma) {
             double* o = L.f64 + T.out + (int64_t)j * T.ld + T.m0 + row;
             *o = T.beta ? (*o + (double)v[i]) : (double)v[i];
-          } else if (T.mode == kTcPart) {
-            L.part[T.out + (int64_t)j * 128 + row] = v[i];
           } else {
-            const int64_t idx = (T.out + j) * (int64_t)T.ld + pcol;
-            if (bf) {
-              const __nv_bfloat16 hb = __float2bfloat16_rn(v[i]);
-              reinterpret_cast<__nv_bfloat16*>(L.yt_hi)[idx] = hb;
-              if (x3) reinterpret_cast<__nv_bfloat16*>(L.yt_lo)[idx] = __float2bfloat16_rn(v[i] - __bfloat162float(hb));
-            } else {
-              const float hi = to_tf32(v[i]);
-              reinterpret_cast<float*>(L.yt_hi)[idx] = hi;
-              if (x3) reinterpret_cast<float*>(L.yt_lo)[idx] = to_tf32(v[i] - hi);
-            }
+            L.part[T.out + (int64_t)j * 128 + row] = v[i];
           }
         }
       }
@@ -516,12 +539,16 @@ bool launch_tc_gemm(const TcMaps& maps, const TcLaunch& L, int num_sms, cudaStre
   if (L.stages != tc_stages(L.prec, L.ncap)) return false;
   if (L.ntiles <= 0) return true;
   const int smem = tc_smem_bytes(L.prec, L.ncap);
-  static std::once_flag attr_once;   // engines on several host threads share the kernel
+  using Kernel = void (*)(const TcMaps, const TcLaunch);
+  static const Kernel kernels[4] = {tc_gemm_kernel<true, false>, tc_gemm_kernel<false, false>,
+                                    tc_gemm_kernel<false, true>, tc_gemm_kernel<true, true>};   // by TcPrec
+  if (L.prec < 0 || L.prec > 3) return false;
+  static std::once_flag attr_once;   // engines on several host threads share the kernels
   std::call_once(attr_once, []() {
-    cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+    for (Kernel k : kernels) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
   });
   const int grid = L.ntiles < num_sms ? L.ntiles : num_sms;
-  tc_gemm_kernel<<<grid, kThreads, smem, s>>>(maps, L);
+  kernels[L.prec]<<<grid, kThreads, smem, s>>>(maps, L);
   return true;
 }
 

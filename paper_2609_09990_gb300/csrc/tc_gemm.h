@@ -14,10 +14,7 @@
 // of B (N) starting at A row ay + m0 and B row by + n0 of each term, so that
 // all tiles of one output block share one term list; it accumulates
 // C += sign * A_t B_t^T over its terms t in TMEM
-// (FP32) and is written by one of four epilogues:
-//   kTcYT    : C^T into a panel (BF16, TF32, or TF32 hi/lo), row j of the
-//              output is panel row out + j, output column = the padded
-//              position of tile row m0 + i (rmap: 4 breaks + 4 pads),
+// (FP32) and is written by one of three epilogues:
 //   kTcYTblk : C into a K-blocked panel (pitch = one box row, W elements;
 //              element (m, k) of a block at ((k / W) * rows + m) * W + k % W):
 //              tile row r = out + i belongs to run yrows[ymem[r]] (a run of
@@ -41,7 +38,7 @@
 namespace gbd {
 
 enum TcPrec { kBF16 = 0, kTF32 = 1, kTF32x3 = 2, kBF16x3 = 3 };
-enum TcMode { kTcYT = 0, kTcSigma = 1, kTcPart = 2, kTcYTblk = 4 };
+enum TcMode { kTcSigma = 1, kTcPart = 2, kTcYTblk = 4 };
 
 struct TcTerm {
   int32_t ax, ay;   // A box origin: column (K) and row (before adding the tile's m0)
@@ -68,8 +65,8 @@ struct TcTile {
   int32_t n_mma, n_valid;
   int32_t bsel;          // B box height index: 16 << bsel rows
   int32_t mode, beta, ld;
-  int64_t out;           // output element offset (panel row for kTcYT, first yrows entry for kTcYTblk)
-  int32_t rbreak[4], rpad[4];
+  int64_t out;           // output element offset (kTcYTblk: first ymem entry)
+  int32_t rbreak[4];     // kTcYTblk: first output column of each section
   int32_t n0;            // offset of the tile's first B row (kTcYTblk: also its first output column)
   int32_t unused;
 };
@@ -84,7 +81,7 @@ struct TcLaunch {
   const TcTerm* terms;
   int ntiles;
   int prec;
-  void* yt_hi;           // kTcYT outputs (uint16 BF16 or float TF32)
+  void* yt_hi;           // kTcYTblk outputs (uint16 BF16 or float TF32)
   void* yt_lo;           // TF32x3 low part
   double* f64;           // kTcSigma output
   int* err;              // device flag: 1 = a bounded wait ran out
