@@ -31,17 +31,20 @@
 // seven digit planes, swizzled for ldmatrix, and the rows' exponents, all
 // contiguous.  gemm_f64_split multiplies 64 x 64 output tiles: one thread
 // streams the records of all chunks of all terms of all tiles of its CTA
-// through a ring of three stages by bulk copies, twelve warps multiply.  Long
+// through a ring of three stages by bulk copies, sixteen warps multiply.  Long
 // chains are cut into pieces with partial sums, added in a fixed order.
-// What bounds it: per 64 x 64 x 32 chunk 4350 clocks of mma.sync (34 pairs)
-// and 4096 clocks of the FP64 pipe (conversion and FMA of every output
-// element), which overlap between the three warps of a sub-core; both pipes
-// are 41 to 47 % busy in the H_eff product of CAS(16,16) M=512 (39 GFLOP):
-// 79 ms with FP64 FMAs, 21 ms with a first kernel that split its operands
-// itself, tile by tile, 9.9 ms here (operands 0.8, products 5.2 + 2.9),
-// 4.0 TFLOP/s against the FP64 pipe's 1.2.  Eight warps that kept all A digits
-// in registers: 7.8 + 3.6 ms for the products, with the work dealt out in
-// turn instead of by a counter.
+// What bounds it: a 64 x 64 x 32 chunk takes 4350 clocks of mma.sync (34
+// pairs) and 2048 clocks of FP64 FMAs, but the sub-blocks are small (35 % of
+// a chunk's products are real in CAS(16,16) M=512, 58 % in CAS(20,20)
+// M=1024), so that a warp has one 16 x 8 block per chunk and its latencies
+// count: loading fragments, putting the weights together, the barriers.
+// Four consumer warps a sub-core hide them best: with 96 registers a thread,
+// the B digits of a block and two planes of A in registers, the header left
+// in shared memory and no division in a chunk, the H_eff product of
+// CAS(16,16) M=512 (39 GFLOP) takes 8.4 ms (operands 0.8) and the one of
+// CAS(20,20) M=1024 (432 GFLOP) 53 ms; twelve warps with all A digits in
+// registers took 9.15 and 56 ms, eight 12 ms, a first kernel that split its
+// operands itself, tile by tile, 21 ms, and FP64 FMAs 79 and 562 ms.
 #include <cuda_runtime.h>
 
 #include <cuda_fp16.h>
@@ -54,7 +57,7 @@ namespace {
 
 constexpr int XM = kSplitTile, XK = kSplitChunk;
 constexpr int NS = 7;                           // digits
-constexpr int kWarps = 12, XT = 32 * kWarps + 32;   // 13 warps: at most 4 on a sub-core, 128 registers
+constexpr int kWarps = 16, XT = 32 * kWarps + 32;   // 17 warps: at most 5 on a sub-core, 96 registers
 constexpr int kStages = 3;
 constexpr int kPlane = XM * 64;                 // bytes of a digit plane in a stage: 64 rows of 32 halves
 constexpr int kRec = NS * kPlane + XM * 4;      // a stage's operand: 7 planes and the exponents
@@ -126,21 +129,22 @@ __device__ __forceinline__ void mma_f16_first(float (&c)[4], const uint32_t (&a)
       : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(kMagic));
 }
-// digit products of 16 columns into the sums of the eight weights (FIRST: their first)
+// digit products of 16 columns into the sums of the eight weights (FIRST:
+// their first): B's seven planes in registers, A's read one ahead
 template <bool FIRST>
 __device__ __forceinline__ void weights(float (&f)[8][4], uint32_t ad, uint32_t bd) {
-  uint32_t a[NS][4];
+  uint32_t b[NS][2], a[2][4];
+  ldsm4(ad, a[0]);
 #pragma unroll
-  for (int x = 0; x < NS; ++x) ldsm4(ad + x * kPlane, a[x]);
+  for (int x = 0; x < NS; ++x) ldsm2(bd + x * kPlane, b[x]);
 #pragma unroll
-  for (int jb = 0; jb < NS; ++jb) {
-    uint32_t b[2];
-    ldsm2(bd + jb * kPlane, b);
+  for (int ia = 0; ia < NS; ++ia) {
+    if (ia + 1 < NS) ldsm4(ad + (ia + 1) * kPlane, a[(ia + 1) & 1]);
 #pragma unroll
-    for (int ia = 0; ia < NS; ++ia) {
+    for (int jb = 0; jb < NS; ++jb) {
       if (ia + jb >= 8) continue;
-      if (FIRST && (jb == 0 || (jb == 1 && ia == 6))) mma_f16_first(f[ia + jb], a[ia], b[0], b[1]);
-      else mma_f16(f[ia + jb], a[ia], b[0], b[1]);
+      if (FIRST && (ia == 0 || (ia == 1 && jb == 6))) mma_f16_first(f[ia + jb], a[ia & 1], b[jb][0], b[jb][1]);
+      else mma_f16(f[ia + jb], a[ia & 1], b[jb][0], b[jb][1]);
     }
   }
 }
@@ -358,23 +362,26 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
     return;
   }
   // ---------------- consumers
-  constexpr int kN8 = 3;   // 8-column groups of a warp: 8 of a tile over 12 / 4 warps
+  constexpr int kN8 = 2;   // 8-column groups of a warp: 8 of a tile over 16 / 4 warps
   double acc[kN8][4];
   int s = 0;
   uint32_t ph = 0;
   for (;;) {
     if (!mbar_wait(&full[s], ph, err)) break;
-    const Head h = heads[s];
-    if (h.flags & kEnd) break;
+    const Head& h = heads[s];   // read where it is needed: registers are short
+    const int flags = h.flags;
+    if (flags & kEnd) break;
     const uint8_t* ra = sm + s * 2 * kRec;
     const uint8_t* rb = ra + kRec;
     const int nh = h.nh;
     // warps: row groups of 16, and the 8-column groups dealt out among the
     // warps of a row group, so that small tiles keep most warps at work
-    const int nm = (h.mr + 15) >> 4, per = kWarps / nm, g = warp % nm, nb = warp / nm;
+    // (warp / nm and kWarps / nm for nm = 1..4 from packed constants)
+    const int nm = (h.mr + 15) >> 4, sh = 8 * (nm - 1);
+    const int nb = warp * (int)(0x10162040u >> sh & 0xFFu) >> 6, per = (int)(0x04050810u >> sh & 0xFFu), g = warp - nb * nm;
     const int n8 = (h.nr + 7) >> 3;
     const bool on = nb < per && nb < n8;
-    if (h.flags & kFirst) {
+    if (flags & kFirst) {
 #pragma unroll
       for (int i = 0; i < kN8; ++i)
 #pragma unroll
@@ -398,6 +405,13 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         if (c8 >= h.nr) break;
         const int c = c8 + 2 * (lane & 3);
         const int y0 = c < h.nr ? expB[c] : 1023, y1 = c + 1 < h.nr ? expB[c + 1] : 1023;
+        // one half of the columns at a time: 14 registers of B digits and 8
+        // of A leave room for four warps a sub-core
+        float f[8][4];
+        const int brow = c8 + (lane & 7), bc = (lane >> 3) & 1;
+        weights<true>(f, ad0, smem_addr(rb + piece(brow, bc, nh)));
+        if (nh == 2) weights<false>(f, ad1, smem_addr(rb + piece(brow, 2 + bc, 2)));
+        // asked for only now, so that the exponents arrive during the products
         if (__any_sync(0xffffffffu, badA || y0 == kBadExp || y1 == kBadExp)) {
           // the chunk of these 16 x 8 outputs by FP64 FMAs from the operands themselves
           const GemmTerm T = terms[h.term];
@@ -414,12 +428,6 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
           }
           continue;
         }
-        // one half of the columns at a time: 28 registers of A digits, read
-        // again for every 8 columns, leave room for three warps a sub-core
-        float f[8][4];
-        const int brow = c8 + (lane & 7), bc = (lane >> 3) & 1;
-        weights<true>(f, ad0, smem_addr(rb + piece(brow, bc, nh)));
-        if (nh == 2) weights<false>(f, ad1, smem_addr(rb + piece(brow, 2 + bc, 2)));
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           // the sums are the accumulators' bits less kMagicBits, 2^8 apart from
@@ -434,10 +442,7 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         }
       }
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&empty[s]);
-    if (++s == kStages) { s = 0; ph ^= 1; }
-    if ((h.flags & kLast) && on) {
+    if ((flags & kLast) && on) {
 #pragma unroll
       for (int i = 0; i < kN8; ++i) {
         const int c = (nb + i * per) * 8 + 2 * (lane & 3);
@@ -446,10 +451,13 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
           const int r = 16 * g + (lane >> 2) + 8 * (j >> 1), cc = c + (j & 1);
           if (r >= h.mr || cc >= h.nr) continue;
           double* d = h.C + (int64_t)r * h.ldc + cc;
-          *d = h.flags & kBeta ? (*d + acc[i][j]) : acc[i][j];
+          *d = flags & kBeta ? (*d + acc[i][j]) : acc[i][j];
         }
       }
     }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
+    if (++s == kStages) { s = 0; ph ^= 1; }
   }
 }
 
