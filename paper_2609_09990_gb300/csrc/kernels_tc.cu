@@ -466,22 +466,108 @@ __device__ __forceinline__ void store_conv(double x, int prec, void* hi, void* l
   }
 }
 
-__global__ void tc_convert_kernel(const TcConv* __restrict__ tasks, int ntasks, int prec, void* hi, void* lo,
-                                  int64_t pitch) {
+// The same for TF32x3 and a finite value of ordinary size without the FP64
+// pipe, which takes 64 clocks for a warp's conversion or addition: x rounded
+// to FP32 and to TF32, and the rest x - hi (an integer of at most 43 bits in
+// units of x's last place) likewise.  Bit for bit what store_conv gives.
+__device__ __forceinline__ bool split_tf32(uint32_t xh, uint32_t xl, float* h, float* l) {
+  const int e = (int)((xh >> 20) & 0x7FFu) - 896;          // exponent field of the FP32 value
+  if (e < 80 || e > 250) return false;
+  const uint32_t m23 = (xh & 0xFFFFFu) << 3 | xl >> 29, rest = xl << 3;
+  uint32_t f = ((uint32_t)e << 23) + m23;
+  f += (rest > 0x80000000u || (rest == 0x80000000u && (m23 & 1u))) ? 1u : 0u;   // to nearest even
+  f = (f + 0x1000u) & 0xFFFFE000u;                          // to nearest, ties away
+  const int64_t mx = (int64_t)((uint64_t)((xh & 0xFFFFFu) | 0x100000u) << 32 | xl);
+  const int64_t mh = (int64_t)(f - ((uint32_t)e << 23) + 0x800000u) << 29;   // a carry into the exponent counts 2^23
+  const uint32_t sg = xh & 0x80000000u;
+  *h = __uint_as_float(f | sg);
+  *l = to_tf32(__ll2float_rn(sg ? mh - mx : mx - mh) * __uint_as_float((uint32_t)(e - 52) << 23));
+  return true;
+}
+
+// Likewise BF16, to nearest even from the FP64 bits.
+__device__ __forceinline__ bool round_bf16(uint32_t xh, uint32_t xl, uint16_t* b) {
+  const int e = (int)((xh >> 20) & 0x7FFu) - 896;
+  if (e < 1 || e > 253) return false;
+  const uint32_t v = (uint32_t)e << 7 | ((xh >> 13) & 0x7Fu), rest = xh << 19 | (xl ? 1u : 0u);
+  *b = (uint16_t)((xh >> 31 << 15) | (v + ((rest > 0x80000000u || (rest == 0x80000000u && (v & 1u))) ? 1u : 0u)));
+  return true;
+}
+
+// A block per sub-block.  Positions advance by additions (256 elements a step),
+// divisions are once a task, and four loads of a thread are in flight together.
+// Transposed sources (the conjugate channels) are read along their rows and
+// turned in shared memory, so that the panel rows are written in runs too:
+// single elements of 32 different sectors were the bound, then the five FP64
+// instructions an element.  The four conversions of a CAS(20,20) M=1024 step:
+// 13.0 -> 6.7 ms; additions for divisions alone 13.0, then without FP64 12.0,
+// turned in shared memory 7.3.
+__global__ void __launch_bounds__(256) tc_convert_kernel(const TcConv* __restrict__ tasks, int ntasks, int prec, void* hi,
+                                                         void* lo, int64_t pitch) {
+  constexpr int kU = 4, kBuf = 2048;
+  __shared__ double buf[kBuf];
+  const int sh = 63 - __clzll(pitch);   // K-blocked panels: pitch is a power of two
   for (int t = blockIdx.x; t < ntasks; t += gridDim.x) {
     const TcConv c = tasks[t];
-    const int64_t n = (int64_t)c.rows * c.cols;
-    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-      // transposed sources are walked along their rows (consecutive r), so
-      // that the reads stay coalesced
-      const int r = c.trans ? (int)(e % c.rows) : (int)(e / c.cols);
-      const int col = c.trans ? (int)(e / c.rows) : (int)(e % c.cols);
+    if (c.rows <= 0 || c.cols <= 0) continue;
+    const bool unit = fabs(c.scale) == 1.0;
+    const uint32_t flip = c.scale < 0.0 ? 0x80000000u : 0u;
+    auto put = [&](int r, int col, double x) {
+      col += c.c0;
       const int64_t dst = c.kstride > 0
-                              ? ((int64_t)c.r0 + (int64_t)((c.c0 + col) / pitch) * c.kstride + r) * pitch +
-                                    (c.c0 + col) % pitch
-                              : (int64_t)(c.r0 + r) * pitch + c.c0 + col;
-      const double x = c.trans ? c.src[(int64_t)col * c.ld_src + r] : c.src[(int64_t)r * c.ld_src + col];
-      store_conv(c.scale * x, prec, hi, lo, dst);
+                              ? (((int64_t)c.r0 + (int64_t)(col >> sh) * c.kstride + r) << sh) + (col & ((1 << sh) - 1))
+                              : (int64_t)(c.r0 + r) * pitch + col;
+      const uint32_t xh = (uint32_t)__double2hiint(x) ^ flip, xl = (uint32_t)__double2loint(x);
+      float h, l;
+      uint16_t b;
+      if (unit && prec == kTF32x3 && split_tf32(xh, xl, &h, &l)) {
+        reinterpret_cast<float*>(hi)[dst] = h;
+        reinterpret_cast<float*>(lo)[dst] = l;
+      } else if (unit && prec == kBF16 && round_bf16(xh, xl, &b)) {
+        reinterpret_cast<uint16_t*>(hi)[dst] = b;
+      } else {
+        store_conv(c.scale * x, prec, hi, lo, dst);
+      }
+    };
+    // elements (o, i) of an outer x inner rectangle, i fastest, 256 apart; four at a time
+    auto walk = [&](int outer, int inner, auto load, auto use) {
+      const int so = 256 / inner, si = 256 - so * inner;
+      int o = threadIdx.x / inner, i = threadIdx.x - o * inner;
+      while (o < outer) {
+        double x[kU];
+        int oo[kU], ii[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          oo[u] = o;
+          ii[u] = i;
+          if (o < outer) x[u] = load(o, i);
+          o += so;
+          i += si;
+          if (i >= inner) {
+            i -= inner;
+            ++o;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+          if (oo[u] < outer) use(oo[u], ii[u], x[u]);
+      }
+    };
+    if (!c.trans || c.rows > kBuf / 8) {
+      const int inner = c.trans ? c.rows : c.cols, outer = c.trans ? c.cols : c.rows;
+      walk(outer, inner, [&](int o, int i) { return c.src[(int64_t)o * c.ld_src + i]; },
+           [&](int o, int i, double x) { put(c.trans ? i : o, c.trans ? o : i, x); });
+      continue;
+    }
+    const int per = ((kBuf / c.rows) - 1) | 1;   // columns at a time, odd: no bank conflicts
+    for (int c0 = 0; c0 < c.cols; c0 += per) {
+      const int nc = min(per, c.cols - c0);
+      walk(nc, c.rows, [&](int o, int i) { return c.src[(int64_t)(c0 + o) * c.ld_src + i]; },
+           [&](int o, int i, double x) { buf[i * per + o] = x; });
+      __syncthreads();
+      walk(c.rows, nc, [&](int r, int o) { return buf[r * per + o]; },
+           [&](int r, int o, double x) { put(r, c0 + o, x); });
+      __syncthreads();
     }
   }
 }

@@ -120,7 +120,8 @@ bool launch_tc_gemm(const TcMaps& maps, const TcLaunch& L, int num_sms, cudaStre
 // conversion of FP64 blocks into panels: rows x cols block at src (ld_src)
 // written at panel row r0, column c0 (pitch); lo != nullptr for the split
 // (x3) types.  kstride > 0: K-blocked panel, column c0 + j goes to row
-// r0 + ((c0 + j) / pitch) * kstride, column (c0 + j) % pitch.
+// r0 + ((c0 + j) / pitch) * kstride, column (c0 + j) % pitch; pitch is
+// then one box row, a power of two.
 struct TcConv {
   const double* src;
   double scale;          // multiplies every element (the sub-block's coefficient)
