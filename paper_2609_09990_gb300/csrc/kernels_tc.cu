@@ -421,19 +421,52 @@ __global__ void bounded_wait_probe_kernel(int arrive, int* err, int* waited_ok) 
   }
 }
 
+// the last of n records (n > 0) whose key, ascending from key(0) <= e, is at
+// most e, found by a converged warp: 32 probes a round instead of one
+template <class Key>
+__device__ __forceinline__ int warp_find(int n, int64_t e, Key key) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, hi = n;
+  while (hi - lo > 1) {
+    const int step = (hi - lo + 31) >> 5, i = lo + lane * step;
+    const int k = __popc(__ballot_sync(0xffffffffu, i < hi && key(i) <= e));
+    hi = min(hi, lo + k * step);
+    lo += (k - 1) * step;
+  }
+  return lo;
+}
+
+// x as FP64 by integer instructions (the conversion instruction would take the
+// FP64 pipe as long as the addition that follows)
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
+  const int sh = m < 0x00800000u ? __clz(m) - 8 : 0;   // subnormal: to the leading one
+  const uint32_t mm = m << sh;
+  uint32_t hi = (mm >> 3) + ((896u - sh) << 20);
+  hi += m >= 0x7F800000u ? 0x38000000u : 0u;            // infinities, NaN
+  return __hiloint2double((int)((m ? hi : 0u) | (u & 0x80000000u)), (int)(mm << 29));
+}
+
 // ---------------------------------------------------------------- split-K sum
 // one thread per output element; the slots are summed in FP64 with eight
 // interleaved partial sums combined in a fixed order (deterministic).  The
 // eight loads of a round are independent, so a long slot list is not a
-// chain of dependent memory latencies.
+// chain of dependent memory latencies; a warp finds the task of its first
+// element together.  Bound by the FP64 pipe, one addition a value: a conversion
+// costs it as much, and one that is predicated off does too, hence widen and
+// the loop exits.  CAS(20,20) M=1024, 227 slots of 1.1 M elements at most: 573
+// -> 310 us; CAS(16,16) M=512, 137 of 0.29 M: 108 -> 71 us.  (One block per
+// column with a warp for every eighth slot: 660 us, lanes past the tile's rows
+// take the pipe too.)
 __global__ void tc_reduce_kernel(const TcRed* __restrict__ tasks, int ntasks, int64_t total,
                                  const float* __restrict__ part, double* __restrict__ out) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = ntasks - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (tasks[mid].e0 <= e) lo = mid; else hi = mid - 1;
-    }
+  const int lane = threadIdx.x & 31;
+  for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; e0 < total;
+       e0 += (int64_t)gridDim.x * blockDim.x) {
+    int lo = warp_find(ntasks, e0, [&](int i) { return tasks[i].e0; });
+    const int64_t e = e0 + lane;
+    if (e >= total) break;
+    while (lo + 1 < ntasks && tasks[lo + 1].e0 <= e) ++lo;
     const TcRed R = tasks[lo];
     const int loc = (int)(e - R.e0);
     const int j = loc / R.m_valid, i = loc - j * R.m_valid;
@@ -446,9 +479,13 @@ __global__ void tc_reduce_kernel(const TcRed* __restrict__ tasks, int ntasks, in
 #pragma unroll
       for (int u = 0; u < 8; ++u) v[u] = p[(s + u) * ss];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) a[u] += (double)v[u];
+      for (int u = 0; u < 8; ++u) a[u] += widen(v[u]);
     }
-    for (int u = 0; s < R.nslot; ++s, ++u) a[u] += (double)p[s * ss];
+#pragma unroll
+    for (int u = 0; u < 7; ++u) {   // the rest, as one round (no indexed array)
+      if (s + u >= R.nslot) break;
+      a[u] += widen(p[(s + u) * ss]);
+    }
     out[R.out + (int64_t)j * R.ld + R.m0 + i] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
   }
 }
@@ -574,22 +611,31 @@ __global__ void __launch_bounds__(256) tc_convert_kernel(const TcConv* __restric
 
 __global__ void tc_convert_psi_kernel(const double* __restrict__ psi, const TcPsiSector* __restrict__ sec, int nsec,
                                       int64_t total, int prec, void* hi, void* lo, int64_t pitch) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    int lo_i = 0, hi_i = nsec - 1;
-    while (lo_i < hi_i) {
-      const int mid = (lo_i + hi_i + 1) >> 1;
-      if (sec[mid].src_off <= e) lo_i = mid; else hi_i = mid - 1;
-    }
-    const TcPsiSector S = sec[lo_i];
-    const int r = (int)((e - S.src_off) / S.cols);
-    const int c = (int)((e - S.src_off) % S.cols);
-    int s = 0, t = 0;
+  const int lane = threadIdx.x & 31;
+  for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; e0 < total;
+       e0 += (int64_t)gridDim.x * blockDim.x) {
+    int si = warp_find(nsec, e0, [&](int i) { return sec[i].src_off; });
+    const int64_t e = e0 + lane;
+    if (e >= total) break;
+    while (si + 1 < nsec && sec[si + 1].src_off <= e) ++si;
+    const TcPsiSector S = sec[si];
+    const int64_t el = e - S.src_off;
+    // (a sector of 2^32 elements and more would need the long division)
+    const int r = el >> 32 ? (int)(el / S.cols) : (int)((uint32_t)el / (uint32_t)S.cols);
+    const int c = (int)(el - (int64_t)r * S.cols);
+    int cp = S.cpad[0], cb = S.cbreak[0], rp = S.rpad[0], rb = S.rbreak[0];
+#pragma unroll
     for (int u = 1; u < 4; ++u) {
-      if (c >= S.cbreak[u]) s = u;
-      if (r >= S.rbreak[u]) t = u;
+      if (c >= S.cbreak[u]) {
+        cp = S.cpad[u];
+        cb = S.cbreak[u];
+      }
+      if (r >= S.rbreak[u]) {
+        rp = S.rpad[u];
+        rb = S.rbreak[u];
+      }
     }
-    const int64_t prow = S.r0 + S.rpad[t] + (r - S.rbreak[t]);
-    store_conv(psi[e], prec, hi, lo, prow * pitch + S.cpad[s] + (c - S.cbreak[s]));
+    store_conv(psi[e], prec, hi, lo, ((int64_t)S.r0 + rp + (r - rb)) * pitch + cp + (c - cb));
   }
 }
 
