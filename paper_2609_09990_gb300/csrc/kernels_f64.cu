@@ -205,8 +205,11 @@ gemm_f64_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ 
 // every element is still summed over its terms in list order.  Bound by the
 // FP64 pipe (93 % busy), so a warp adds only the vectors of a chunk that it has
 // elements of: sector blocks of about 1200 elements filled 58 % of their
-// chunks (CAS(16,16) M=512, right and left operators: 3.80 + 0.51 ms with
-// whole chunks, 2.01 + 0.29 ms now, 8.7 GB of terms).
+// chunks (CAS(16,16) M=512, right and left operators, 8.7 GB of terms: 4.31 ms
+// with whole chunks, 2.31 ms so).  A CTA per chunk, so that the device deals
+// them out: dealt in turn to 8 CTAs an SM, whose chunks have 1 to hundreds of
+// terms, the busiest SM worked 1.4 times as long as the idlest (1.89 ms now;
+// CAS(20,20) M=1024 17.8 -> 15.5 ms).
 constexpr int kAxpyThreads = 256;
 constexpr int kAxpyStage = 256;   // term descriptors staged per round
 __global__ void __launch_bounds__(kAxpyThreads) axpy_kernel(const AxpyTerm* __restrict__ terms,
@@ -218,10 +221,13 @@ __global__ void __launch_bounds__(kAxpyThreads) axpy_kernel(const AxpyTerm* __re
   __shared__ const double* sp[kAxpyStage];
   __shared__ double sc[kAxpyStage];
   for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    int lo = 0, hi = nouts - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (cstart[mid] <= c) lo = mid; else hi = mid - 1;
+    // the output of this chunk: 32 probes of the list a round
+    int lo = 0;
+    for (int hi = nouts; hi - lo > 1;) {
+      const int step = (hi - lo + 31) >> 5, at = lo + (int)(threadIdx.x & 31) * step;
+      const int below = __popc(__ballot_sync(0xffffffffu, at < hi && cstart[at] <= c));
+      hi = min(hi, lo + below * step);
+      lo += (below - 1) * step;
     }
     const AxpyOut o = outs[lo];
     const int64_t e0 = (c - cstart[lo]) * kAxpyChunk + threadIdx.x;
@@ -576,7 +582,7 @@ void launch_gather(const GatherTask* tasks, int ntasks, cudaStream_t s) {
 void launch_axpy(const AxpyPlan& p, cudaStream_t s) {
   const int no = (int)p.outs.size();
   if (no == 0 || p.nchunks == 0) return;
-  const int64_t grid = p.nchunks < 152 * 8 ? p.nchunks : 152 * 8;
+  const int64_t grid = p.nchunks < INT32_MAX ? p.nchunks : INT32_MAX;
   axpy_kernel<<<(int)grid, kAxpyThreads, 0, s>>>(p.d_terms, p.d_outs, p.d_cstart, no, p.nchunks);
 }
 
