@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(256) split_operands_kernel(const SplitOperand*
     int E = zero ? 1023 : (int)(mx >> 20) + 1;   // all |x| < 2^(E - 1023)
     if (mx < (700u << 20) ? (mx != 0 || any != 0) : mx >= (1300u << 20)) E = kBadExp;
     const int sh0 = zero ? 5000 : (int)(mx >> 20) + 8;   // right shift of the left-aligned mantissa: sh0 - exponent
-    const uint64_t bias = 2 * 0x0080808080808080ull + 1;
+    const uint64_t bias = 0x0080808080808080ull;
     const int tile = row / XM, trow = row - tile * XM, rt = min(XM, rp - tile * XM);
     const int plane = rt * nh * 32;
     // chunks before this one are full: rp rows of 7 x 64 + 4 bytes
@@ -233,7 +233,8 @@ __global__ void __launch_bounds__(256) split_operands_kernel(const SplitOperand*
           uint64_t t;   // 2 |x| in units of the last digit; 0 for shifts of 64 and more
           asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(m), "r"(s));
           const int64_t sg = (int64_t)((int32_t)xh >> 31);
-          const uint64_t q = (uint64_t)((int64_t)((t ^ (uint64_t)sg) - (uint64_t)sg + bias)) >> 1;
+          const uint64_t r = (t + 1) >> 1;   // to nearest, before the sign: either sign rounds alike
+          const uint64_t q = (r ^ (uint64_t)sg) - (uint64_t)sg + bias;
           wl[u] = (uint32_t)q;
           wh[u] = (uint32_t)(q >> 32);
         }
