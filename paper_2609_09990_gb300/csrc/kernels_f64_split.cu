@@ -50,6 +50,7 @@
 #include <cuda_fp16.h>
 
 #include "gbd_internal.h"
+#include "smem_limit.h"
 
 namespace gbd {
 
@@ -484,9 +485,7 @@ split_sum_kernel(const GemmOut* __restrict__ outs, const SplitSum* __restrict__ 
 int launch_gemm_f64_split(const GemmPlan& p, int num_sms, int* err, cudaStream_t s) {
   const int n = (int)p.swork.size();
   if (n == 0) return 0;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(gemm_f64_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  if (attr != cudaSuccess) return -1;
+  if (!allow_shared_memory(gemm_f64_split_kernel, kSmem)) return -1;
   const int64_t blocks = (p.split_items + 7) / 8;
   split_operands_kernel<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, s>>>(
       p.d_operands, (int)p.operands.size(), p.split_items, p.d_digits, err + 1);

@@ -27,11 +27,10 @@
 // Per sigma: CAS(16,16) M=512 12.9 -> 9.1 ms for 38 launches, CAS(20,20)
 // M=1024 58.8 -> 45.2 ms for 40, a full solve of CAS(10,10) 19.5 -> 13.2 ms
 // for 634.  Now stage A waits for its boxes (two stages of 96 KB at N = 256).
-#include <mutex>
-
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "smem_limit.h"
 #include "tc_gemm.h"
 
 namespace gbd {
@@ -675,10 +674,7 @@ bool launch_tc_gemm(const TcMaps& maps, const TcLaunch& L, int num_sms, cudaStre
   static const Kernel kernels[4] = {tc_gemm_kernel<true, false>, tc_gemm_kernel<false, false>,
                                     tc_gemm_kernel<false, true>, tc_gemm_kernel<true, true>};   // by TcPrec
   if (L.prec < 0 || L.prec > 3) return false;
-  static std::once_flag attr_once;   // engines on several host threads share the kernels
-  std::call_once(attr_once, []() {
-    for (Kernel k : kernels) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-  });
+  if (!allow_shared_memory(kernels[L.prec], kSmemBudget)) return false;
   const int grid = L.ntiles < num_sms ? L.ntiles : num_sms;
   kernels[L.prec]<<<grid, kThreads, smem, s>>>(maps, L);
   return true;
