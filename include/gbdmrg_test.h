@@ -320,6 +320,12 @@ int gbd_gemm_f64(gbd_ctx *ctx, int32_t M, int32_t N, int32_t K, int32_t nterms, 
  * returns with *err_flag = 1, *waited_ok = 0; arrive = 1: *err_flag = 0,
  * *waited_ok = 1. */
 int gbd_wait_selftest(int32_t device, int32_t arrive, int32_t *err_flag, int32_t *waited_ok);
+/* How a wait that ran out is reported, without one: raises the context's flag
+ * (sigma 1: the tensor-core sigma's, 0: the one of the other tensor-core
+ * GEMMs) as the kernels do, and synchronises.  Returns GBD_ERR_TIMEOUT; the
+ * flag is taken down, so that the context's next calls succeed.  GBD_ERR_ARG
+ * for another sigma. */
+int gbd_wait_flag_selftest(gbd_ctx *ctx, int32_t sigma);
 /* Preconditioner network pieces for gradient checks: install FP32 weights
  * (kept FP16 on the device for inference); loss sum w (g-y)^2 / sum w +
  * lam mean(g^2) and its gradient over n feature rows X [n*8] with targets y

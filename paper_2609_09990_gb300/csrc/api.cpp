@@ -483,6 +483,15 @@ int gbd_gemm_tc_selftest(gbd_ctx* ctx, int32_t M, int32_t N, int32_t K, int32_t 
   });
 }
 
+int gbd_wait_flag_selftest(gbd_ctx* ctx, int32_t sigma) {
+  return guarded(ctx, [&]() {
+    if (sigma != 0 && sigma != 1) return fail(ctx, GBD_ERR_ARG, "sigma must be 0 or 1");
+    if (!ctx->eng) ctx->eng.reset(new gbd::Engine(ctx->device));
+    ctx->eng->wait_flag_selftest(sigma == 1);
+    return GBD_OK;
+  });
+}
+
 int gbd_gemm_f64(gbd_ctx* ctx, int32_t M, int32_t N, int32_t K, int32_t nterms, int32_t flags, double alpha,
                  int32_t beta, const double* A, const double* B, double* C) {
   return guarded(ctx, [&]() {

@@ -455,7 +455,10 @@ void Engine::drain_timers() {
     wait_pending = false;
     int flag = 0;
     CK(cudaMemcpy(&flag, d_wait_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (flag) throw Error(-5, "grouped GEMM on the tensor cores: a bounded device wait ran out");
+    if (flag) {   // reported once: the context's next call starts without it
+      CK(cudaMemsetAsync(d_wait_err, 0, sizeof(int), stream));
+      throw Error(-5, "grouped GEMM on the tensor cores: a bounded device wait ran out");
+    }
   }
   for (auto& t : env_timers) {
     float ms = 0;
@@ -1603,6 +1606,8 @@ void Engine::sigma_run(Sigma& sg) {
     run(sg.B);
   });
   CK(cudaEventRecord(ev1, stream));
+  // a replay does not pass through run()
+  if (!sg.A.swork.empty() || !sg.B.swork.empty()) wait_pending = true;
   sigma_pending = 1;
   stats.sigma_flops += sg.A.flops + sg.B.flops;
   stats.n_sigma++;
@@ -1968,6 +1973,23 @@ double Engine::davidson(const SigmaOp& op, const double* diag, double tol, int m
   return theta;
 }
 
+// leaves the flags as kernels whose bounded waits ran out leave them, then
+// synchronises as the calls do (sigma: the flag of a tensor-core sigma, else
+// the one that the grouped GEMMs share)
+void Engine::wait_flag_selftest(bool sigma) {
+  if (sigma) {
+    for (cudaEvent_t e : {ev0, evg0, evgm, evg1, ev1}) CK(cudaEventRecord(e, stream));
+    *tc_err_host = 1;
+    sigma_pending = 2;
+    settle();
+  } else {
+    const int one = 1;
+    CK(cudaMemcpyAsync(wait_flag(), &one, sizeof(int), cudaMemcpyHostToDevice, stream));
+    wait_pending = true;
+    sync();
+  }
+}
+
 // account the sigma build recorded by the last sigma()/tc_apply() once the
 // stream has passed it
 void Engine::settle() {
@@ -1986,7 +2008,11 @@ void Engine::settle() {
     stats.tc_gemm_ms_st[1] += g - ga;
     stats.tc_gemm_ms += g;
     stats.tc_gemm_ms_p[stats.last_tc_prec] += g;
-    if (*tc_err_host) throw Error(-5, "tensor-core sigma: a bounded device wait ran out");
+    if (*tc_err_host) {   // reported once; the plan that holds the device's flag is not used again
+      *tc_err_host = 0;
+      sigma_pending = 0;
+      throw Error(-5, "tensor-core sigma: a bounded device wait ran out");
+    }
   }
   sigma_pending = 0;
 }

@@ -502,6 +502,7 @@ class Engine {
   void probe_step(int k, int precision, int refine, double tol, double* theta, double* e64, double* r64);
   void gemm_tc_selftest(int M, int N, int K, int nterms, int flags, int prec, uint64_t seed, double* max_err,
                         double* max_ref);
+  void wait_flag_selftest(bool sigma);
   void gemm_f64_host(int M, int N, int K, int nterms, int flags, double alpha, int beta, const double* A,
                      const double* B, double* C);
   // the inner-PCG correction of the Davidson solver at centre k with the

@@ -104,6 +104,7 @@ def lib():
         "gbd_set_env_precision": (C.c_int, [vp, C.c_int32]),
         "gbd_gemm_tc_selftest": (C.c_int, [vp, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32,
                                            C.c_uint64, _dp, _dp]),
+        "gbd_wait_flag_selftest": (C.c_int, [vp, C.c_int32]),
         "gbd_gemm_f64": (C.c_int, [vp, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_double, C.c_int32,
                                    _dp, _dp, _dp]),
         "gbd_set_preconditioner": (C.c_int, [vp, C.c_int32]),
@@ -389,6 +390,9 @@ class Context:
         self._check(self.L.gbd_gemm_tc_selftest(self.ptr, M, N, K, nterms, flags, prec, seed, C.byref(e),
                                                 C.byref(r)), "gbd_gemm_tc_selftest")
         return e.value, r.value
+
+    def wait_flag_selftest(self, sigma):
+        self._check(self.L.gbd_wait_flag_selftest(self.ptr, int(sigma)), "gbd_wait_flag_selftest")
 
     def gemm_f64(self, A, B, flags=0, alpha=1.0, C0=None):
         """C0 + alpha sum_t op(A[t]) op(B[t]) by the FP64 grouped GEMM (flags 1: A[t] is K x M, 2: B[t] is N x K,
