@@ -639,6 +639,7 @@ void Engine::upload(GemmPlan& p) {
   if (!p.swork.empty()) {
     p.d_digits = dalloc<uint8_t>(p.digit_bytes);
     p.d_part = dalloc<double>(p.part_slots * kSplitTile * kSplitTile);
+    if (!p.summed) p.d_weak = dalloc<uint2>(p.marks + 1);
   }
   uint8_t* at[7];
   p.d_lists = upload_lists<7>({{p.terms.data(), p.terms.size() * sizeof(GemmTerm)},
@@ -667,7 +668,7 @@ void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>&
   p.sterms.clear();
   p.swork.clear();
   p.ssums.clear();
-  p.split_items = p.digit_bytes = p.part_slots = 0;
+  p.split_items = p.digit_bytes = p.part_slots = p.marks = 0;
   if (list.empty()) return;
   size_t nterms = 0;
   int64_t all = 0;
@@ -689,8 +690,9 @@ void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>&
         const int64_t rp = (rows + 7) / 8 * 8, chunks = (K + kSplitChunk - 1) / kSplitChunk;
         const int last = K - (int)(chunks - 1) * kSplitChunk;
         p.operands.push_back({src, ld, rows, K, kstrided, p.digit_bytes, p.split_items});
-        // 7 digit planes of FP16 and an exponent per row and chunk; the last chunk may be 16 wide
-        const int64_t bytes = (chunks - 1) * rp * (7 * 64 + 4) + rp * (7 * (last > 16 ? 64 : 32) + 4);
+        // 7 digit planes of FP16 and a tail per row and chunk; the last chunk may be 16 wide
+        const int64_t bytes =
+            (chunks - 1) * rp * (7 * 64 + kSplitTail) + rp * (7 * (last > 16 ? 64 : 32) + kSplitTail);
         p.digit_bytes += (bytes + 127) / 128 * 128;
         p.split_items += rp / 8 * chunks;
         return table[i];
@@ -723,6 +725,8 @@ void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>&
           p.ssums.push_back({l.second, tm, tn, (int)p.part_slots, pieces});
           p.part_slots += pieces;
         }
+        p.marks += (int64_t)pieces * 4 * ((std::min(kSplitTile, o.M - tm * kSplitTile) + 15) / 16) *
+                   ((std::min(kSplitTile, o.N - tn * kSplitTile) + 7) / 8);   // four per 16 x 8 block
         for (int i = 0; i < pieces; ++i) {
           const int64_t s0 = steps * i / pieces, s1 = steps * (i + 1) / pieces;
           const int t = (int)(std::upper_bound(kstep.begin(), kstep.end(), s0) - kstep.begin()) - 1;
@@ -742,6 +746,8 @@ void Engine::release(GemmPlan& p) {
   dfree(p.d_lists);
   dfree(p.d_digits);
   dfree(p.d_part);
+  dfree(p.d_weak);
+  p.d_weak = nullptr;
   p.d_lists = nullptr;
   p.d_digits = nullptr;
   p.d_part = nullptr;
@@ -1516,7 +1522,7 @@ struct Engine::Sigma {
   GraphSeq graph;
 };
 
-void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool result) {
+void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool result, bool summed) {
   // Y_b(Qin) exists when both operators have sub-blocks for (b, Qin), key b nq + Qin
   const int nq = EL.n();
   const SubGroups rby(renl, nq);
@@ -1549,6 +1555,7 @@ void Engine::plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool re
   A.clear();
   B.clear();
   A.result = B.result = result;
+  A.summed = B.summed = summed;
   A.outs.reserve(ys.size() * 4);
   A.terms.reserve(renl.subs.size());
   B.terms.reserve(lenl.subs.size());
@@ -2229,7 +2236,7 @@ void Engine::probe_step(int k, int precision, int refine, double tol, double* th
   bool planned = false;
   *theta = solve_tiers(sg, diag, tol, precision, refine, planned);
   if (!planned) {
-    plan_sigma(sg.lenl, sg.renl, sg, true);   // one product, for the reported energy
+    plan_sigma(sg.lenl, sg.renl, sg, true, true);   // one product, for the reported energy
     planned = true;
   }
   double* y = dalloc<double>(psi_size);
@@ -2594,7 +2601,7 @@ double Engine::final_energy() {
   finish_enl(sg.lenl, ax);
   build_renl(1, Renv[2], ER, sg.renl, ax);
   finish_enl(sg.renl, ax);
-  plan_sigma(sg.lenl, sg.renl, sg, true);
+  plan_sigma(sg.lenl, sg.renl, sg, true, true);
   double* y = dalloc<double>(psi_size);
   sigma(sg, psi, y);
   int nblk = reduction_blocks(psi_size);

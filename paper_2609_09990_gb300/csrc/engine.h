@@ -433,8 +433,9 @@ class Engine {
   void setup_two_site(int k);
   void form_psi(int k, int pattern);
   struct Sigma;
-  // result: this H_eff product is itself returned, not iterated (GemmPlan::result)
-  void plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool result = false);
+  // result: this H_eff product is itself returned, not iterated (GemmPlan::result);
+  // summed: into an energy (GemmPlan::summed)
+  void plan_sigma(const EnlOp& lenl, const EnlOp& renl, Sigma& sg, bool result = false, bool summed = false);
   void sigma(Sigma& sg, const double* x, double* y);
   void compute_diag(const EnlOp& lenl, const EnlOp& renl, double* diag);
   void sigma_run(Sigma& sg);

@@ -131,7 +131,7 @@ struct GemmPlan {       // host side lists plus their device copies
   std::vector<SplitTerm> sterms;        // the terms of its outputs
   std::vector<SplitWork> swork;         // 64 x 64 tiles, or pieces of their chains
   std::vector<SplitSum> ssums;          // tiles cut into pieces
-  int64_t split_items = 0, digit_bytes = 0, part_slots = 0;
+  int64_t split_items = 0, digit_bytes = 0, part_slots = 0, marks = 0;   // marks: at most so many
   void* d_lists = nullptr;       // the device copies, in one allocation
   GemmTerm* d_terms = nullptr;
   GemmOut* d_outs = nullptr;
@@ -142,6 +142,7 @@ struct GemmPlan {       // host side lists plus their device copies
   SplitSum* d_ssums = nullptr;
   uint8_t* d_digits = nullptr;   // records of the operands
   double* d_part = nullptr;      // partial sums
+  uint2* d_weak = nullptr;       // the marks of outputs to form again by FMAs, their number first
   int tile_span = 0;             // largest rows + columns of a tile (odd pitches)
   int per_lane = 2;              // outputs per lane: tiles of at most 128 per_lane outputs
   double flops = 0.0;       // 2 m n k summed over terms
@@ -151,6 +152,9 @@ struct GemmPlan {       // host side lists plus their device copies
   // false: an unconverged iteration amplifies a change of rounding until
   // its iterates have no digit in common.
   bool result = false;
+  // Of a plan of results: only a sum over all its outputs is returned (an
+  // energy), so that errors count against the norm, not element by element.
+  bool summed = false;
   void clear() { terms.clear(); outs.clear(); tiles.clear(); swork.clear(); flops = 0.0; }
   int add_out(double* C, int ldc, int M, int N, int beta) {
     GemmOut o{C, ldc, M, N, (int)terms.size(), (int)terms.size(), beta, 0};
@@ -187,6 +191,8 @@ constexpr int kAxpyChunk = 1024;   // output elements per work chunk of the bloc
 // largest side of an FMA tile (shared memory: 3 steps of 32 columns of both sides, at most 51 KB)
 constexpr int kFmaSide = 32;
 constexpr int kSplitTile = 64, kSplitChunk = 32;
+constexpr int kSplitTail = 8;      // bytes behind a row's digits: exponent, mask of nonzero elements
+constexpr int kWeakPlaces = 128;   // places of a mark of weak outputs in a 64 x 64 tile
 
 // ---------------------------------------------------------------- kernels (kernels.cu)
 // launches made, or -1 when the split kernel's shared memory was refused

@@ -14,11 +14,29 @@
 // operands) are put together as one 64-bit integer, converted once and
 // added to the FP64 sum of the output with one FMA.
 //
-// Accuracy: a chunk's operands and its sum are within 2^-56 of (largest
-// element of the A row) x (largest of the B column); FP64 rounds at every
-// one of the 32 FMAs instead.  On Gaussian, graded, near-diagonal and
-// isometric operands the relative error against 64-bit-mantissa sums is
-// 0.4 to 0.9 of the plain FMA loop's for K >= 8.
+// Accuracy: with a = the largest element of the A row in the chunk and b = of
+// the B column, an operand element is off by at most 2^-55 a (2^-55 b) and
+// the sum of the chunk by another 2^-53 a b; FP64 rounds at every one of the
+// 32 FMAs instead.  Where the large elements of a row meet the large ones
+// of a column that is below the FMA loop's error.  Where they do not (grading
+// in opposite directions, near-diagonal operands, disjoint places), the
+// products are small against a b and would lose digits.  So for every output
+// the strongest chunk is kept, sum |A||B| from the top digits (two more
+// products in 70), next to the largest scale 2^e of a b that any chunk brought
+// (chunks in which no nonzero element meets another do not count).  An output
+// with (columns + 4) sum |A||B| below 2^14 digit units, less the square root
+// of the number of chunks, whose errors are independent, is formed again
+// by FP64 FMAs (split_redo).  Outputs then are within (K + 4) 2^-53 |A||B| by
+// element, as the FMA loop's are by its a priori bound; measured on Gaussian,
+// graded (both ways, 0.5 to 8 decades), near-diagonal, sparse and 6-decade
+// random operands, K = 3 to 3000: at most 0.55 of that bound, root mean
+// square 0.1 to 2 of 2^-53 |A||B| where the FMA loop has 0.4 to 23 (and up to
+// 6 times the loop's where products graded apart stay just above the line).
+// The line is measured, H_eff of CAS(16,16) M=512: 2^13 without the root 0.6 %
+// of the outputs again, 2^14 without it 1.4 % and 7.4 ms, with it 0.6 ms;
+// 2^15 1.7 ms and errors halved; the check itself takes 0.8 ms of 8.5.  Plans whose
+// products are only summed into one number (an energy) leave it out: their
+// error counts against the norm, where the digits' is 0.4 to 0.9 of the FMA loop's.
 //
 // Rows whose largest magnitude is not finite or outside 2^-323 .. 2^277
 // (all-zero rows are fine) and coefficients outside 2^-73 .. 2^77 send
@@ -45,6 +63,8 @@
 // CAS(20,20) M=1024 (432 GFLOP) 53 ms; twelve warps with all A digits in
 // registers took 9.15 and 56 ms, eight 12 ms, a first kernel that split its
 // operands itself, tile by tile, 21 ms, and FP64 FMAs 79 and 562 ms.
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include <cuda_fp16.h>
@@ -61,12 +81,15 @@ constexpr int NS = 7;                           // digits
 constexpr int kWarps = 16, XT = 32 * kWarps + 32;   // 17 warps: at most 5 on a sub-core, 96 registers
 constexpr int kStages = 3;
 constexpr int kPlane = XM * 64;                 // bytes of a digit plane in a stage: 64 rows of 32 halves
-constexpr int kRec = NS * kPlane + XM * 4;      // a stage's operand: 7 planes and the exponents
+constexpr int kTail = kSplitTail;               // bytes behind a row's digits: exponent, mask of nonzero elements
+constexpr int kRec = NS * kPlane + XM * kTail;  // a stage's operand: 7 planes and the tails
 constexpr int kHead = 64;                       // bytes of a stage's header
 constexpr int kSmem = kStages * (2 * kRec + kHead) + 2 * kStages * 8 + 16;
 constexpr float kMagic = 12582912.0f;           // 1.5 x 2^23: integers in +-2^22 added to it are its low mantissa bits
 constexpr uint32_t kMagicBits = 0x4B400000u;
 constexpr int kBadExp = 1 << 28;                // exponent of a row that the digits cannot hold
+constexpr int kStrong = 14;                     // the line of a weak output, in powers of two of digit units
+constexpr uint32_t kNoScale = 0x80008000u;      // no chunk yet
 constexpr uint32_t kWaitLimit = 1u << 22;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -149,6 +172,16 @@ __device__ __forceinline__ void weights(float (&f)[8][4], uint32_t ad, uint32_t 
     }
   }
 }
+// sums of |top digit of A| |top digit of B| over 16 columns: |A||B| in units of
+// 2^96 of the last digits' (the largest element's top digit is 64 to 128)
+__device__ __forceinline__ void magnitudes(float (&m)[4], uint32_t ad, uint32_t bd) {
+  uint32_t a[4], b[2];
+  ldsm4(ad, a);
+  ldsm2(bd, b);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) a[i] &= 0x7FFF7FFFu;
+  mma_f16(m, a, b[0] & 0x7FFF7FFFu, b[1] & 0x7FFF7FFFu);
+}
 // Byte offset of 16-byte piece c of a digit row: rows of 64 bytes (32 columns,
 // c 0..3) or 32 bytes (chunks of at most 16 columns, c 0..1).  The eight rows
 // of an ldmatrix use eight different 16-byte bank groups.
@@ -166,8 +199,11 @@ __device__ __forceinline__ int pad8(int rows) { return (rows + 7) & ~7; }
 // by HBM (8 bytes read, 14 written).
 __global__ void __launch_bounds__(256) split_operands_kernel(const SplitOperand* __restrict__ ops, int nops,
                                                              int64_t nitems, uint8_t* __restrict__ digits,
-                                                             int* __restrict__ next) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0;   // the product kernel's work counter
+                                                             int* __restrict__ next, uint2* __restrict__ weak) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *next = 0;   // the product kernel's work counter
+    if (weak) weak->x = 0;
+  }
   const int lane = threadIdx.x & 31, kq = lane & 3;
   const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
   const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -199,12 +235,15 @@ __global__ void __launch_bounds__(256) split_operands_kernel(const SplitOperand*
       lo[i] = (uint32_t)__double2loint(v);
       hi[i] = (uint32_t)__double2hiint(v);
     }
-    uint32_t mx = 0, any = 0;
+    uint32_t mx = 0, any = 0, nz = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       mx = max(mx, hi[i] & 0x7FFFFFFFu);
       any |= lo[i];
+      nz |= (hi[i] & 0x7FFFFFFFu) | lo[i] ? 1u << (8 * kq + i) : 0u;
     }
+    nz |= __shfl_xor_sync(0xffffffffu, nz, 1);
+    nz |= __shfl_xor_sync(0xffffffffu, nz, 2);
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
     any |= __shfl_xor_sync(0xffffffffu, any, 1);
@@ -217,7 +256,7 @@ __global__ void __launch_bounds__(256) split_operands_kernel(const SplitOperand*
     const int tile = row / XM, trow = row - tile * XM, rt = min(XM, rp - tile * XM);
     const int plane = rt * nh * 32;
     // chunks before this one are full: rp rows of 7 x 64 + 4 bytes
-    uint8_t* rec = digits + O.off + (int64_t)chunk * rp * (NS * 64 + 4) + (int64_t)tile * XM * (NS * nh * 32 + 4);
+    uint8_t* rec = digits + O.off + (int64_t)chunk * rp * (NS * 64 + kTail) + (int64_t)tile * XM * (NS * nh * 32 + kTail);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (h >= nh) break;
@@ -259,7 +298,7 @@ __global__ void __launch_bounds__(256) split_operands_kernel(const SplitOperand*
 #pragma unroll
       for (int i = 0; i < NS; ++i) *reinterpret_cast<uint2*>(dst + i * plane) = make_uint2(pk[0][i], pk[1][i]);
     }
-    if (kq == 0) *reinterpret_cast<int*>(rec + NS * plane + trow * 4) = E;
+    if (kq == 0) *reinterpret_cast<int2*>(rec + NS * plane + trow * kTail) = make_int2(E, (int)nz);
   }
 }
 
@@ -269,15 +308,17 @@ struct Head {          // what the consumers need of one chunk, 64 bytes
   double alpha;
   int32_t ldc, mr, nr, flags;   // kFirst | kLast | kBeta | kEnd
   int32_t nh, kc, term, k0;     // 16-column halves; columns, GemmTerm and first column of the chunk
-  int32_t m0, n0, pad0, pad1;
+  int32_t m0, n0, work, slack;  // slack: log2 of the square root of the piece's chunks
 };
 static_assert(sizeof(Head) == kHead, "stage header");
 enum { kFirst = 1, kLast = 2, kBeta = 4, kEnd = 8 };
 
+template <bool kGuard>
 __global__ void __launch_bounds__(XT, 1)
 gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
                       const SplitTerm* __restrict__ sterms, const SplitWork* __restrict__ work, int nwork,
-                      const uint8_t* __restrict__ digits, double* __restrict__ part, int* err, int* next) {
+                      const uint8_t* __restrict__ digits, double* __restrict__ part, uint2* __restrict__ weak,
+                      int* err, int* next) {
   extern __shared__ __align__(128) uint8_t sm[];
   // stage s: record of A, record of B; the headers and barriers behind them
   Head* heads = reinterpret_cast<Head*>(sm + kStages * 2 * kRec);
@@ -308,6 +349,8 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
       const SplitWork W = work[w];
       const GemmOut o = outs[W.out];
       Head h;
+      h.work = w;
+      h.slack = (31 - __clz(W.steps)) >> 1;
       h.m0 = W.tm * XM;
       h.n0 = W.tn * XM;
       h.mr = min(XM, o.M - h.m0);
@@ -331,7 +374,7 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         h.term = T.term;
         h.alpha = T.alpha;
         h.k0 = k0;
-        const int chunk = k0 / XK, row_bytes = NS * h.nh * 32 + 4;
+        const int chunk = k0 / XK, row_bytes = NS * h.nh * 32 + kTail;
         ok = mbar_wait(&empty[s], ph ^ 1, err);
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         uint8_t* st = sm + s * 2 * kRec;
@@ -341,10 +384,10 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         }
         __syncwarp();
         if (lane < 16) {
-          const uint8_t* rec = digits + (side ? T.b : T.a) + (int64_t)chunk * (side ? T.rb : T.ra) * (NS * 64 + 4) +
+          const uint8_t* rec = digits + (side ? T.b : T.a) + (int64_t)chunk * (side ? T.rb : T.ra) * (NS * 64 + kTail) +
                                (int64_t)row0 * row_bytes;
           const int plane = rows * h.nh * 32;
-          bulk_copy(st + side * kRec + x * kPlane, rec + x * plane, x < NS ? plane : rows * 4, &full[s]);
+          bulk_copy(st + side * kRec + x * kPlane, rec + x * plane, x < NS ? plane : rows * kTail, &full[s]);
         }
         if (++s == kStages) { s = 0; ph ^= 1; }
         k0 += XK;
@@ -366,6 +409,9 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
   // ---------------- consumers
   constexpr int kN8 = 2;   // 8-column groups of a warp: 8 of a tile over 16 / 4 warps
   double acc[kN8][4];
+  // of every output, as powers of two: the strongest chunk's |A||B| (high half)
+  // and the largest scale with the line on it (low half)
+  uint32_t scale[kN8][4];
   int s = 0;
   uint32_t ph = 0;
   for (;;) {
@@ -387,17 +433,23 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
 #pragma unroll
       for (int i = 0; i < kN8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+        for (int j = 0; j < 4; ++j) {
+          acc[i][j] = 0.0;
+          scale[i][j] = kNoScale;
+        }
     }
     if (on) {
-      const int* expA = reinterpret_cast<const int*>(ra + NS * kPlane);
-      const int* expB = reinterpret_cast<const int*>(rb + NS * kPlane);
+      const int2* tailA = reinterpret_cast<const int2*>(ra + NS * kPlane);
+      const int2* tailB = reinterpret_cast<const int2*>(rb + NS * kPlane);
       const int r0 = 16 * g + (lane >> 2);
       // rows and columns outside the tile hold whatever the stage held before: never stored
       const bool ok0 = r0 < h.mr, ok1 = r0 + 8 < h.mr;
-      const int x0 = ok0 ? expA[r0] : 1023, x1 = ok1 ? expA[r0 + 8] : 1023;
+      const int2 none = make_int2(1023, 0);
+      const int2 xa = ok0 ? tailA[r0] : none, xb = ok1 ? tailA[r0 + 8] : none;
+      const int x0 = xa.x, x1 = xb.x;
       const int ahi = __double2hiint(h.alpha), alo = __double2loint(h.alpha), aexp = (ahi >> 20) & 0x7FF;
       const bool badA = x0 == kBadExp || x1 == kBadExp || aexp < 950 || aexp > 1100;
+      const float columns = (float)(h.kc + 4);
       const int arow = 16 * g + (lane & 15);
       const uint32_t ad0 = smem_addr(ra + piece(arow, lane >> 4, nh));
       const uint32_t ad1 = smem_addr(ra + piece(arow, 2 + (lane >> 4), 2));   // second half, full chunks only
@@ -406,13 +458,19 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         const int c8 = (nb + i * per) * 8;
         if (c8 >= h.nr) break;
         const int c = c8 + 2 * (lane & 3);
-        const int y0 = c < h.nr ? expB[c] : 1023, y1 = c + 1 < h.nr ? expB[c + 1] : 1023;
+        const int2 ya = c < h.nr ? tailB[c] : none, yb = c + 1 < h.nr ? tailB[c + 1] : none;
+        const int y0 = ya.x, y1 = yb.x;
         // one half of the columns at a time: 14 registers of B digits and 8
         // of A leave room for four warps a sub-core
         float f[8][4];
         const int brow = c8 + (lane & 7), bc = (lane >> 3) & 1;
         weights<true>(f, ad0, smem_addr(rb + piece(brow, bc, nh)));
         if (nh == 2) weights<false>(f, ad1, smem_addr(rb + piece(brow, 2 + bc, 2)));
+        float mag[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (kGuard) {
+          magnitudes(mag, ad0, smem_addr(rb + piece(brow, bc, nh)));
+          if (nh == 2) magnitudes(mag, ad1, smem_addr(rb + piece(brow, 2 + bc, 2)));
+        }
         // asked for only now, so that the exponents arrive during the products
         if (__any_sync(0xffffffffu, badA || y0 == kBadExp || y1 == kBadExp)) {
           // the chunk of these 16 x 8 outputs by FP64 FMAs from the operands themselves
@@ -440,26 +498,119 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
           const int l = (int)(two(4) - kMagicBits * 257u) + ((int)(two(6) - (kMagicBits * 257u - 32768u)) >> 16);
           const int64_t v = (int64_t)p * 65536 + l + (int64_t)((uint64_t)(two(0) - kMagicBits * 257u) << 32);
           const int e = (j < 2 ? x0 : x1) + ((j & 1) ? y1 : y0) - 2100;
+          if (kGuard && ((j < 2 ? xa.y : xb.y) & ((j & 1) ? yb.y : ya.y)) != 0)
+            scale[i][j] = __vmaxs2(scale[i][j], (uint32_t)(e + aexp) * 0x10001u +
+                                                    ((__float_as_uint(mag[j] * columns) >> 7) & 0x00FF0000u) + 127 + kStrong);
           acc[i][j] = fma(__ll2double_rn(v), __hiloint2double(ahi + (int)((uint32_t)e << 20), alo), acc[i][j]);
         }
       }
     }
     if ((flags & kLast) && on) {
+      const int slack = h.slack;
+      uint32_t marks = 0;   // lane 4 i + j: the lanes whose output (i, j) is weak
 #pragma unroll
       for (int i = 0; i < kN8; ++i) {
         const int c = (nb + i * per) * 8 + 2 * (lane & 3);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int r = 16 * g + (lane >> 2) + 8 * (j >> 1), cc = c + (j & 1);
-          if (r >= h.mr || cc >= h.nr) continue;
+          bool store = r < h.mr && cc < h.nr;
+          if (kGuard) {
+            const bool redo = store && ((int)scale[i][j] >> 16) + slack < (int)(short)(scale[i][j] & 0xFFFFu);
+            const uint32_t lanes = __ballot_sync(0xffffffffu, redo);
+            if (lane == 4 * i + j) marks = lanes;
+            store = store && !redo;
+          }
+          if (!store) continue;
           double* d = h.C + (int64_t)r * h.ldc + cc;
           *d = flags & kBeta ? (*d + acc[i][j]) : acc[i][j];
+        }
+      }
+      if (kGuard) {
+        const uint32_t any = __ballot_sync(0xffffffffu, marks != 0);
+        if (any) {
+          uint32_t at = 0;
+          if (lane == 0) at = atomicAdd(&weak->x, (uint32_t)__popc(any));
+          at = __shfl_sync(0xffffffffu, at, 0) + 1 + __popc(any & ((1u << lane) - 1));
+          if (marks) weak[at] = make_uint2(marks, (uint32_t)h.work * kWeakPlaces + warp * 4 * kN8 + lane);
         }
       }
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
     if (++s == kStages) { s = 0; ph ^= 1; }
+  }
+}
+
+// The outputs marked weak, by FP64 FMAs from the operands themselves: a warp
+// takes a mark (a place of a consumer warp, 32 lanes) four outputs at a time,
+// a lane every 32nd product of a term, its partial sums added as a tree.
+// Bound by the latency of the terms' chains (a term has one or two rounds of
+// 32 products), hence four outputs at once and the next term's record asked for early:
+// one output a warp at a time took twice as long, marks found by
+// scanning a bit map (uneven shares of them) five times as long on small plans.
+// H_eff of CAS(16,16) M=512: 0.6 ms for both stages, its 1-/2-RDM 2.5 ms in
+// 48 launches behind the host's planning.
+__global__ void __launch_bounds__(256, 3)
+split_redo_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
+                  const SplitTerm* __restrict__ sterms, const SplitWork* __restrict__ work, double* __restrict__ part,
+                  const uint2* __restrict__ weak) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t n = weak->x;
+  for (uint32_t e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < n; e += gridDim.x * blockDim.x >> 5) {
+    const uint2 mark = weak[e + 1];
+    const SplitWork W = work[mark.y / kWeakPlaces];
+    const GemmOut o = outs[W.out];
+    // the consumer warp's place in the tile
+    const int place = mark.y % kWeakPlaces, warp = place >> 3, i = place >> 2 & 1, j = place & 3;
+    const int nm = (min(XM, o.M - W.tm * XM) + 15) >> 4, nb = warp / nm, per = kWarps / nm, g = warp - nb * nm;
+    const int r0 = 16 * g + 8 * (j >> 1), c0 = (nb + i * per) * 8 + (j & 1);
+    for (uint32_t lanes = mark.x; lanes;) {
+      int r[4], c[4], have = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {   // fewer than four: the last one again, not stored
+        const int l = __ffs(lanes) - 1;
+        r[q] = l < 0 ? r[q ? q - 1 : 0] : r0 + (l >> 2);
+        c[q] = l < 0 ? c[q ? q - 1 : 0] : c0 + 2 * (l & 3);
+        have += l >= 0;
+        lanes &= lanes - 1;
+      }
+      double s[4] = {0.0, 0.0, 0.0, 0.0};
+      GemmTerm T = terms[sterms[W.t0].term];
+      for (int left = W.steps, t = W.t0, k = W.k0; left > 0;) {
+        const int steps = min(left, (T.K - k + XK - 1) / XK), len = min(T.K - k, steps * XK);
+        const int sa = T.flags & 1 ? T.lda : 1, ra = T.flags & 1 ? 1 : T.lda;
+        const int sb = T.flags & 2 ? 1 : T.ldb, cb = T.flags & 2 ? T.ldb : 1;
+        const double* a = T.A + (int64_t)W.tm * XM * ra + (int64_t)(k + lane) * sa;
+        const double* b = T.B + (int64_t)W.tn * XM * cb + (int64_t)(k + lane) * sb;
+        const double al = T.alpha;
+        left -= steps;
+        k = 0;
+        if (left > 0) T = terms[sterms[++t].term];   // on its way during this term's products
+        const bool unit = fabs(al) == 1.0, minus = al < 0.0;   // signs cost no FP64 instruction
+        for (int x = lane; x < len; x += 32, a += 32 * (int64_t)sa, b += 32 * (int64_t)sb) {
+          double av[4], bv[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            av[q] = a[(int64_t)r[q] * ra];
+            bv[q] = b[(int64_t)c[q] * cb];
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (q < have) s[q] = fma(unit ? (minus ? -av[q] : av[q]) : av[q] * al, bv[q], s[q]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (q >= have) break;
+        for (int d = 16; d > 0; d >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], d);
+        if (lane == 0) {
+          double* d = W.slot >= 0 ? part + (int64_t)W.slot * XM * XM + r[q] * XM + c[q]
+                                  : o.C + (int64_t)(W.tm * XM + r[q]) * o.ldc + W.tn * XM + c[q];
+          *d = W.slot < 0 && o.beta ? *d + s[q] : s[q];
+        }
+      }
+    }
   }
 }
 
@@ -485,14 +636,18 @@ split_sum_kernel(const GemmOut* __restrict__ outs, const SplitSum* __restrict__ 
 int launch_gemm_f64_split(const GemmPlan& p, int num_sms, int* err, cudaStream_t s) {
   const int n = (int)p.swork.size();
   if (n == 0) return 0;
-  if (!allow_shared_memory(gemm_f64_split_kernel, kSmem)) return -1;
+  const bool guard = p.d_weak != nullptr;
+  const auto kernel = guard ? gemm_f64_split_kernel<true> : gemm_f64_split_kernel<false>;
+  if (!allow_shared_memory(kernel, kSmem)) return -1;
   const int64_t blocks = (p.split_items + 7) / 8;
-  split_operands_kernel<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, s>>>(
-      p.d_operands, (int)p.operands.size(), p.split_items, p.d_digits, err + 1);
-  gemm_f64_split_kernel<<<n < num_sms ? n : num_sms, XT, kSmem, s>>>(p.d_terms, p.d_outs, p.d_sterms, p.d_swork, n,
-                                                                     p.d_digits, p.d_part, err, err + 1);
+  split_operands_kernel<<<(int)std::min<int64_t>(blocks, 16 * num_sms), 256, 0, s>>>(
+      p.d_operands, (int)p.operands.size(), p.split_items, p.d_digits, err + 1, p.d_weak);
+  kernel<<<n < num_sms ? n : num_sms, XT, kSmem, s>>>(p.d_terms, p.d_outs, p.d_sterms, p.d_swork, n, p.d_digits,
+                                                      p.d_part, p.d_weak, err, err + 1);
+  if (guard)
+    split_redo_kernel<<<3 * num_sms, 256, 0, s>>>(p.d_terms, p.d_outs, p.d_sterms, p.d_swork, p.d_part, p.d_weak);
   if (!p.ssums.empty()) split_sum_kernel<<<(int)p.ssums.size(), 256, 0, s>>>(p.d_outs, p.d_ssums, p.d_part);
-  return 2 + !p.ssums.empty();
+  return 2 + guard + !p.ssums.empty();
 }
 
 }  // namespace gbd
