@@ -718,6 +718,7 @@ void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>&
       kstep.push_back(kstep.back() + (g.K + kSplitChunk - 1) / kSplitChunk);
     }
     const int64_t steps = kstep.back();
+    const int slack = (63 - __builtin_clzll((uint64_t)std::max<int64_t>(steps, 1))) / 2;
     const int pieces = 2 * steps > 3 * piece ? (int)((steps + piece - 1) / piece) : 1;
     for (int tm = 0; tm * kSplitTile < o.M; ++tm)
       for (int tn = 0; tn * kSplitTile < o.N; ++tn) {
@@ -732,7 +733,7 @@ void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>&
           const int t = (int)(std::upper_bound(kstep.begin(), kstep.end(), s0) - kstep.begin()) - 1;
           work.push_back({s1 - s0, (int)w.size()});
           w.push_back({l.second, tm, tn, t0 + t, (int)(s0 - kstep[t]) * kSplitChunk, (int)(s1 - s0),
-                       pieces > 1 ? (int)p.part_slots - pieces + i : -1, 0});
+                       pieces > 1 ? (int)p.part_slots - pieces + i : -1, slack});
         }
       }
   }

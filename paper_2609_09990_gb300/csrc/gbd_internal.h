@@ -118,7 +118,8 @@ struct SplitTerm {
   double alpha;
 };
 struct SplitWork {       // `steps` chunks of 32 columns of one tile, from column k0 of sterm t0
-  int32_t out, tm, tn, t0, k0, steps, slot, pad;   // slot: partial sum, -1 = the output itself
+  int32_t out, tm, tn, t0, k0, steps, slot;   // slot: partial sum, -1 = the output itself
+  int32_t slack;           // log2 of the square root of the output's chunks
 };
 struct SplitSum { int32_t out, tm, tn, slot, count; };
 

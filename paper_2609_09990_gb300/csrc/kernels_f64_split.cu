@@ -25,18 +25,19 @@
 // products in 70), next to the largest scale 2^e of a b that any chunk brought
 // (chunks in which no nonzero element meets another do not count).  An output
 // with (columns + 4) sum |A||B| below 2^14 digit units, less the square root
-// of the number of chunks, whose errors are independent, is formed again
+// of the number of its chunks, whose errors are independent, is formed again
 // by FP64 FMAs (split_redo).  Outputs then are within (K + 4) 2^-53 |A||B| by
 // element, as the FMA loop's are by its a priori bound; measured on Gaussian,
 // graded (both ways, 0.5 to 8 decades), near-diagonal, sparse and 6-decade
 // random operands, K = 3 to 3000: at most 0.55 of that bound, root mean
-// square 0.1 to 2 of 2^-53 |A||B| where the FMA loop has 0.4 to 23 (and up to
-// 6 times the loop's where products graded apart stay just above the line).
+// square 0.05 to 7 times 2^-53 |A||B| where the FMA loop has 0.4 to 23 (and up
+// to 6 times the loop's where products graded apart stay just above the line).
 // The line is measured, H_eff of CAS(16,16) M=512: 2^13 without the root 0.6 %
-// of the outputs again, 2^14 without it 1.4 % and 7.4 ms, with it 0.6 ms;
-// 2^15 1.7 ms and errors halved; the check itself takes 0.8 ms of 8.5.  Plans whose
-// products are only summed into one number (an energy) leave it out: their
-// error counts against the norm, where the digits' is 0.4 to 0.9 of the FMA loop's.
+// of the outputs again, 2^14 without it 1.4 % and 7.4 ms, with it 0.5 ms;
+// 2^15 1.7 ms and errors halved; the check itself takes 1.0 ms of 8.6.  Plans
+// whose products are only summed into one number (an energy) leave it out:
+// their error counts against the norm, where the digits' is 0.4 to 0.9 of the
+// FMA loop's.
 //
 // Rows whose largest magnitude is not finite or outside 2^-323 .. 2^277
 // (all-zero rows are fine) and coefficients outside 2^-73 .. 2^77 send
@@ -308,7 +309,7 @@ struct Head {          // what the consumers need of one chunk, 64 bytes
   double alpha;
   int32_t ldc, mr, nr, flags;   // kFirst | kLast | kBeta | kEnd
   int32_t nh, kc, term, k0;     // 16-column halves; columns, GemmTerm and first column of the chunk
-  int32_t m0, n0, work, slack;  // slack: log2 of the square root of the piece's chunks
+  int32_t m0, n0, work, slack;
 };
 static_assert(sizeof(Head) == kHead, "stage header");
 enum { kFirst = 1, kLast = 2, kBeta = 4, kEnd = 8 };
@@ -350,7 +351,7 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
       const GemmOut o = outs[W.out];
       Head h;
       h.work = w;
-      h.slack = (31 - __clz(W.steps)) >> 1;
+      h.slack = W.slack;
       h.m0 = W.tm * XM;
       h.n0 = W.tn * XM;
       h.mr = min(XM, o.M - h.m0);
@@ -549,7 +550,7 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
 // 32 products), hence four outputs at once and the next term's record asked for early:
 // one output a warp at a time took twice as long, marks found by
 // scanning a bit map (uneven shares of them) five times as long on small plans.
-// H_eff of CAS(16,16) M=512: 0.6 ms for both stages, its 1-/2-RDM 2.5 ms in
+// H_eff of CAS(16,16) M=512: 0.5 ms for both stages, its 1-/2-RDM 2.5 ms in
 // 48 launches behind the host's planning.
 __global__ void __launch_bounds__(256, 3)
 split_redo_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
