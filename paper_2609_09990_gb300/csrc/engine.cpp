@@ -659,9 +659,10 @@ void Engine::upload(GemmPlan& p) {
 }
 
 // The split kernel's lists for the outputs `list` (chunks per tile, output):
-// every distinct operand block once, the chunks of every 64 x 64 tile, long
-// chains cut into pieces of about a sixth of an SM's share of all chunks (at
-// least 16: a piece costs a partial tile written and read).  The cuts depend
+// every distinct operand block once (blocks that are the first rows of another
+// are part of it), the chunks of every 64 x 64 tile, long chains cut into
+// pieces of about a sixth of an SM's share of all chunks (at least 16: a piece
+// costs a partial tile written and read).  The cuts depend
 // on the plan alone, so results do not depend on the device's load.
 void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>& list) const {
   p.operands.clear();
@@ -680,25 +681,37 @@ void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>&
   size_t cap = 64;
   while (cap < 4 * nterms) cap *= 2;
   std::vector<int> table(cap, -1);   // open addressing
+  auto pad8 = [](int rows) { return (rows + 7) / 8 * 8; };
+  auto place = [&](SplitOperand& o) {   // its records behind those before it
+    const int64_t rp = (o.rows + 7) / 8 * 8, chunks = (o.K + kSplitChunk - 1) / kSplitChunk;
+    const int last = o.K - (int)(chunks - 1) * kSplitChunk;
+    o.off = p.digit_bytes;
+    o.first = p.split_items;
+    // 7 digit planes of FP16 and a tail per row and chunk; the last chunk may be 16 wide
+    const int64_t bytes = (chunks - 1) * rp * (7 * 64 + kSplitTail) + rp * (7 * (last > 16 ? 64 : 32) + kSplitTail);
+    p.digit_bytes += (bytes + 127) / 128 * 128;
+    p.split_items += rp / 8 * chunks;
+  };
+  bool grown = false;
   auto operand = [&](const double* src, int ld, int rows, int K, bool kstrided) -> int {
     uint64_t x = (uint64_t)(uintptr_t)src >> 3;
-    x = (x ^ ((uint64_t)rows << 40) ^ ((uint64_t)K << 52) ^ (uint64_t)kstrided) * 0x9E3779B97F4A7C15ull;
+    x = (x ^ ((uint64_t)K << 48) ^ (uint64_t)kstrided) * 0x9E3779B97F4A7C15ull;
     for (size_t i = (x >> 20) & (cap - 1);; i = (i + 1) & (cap - 1)) {
       const int e = table[i];
       if (e < 0) {
         table[i] = (int)p.operands.size();
-        const int64_t rp = (rows + 7) / 8 * 8, chunks = (K + kSplitChunk - 1) / kSplitChunk;
-        const int last = K - (int)(chunks - 1) * kSplitChunk;
-        p.operands.push_back({src, ld, rows, K, kstrided, p.digit_bytes, p.split_items});
-        // 7 digit planes of FP16 and a tail per row and chunk; the last chunk may be 16 wide
-        const int64_t bytes =
-            (chunks - 1) * rp * (7 * 64 + kSplitTail) + rp * (7 * (last > 16 ? 64 : 32) + kSplitTail);
-        p.digit_bytes += (bytes + 127) / 128 * 128;
-        p.split_items += rp / 8 * chunks;
+        p.operands.push_back({src, ld, rows, K, kstrided, 0, 0});
+        place(p.operands.back());
         return table[i];
       }
-      const SplitOperand& o = p.operands[e];
-      if (o.src == src && o.ld == ld && o.rows == rows && o.K == K && o.kstrided == (int)kstrided) return e;
+      SplitOperand& o = p.operands[e];
+      if (o.src == src && o.ld == ld && o.K == K && o.kstrided == (int)kstrided) {
+        if (rows > o.rows) {   // terms of fewer rows use its first ones
+          o.rows = rows;
+          grown = true;
+        }
+        return e;
+      }
     }
   };
   const int64_t piece = std::max<int64_t>(16, all / (6 * num_sms) + 1);
@@ -714,7 +727,8 @@ void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>&
       const GemmTerm& g = p.terms[t];
       if (g.K <= 0) continue;
       const int a = operand(g.A, g.lda, o.M, g.K, g.flags & 1), b = operand(g.B, g.ldb, o.N, g.K, !(g.flags & 2));
-      p.sterms.push_back({p.operands[a].off, p.operands[b].off, (o.M + 7) / 8 * 8, (o.N + 7) / 8 * 8, g.K, t, g.alpha});
+      p.sterms.push_back(
+          {p.operands[a].off, p.operands[b].off, pad8(p.operands[a].rows), pad8(p.operands[b].rows), g.K, t, g.alpha});
       kstep.push_back(kstep.back() + (g.K + kSplitChunk - 1) / kSplitChunk);
     }
     const int64_t steps = kstep.back();
@@ -736,6 +750,21 @@ void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>&
                        pieces > 1 ? (int)p.part_slots - pieces + i : -1, slack});
         }
       }
+  }
+  if (grown) {   // operands that a later term has more rows of: all places and terms once more
+    p.split_items = p.digit_bytes = 0;
+    for (SplitOperand& o : p.operands) place(o);
+    size_t i = 0;
+    for (const auto& l : list) {
+      const GemmOut& o = p.outs[l.second];
+      for (int t = o.t0; t < o.t1; ++t) {
+        const GemmTerm& g = p.terms[t];
+        if (g.K <= 0) continue;
+        const SplitOperand& a = p.operands[operand(g.A, g.lda, o.M, g.K, g.flags & 1)];
+        const SplitOperand& b = p.operands[operand(g.B, g.ldb, o.N, g.K, !(g.flags & 2))];
+        p.sterms[i++] = {a.off, b.off, pad8(a.rows), pad8(b.rows), g.K, t, g.alpha};
+      }
+    }
   }
   std::vector<int> order;
   longest_first(work, order);

@@ -25,19 +25,18 @@
 // products in 70), next to the largest scale 2^e of a b that any chunk brought
 // (chunks in which no nonzero element meets another do not count).  An output
 // with (columns + 4) sum |A||B| below 2^14 digit units, less the square root
-// of the number of its chunks, whose errors are independent, is formed again
+// of the number of chunks, whose errors are independent, is formed again
 // by FP64 FMAs (split_redo).  Outputs then are within (K + 4) 2^-53 |A||B| by
 // element, as the FMA loop's are by its a priori bound; measured on Gaussian,
 // graded (both ways, 0.5 to 8 decades), near-diagonal, sparse and 6-decade
 // random operands, K = 3 to 3000: at most 0.55 of that bound, root mean
-// square 0.05 to 7 times 2^-53 |A||B| where the FMA loop has 0.4 to 23 (and up
-// to 6 times the loop's where products graded apart stay just above the line).
+// square 0.1 to 2 of 2^-53 |A||B| where the FMA loop has 0.4 to 23 (and up to
+// 6 times the loop's where products graded apart stay just above the line).
 // The line is measured, H_eff of CAS(16,16) M=512: 2^13 without the root 0.6 %
-// of the outputs again, 2^14 without it 1.4 % and 7.4 ms, with it 0.5 ms;
-// 2^15 1.7 ms and errors halved; the check itself takes 1.0 ms of 8.6.  Plans
-// whose products are only summed into one number (an energy) leave it out:
-// their error counts against the norm, where the digits' is 0.4 to 0.9 of the
-// FMA loop's.
+// of the outputs again, 2^14 without it 1.4 % and 7.4 ms, with it 0.6 ms;
+// 2^15 1.7 ms and errors halved; the check itself takes 0.8 ms of 8.5.  Plans whose
+// products are only summed into one number (an energy) leave it out: their
+// error counts against the norm, where the digits' is 0.4 to 0.9 of the FMA loop's.
 //
 // Rows whose largest magnitude is not finite or outside 2^-323 .. 2^277
 // (all-zero rows are fine) and coefficients outside 2^-73 .. 2^77 send
@@ -385,10 +384,11 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         }
         __syncwarp();
         if (lane < 16) {
-          const uint8_t* rec = digits + (side ? T.b : T.a) + (int64_t)chunk * (side ? T.rb : T.ra) * (NS * 64 + kTail) +
+          // the operand may have more rows than the output: its tile's planes are `pitch` apart
+          const int have = side ? T.rb : T.ra, pitch = min(XM, have - row0) * h.nh * 32;
+          const uint8_t* rec = digits + (side ? T.b : T.a) + (int64_t)chunk * have * (NS * 64 + kTail) +
                                (int64_t)row0 * row_bytes;
-          const int plane = rows * h.nh * 32;
-          bulk_copy(st + side * kRec + x * kPlane, rec + x * plane, x < NS ? plane : rows * kTail, &full[s]);
+          bulk_copy(st + side * kRec + x * kPlane, rec + x * pitch, x < NS ? rows * h.nh * 32 : rows * kTail, &full[s]);
         }
         if (++s == kStages) { s = 0; ph ^= 1; }
         k0 += XK;
@@ -550,7 +550,7 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
 // 32 products), hence four outputs at once and the next term's record asked for early:
 // one output a warp at a time took twice as long, marks found by
 // scanning a bit map (uneven shares of them) five times as long on small plans.
-// H_eff of CAS(16,16) M=512: 0.5 ms for both stages, its 1-/2-RDM 2.5 ms in
+// H_eff of CAS(16,16) M=512: 0.6 ms for both stages, its 1-/2-RDM 2.5 ms in
 // 48 launches behind the host's planning.
 __global__ void __launch_bounds__(256, 3)
 split_redo_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
@@ -615,21 +615,22 @@ split_redo_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict_
   }
 }
 
-// tiles whose chain was cut: the pieces' partial sums in their order
+// Tiles whose chain was cut: the pieces' partial sums in their order, a lane
+// per output (16 blocks a tile: with one, a plan of few tiles and a hundred
+// pieces each waited 300 us for its loads).
 __global__ void __launch_bounds__(256)
 split_sum_kernel(const GemmOut* __restrict__ outs, const SplitSum* __restrict__ sums, const double* __restrict__ part) {
   const SplitSum S = sums[blockIdx.x];
   const GemmOut o = outs[S.out];
-  const int m0 = S.tm * XM, n0 = S.tn * XM, mr = min(XM, o.M - m0), nr = min(XM, o.N - n0);
-  for (int x = threadIdx.x; x < mr * XM; x += 256) {
-    const int r = x / XM, c = x - r * XM;
-    if (c >= nr) continue;
-    const double* p = part + (int64_t)S.slot * XM * XM + x;
-    double v = 0.0;
-    for (int i = 0; i < S.count; ++i) v += p[(int64_t)i * XM * XM];
-    double* d = o.C + (int64_t)(m0 + r) * o.ldc + n0 + c;
-    *d = o.beta ? *d + v : v;
-  }
+  const int x = blockIdx.y * 256 + threadIdx.x, r = x / XM, c = x - r * XM;
+  const int m = S.tm * XM + r, n = S.tn * XM + c;
+  if (m >= o.M || n >= o.N) return;
+  const double* p = part + (int64_t)S.slot * XM * XM + x;
+  double v = 0.0;
+#pragma unroll 8
+  for (int i = 0; i < S.count; ++i) v += p[(int64_t)i * XM * XM];
+  double* d = o.C + (int64_t)m * o.ldc + n;
+  *d = o.beta ? *d + v : v;
 }
 
 }  // namespace
@@ -647,7 +648,7 @@ int launch_gemm_f64_split(const GemmPlan& p, int num_sms, int* err, cudaStream_t
                                                       p.d_part, p.d_weak, err, err + 1);
   if (guard)
     split_redo_kernel<<<3 * num_sms, 256, 0, s>>>(p.d_terms, p.d_outs, p.d_sterms, p.d_swork, p.d_part, p.d_weak);
-  if (!p.ssums.empty()) split_sum_kernel<<<(int)p.ssums.size(), 256, 0, s>>>(p.d_outs, p.d_ssums, p.d_part);
+  if (!p.ssums.empty()) split_sum_kernel<<<dim3(p.ssums.size(), XM * XM / 256), 256, 0, s>>>(p.d_outs, p.d_ssums, p.d_part);
   return 2 + guard + !p.ssums.empty();
 }
 

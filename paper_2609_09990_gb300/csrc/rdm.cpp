@@ -378,12 +378,13 @@ void Engine::rdms_ci(double* rdm1, double* rdm2) {
 //                      + d_qr Gamma_pstu + d_qr d_st gamma_pu,
 // and <E_pq E_rs E_tu> = D[qp] . (E_rs D[tu]) with D[tu] = E_tu C.  Gamma3
 // does not change when its index pairs (pq), (rs), (tu) change places, so one
-// order of each triple is computed, tu <= rs <= pq as numbers: for each rs the
-// rs + 1 vectors E_rs D[tu] and a Gram GEMM against the n^2 - rs vectors D[qp],
-// a sixth of all products.  The GEMMs of as many rs as fit 1 GiB of vectors
-// are one launch, each split over K until the launch has a few tiles for
-// every SM (CAS(9,9) M=96: 88 ms with one launch of a dozen tiles per rs and
-// all triples, 4.1 ms).
+// order of each triple is computed: pq <= rs <= tu in a list of the pairs that
+// has (pq) and (qp) next to each other.  For each rs the vectors E_rs D[tu],
+// tu >= rs, and a Gram GEMM against the first vectors D[qp], a sixth of all
+// products, and the D of every rs are the first rows of one operand.  The
+// GEMMs of as many rs as fit 1 GiB of vectors are one launch, or one for every
+// range of K whose digits fit 1 GiB (CAS(9,9) M=96: 88 ms with one launch of a
+// dozen tiles per rs and all triples).
 void Engine::rdm3(double* out) {
   int64_t NaS = 0, NbS = 0;
   double* C = expand_ci(NaS, NbS);
@@ -393,7 +394,21 @@ void Engine::rdm3(double* out) {
     dfree(C);
     throw Error(-1, "3-RDM: the determinant expansion needs 2 n^2 vectors of the determinant length (at most 64 GB)");
   }
-  auto excA = excitations(n, Na), excB = excitations(n, Nb);
+  // the pairs in the order (pp) or (pq) (qp), the place of each, and of its transpose
+  std::vector<int> pair, at(n2), swapped(n2);
+  for (int p = 0; p < n; ++p)
+    for (int q = p; q < n; ++q) {
+      pair.push_back(p * n + q);
+      if (q > p) pair.push_back(q * n + p);
+    }
+  for (int i = 0; i < n2; ++i) at[pair[i]] = i;
+  for (int i = 0; i < n2; ++i) swapped[i] = at[pair[i] % n * n + pair[i] / n];
+  auto ordered = [&](const std::vector<int>& exc) {
+    std::vector<int> o(exc.size());
+    for (size_t j = 0; j < exc.size(); ++j) o[j] = exc[j / n2 * n2 + pair[j % n2]];
+    return o;
+  };
+  auto excA = ordered(excitations(n, Na)), excB = ordered(excitations(n, Nb));
   int* d_excA = dalloc<int>(excA.size());
   int* d_excB = dalloc<int>(excB.size());
   CK(cudaMemcpyAsync(d_excA, excA.data(), excA.size() * sizeof(int), cudaMemcpyHostToDevice, stream));
@@ -402,73 +417,56 @@ void Engine::rdm3(double* out) {
   launch_apply_e_chunk(C, NbS, d_excA, d_excB, n2, 0, (int)NaS, D, stream);
   stats.launches++;
   CK(cudaGetLastError());
-  double* Dt = dalloc<double>((size_t)n2 * ndet);   // Dt[pq] = D[qp]
-  for (int i = 0; i < n2; ++i)
-    CK(cudaMemcpyAsync(Dt + (size_t)i * ndet, D + (size_t)(i % n * n + i / n) * ndet, ndet * sizeof(double),
-                       cudaMemcpyDeviceToDevice, stream));
-  // batches of rs: [first, last), their vectors in F
+  // batches of rs: [first, last), their n2 - rs vectors each in F
   std::vector<int> first{0};
   int64_t fvec = 0, fmax = 0;
   for (int rs = 0; rs < n2; ++rs) {
-    if (fvec > 0 && (fvec + rs + 1) * ndet > ((int64_t)1 << 27)) {
+    if (fvec > 0 && (fvec + n2 - rs) * ndet > ((int64_t)1 << 27)) {
       first.push_back(rs);
       fvec = 0;
     }
-    fvec += rs + 1;
+    fvec += n2 - rs;
     fmax = std::max(fmax, fvec);
   }
   first.push_back(n2);
   double* F = dalloc<double>((size_t)fmax * ndet);
-  std::vector<int64_t> off3(n2 + 1, 0);   // M3: (n2 - rs) x (rs + 1) per rs
-  for (int rs = 0; rs < n2; ++rs) off3[rs + 1] = off3[rs] + (int64_t)(n2 - rs) * (rs + 1);
+  // rows of D that rs needs: the transposes of the pairs up to it
+  auto rows = [&](int rs) { return std::max(rs, swapped[rs]) + 1; };
+  std::vector<int64_t> off3(n2 + 1, 0);   // M3: rows(rs) x (n2 - rs) per rs
+  for (int rs = 0; rs < n2; ++rs) off3[rs + 1] = off3[rs] + (int64_t)rows(rs) * (n2 - rs);
   double* M3 = dalloc<double>((size_t)off3[n2]);
   double* M2 = dalloc<double>((size_t)n2 * n2 + n2);
-  // products of rows of X with rows of Y (or one vector Y), all of a list in
-  // one launch: K split into equal parts, summed in a fixed order
-  struct Gram { const double* X; const double* Y; double* dst; int rows, cols; bool vec; };
+  // products of the first rows of D with the rows of Y (or one vector Y), all
+  // of a list in one launch for every range of K, whose pieces the plan cuts
+  struct Gram { const double* Y; double* dst; int rows, cols; bool vec; };
   auto grams = [&](const std::vector<Gram>& list) {
-    int64_t tiles = 0, elems = 0;
-    for (const Gram& g : list) {
-      tiles += (int64_t)((g.rows + kSplitTile - 1) / kSplitTile) * ((g.cols + kSplitTile - 1) / kSplitTile);
-      elems += (int64_t)g.rows * g.cols;
-    }
-    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>((8 * num_sms + tiles - 1) / tiles, ndet / 1024));
-    const int64_t step = (ndet + parts - 1) / parts;
-    double* Mp = dalloc<double>((size_t)parts * elems);
-    GemmPlan p;
-    p.result = true;
-    AxpyPlan ax;
-    int64_t at = 0;
-    for (const Gram& g : list) {
-      const int64_t len = (int64_t)g.rows * g.cols;
-      ax.outs.push_back({g.dst, len, (int)ax.terms.size(), 0});
-      for (int s = 0; s < parts; ++s, at += len) {
-        const int64_t k0 = (int64_t)s * step, k1 = std::min<int64_t>(ndet, k0 + step);
-        p.add_out(Mp + at, g.cols, g.rows, g.cols, 0);
-        if (k1 > k0)
-          p.add_term(g.X + k0, (int)ndet, g.Y + k0, g.vec ? 1 : (int)ndet, (int)(k1 - k0), g.vec ? 0 : 2, 1.0);
-        ax.terms.push_back({Mp + at, 1.0});
+    int64_t vecs = n2;
+    for (const Gram& g : list) vecs += g.cols;
+    // 14.25 bytes of digits an element
+    const int64_t most = std::max<int64_t>(4096, ((int64_t)1 << 32) / (57 * vecs)), ranges = (ndet + most - 1) / most;
+    for (int64_t u = 0; u < ranges; ++u) {
+      const int64_t k0 = ndet * u / ranges, k1 = ndet * (u + 1) / ranges;
+      GemmPlan p;
+      p.result = true;
+      for (const Gram& g : list) {
+        p.add_out(g.dst, g.cols, g.rows, g.cols, u > 0);
+        p.add_term(D + k0, (int)ndet, g.Y + k0, g.vec ? 1 : (int)ndet, (int)(k1 - k0), g.vec ? 0 : 2, 1.0);
       }
-      ax.outs.back().t1 = (int)ax.terms.size();
+      upload(p);
+      run(p);
+      release(p);
     }
-    upload(p);
-    run(p);
-    release(p);
-    upload(ax);
-    run(ax);
-    release(ax);
-    dfree(Mp);
   };
   // <E_qp C | E_rs C> and <E_qp C | C>
-  grams({{D, D, M2, n2, n2, false}, {D, C, M2 + (size_t)n2 * n2, n2, 1, true}});
+  grams({{D, M2, n2, n2, false}, {C, M2 + (size_t)n2 * n2, n2, 1, true}});
   for (size_t u = 0; u + 1 < first.size(); ++u) {
     std::vector<Gram> list;
     double* f = F;
     for (int rs = first[u]; rs < first[u + 1]; ++rs) {
-      launch_apply_e_vecs(D, rs + 1, NaS, NbS, d_excA, d_excB, n2, rs, f, stream);
+      launch_apply_e_vecs(D + (size_t)rs * ndet, n2 - rs, NaS, NbS, d_excA, d_excB, n2, rs, f, stream);
       stats.launches++;
-      list.push_back({Dt + (size_t)rs * ndet, f, M3 + off3[rs], n2 - rs, rs + 1, false});
-      f += (size_t)(rs + 1) * ndet;
+      list.push_back({f, M3 + off3[rs], rows(rs), n2 - rs, false});
+      f += (size_t)(n2 - rs) * ndet;
     }
     CK(cudaGetLastError());
     grams(list);
@@ -485,29 +483,28 @@ void Engine::rdm3(double* out) {
   CK(cudaMemcpyAsync(&nrm2, nrm_d, sizeof(double), cudaMemcpyDeviceToHost, stream));
   sync();
   stats.d2h += (h3.size() + h2.size() + 1) * sizeof(double);
-  for (void* q : {(void*)C, (void*)d_excA, (void*)d_excB, (void*)D, (void*)Dt, (void*)F, (void*)M3, (void*)M2,
-                  (void*)partial, (void*)nrm_d})
+  for (void* q : {(void*)C, (void*)d_excA, (void*)d_excB, (void*)D, (void*)F, (void*)M3, (void*)M2, (void*)partial,
+                  (void*)nrm_d})
     dfree(q);
   if (!(nrm2 > 0)) throw Error(-4, "MPS has zero norm in the determinant expansion");
   // gamma_pq = <E_pq> = <E_qp C | C>; Gamma_pqrs = <E_pq E_rs> - d_qr gamma_ps
   std::vector<double> g1(n2), g2((size_t)n2 * n2);
-  for (int p = 0; p < n; ++p)
-    for (int q = 0; q < n; ++q) g1[p * n + q] = h2[(size_t)n2 * n2 + q * n + p] / nrm2;
-  for (int p = 0; p < n; ++p)
-    for (int q = 0; q < n; ++q)
-      for (int r = 0; r < n; ++r)
-        for (int s2 = 0; s2 < n; ++s2) {
-          double v = h2[(size_t)(q * n + p) * n2 + r * n + s2] / nrm2;
-          if (q == r) v -= g1[p * n + s2];
-          g2[(size_t)(p * n + q) * n2 + r * n + s2] = v;
-        }
+  for (int i = 0; i < n2; ++i) g1[pair[i]] = h2[(size_t)n2 * n2 + swapped[i]] / nrm2;
+  for (int i = 0; i < n2; ++i)
+    for (int j = 0; j < n2; ++j) {
+      const int p = pair[i] / n, q = pair[i] % n, r = pair[j] / n, s2 = pair[j] % n;
+      double v = h2[(size_t)swapped[i] * n2 + j] / nrm2;
+      if (q == r) v -= g1[p * n + s2];
+      g2[(size_t)pair[i] * n2 + pair[j]] = v;
+    }
   auto G2 = [&](int p, int q, int r, int s2) { return g2[(size_t)(p * n + q) * n2 + r * n + s2]; };
   auto put = [&](int x, int y, int z, double v) { out[((size_t)x * n2 + y) * n2 + z] = v; };
-  for (int rs = 0; rs < n2; ++rs)
-    for (int pq = rs; pq < n2; ++pq)
-      for (int tu = 0; tu <= rs; ++tu) {
+  for (int j = 0; j < n2; ++j)
+    for (int i = 0; i <= j; ++i)
+      for (int k = j; k < n2; ++k) {
+        const int pq = pair[i], rs = pair[j], tu = pair[k];
         const int p = pq / n, q = pq % n, r = rs / n, s2 = rs % n, t = tu / n, u = tu % n;
-        double v = h3[off3[rs] + (int64_t)(pq - rs) * (rs + 1) + tu] / nrm2;
+        double v = h3[off3[j] + (int64_t)swapped[i] * (n2 - j) + k - j] / nrm2;
         if (q == t) v -= G2(p, u, r, s2);
         if (s2 == t) v -= G2(p, q, r, u);
         if (q == r) v -= G2(p, s2, t, u);
