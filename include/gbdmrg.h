@@ -184,7 +184,8 @@ int gbd_host_fiedler_order(int32_t n, const double *W, int32_t *order);
  * the MPS; it needs 2 n^2 vectors of the determinant length on the device,
  * so it is refused (GBD_ERR_ARG) above 64 GB of them (CAS(12,12): 2 GB).
  * In all the device holds n^2 vectors, another n^2 or 1 GiB if that is more,
- * and about 1.2 GiB of operands and partial sums of the products under way.
+ * and about 1.2 GiB of operands and partial sums of the products under way
+ * (without room for these, the products run on plain FP64 instructions).
  * GBD_ERR_STATE without a state. */
 int gbd_rdm3(gbd_ctx *ctx, double *rdm3);
 

@@ -313,6 +313,10 @@ int gbd_gemm_tc_selftest(gbd_ctx *ctx, int32_t M, int32_t N, int32_t K, int32_t 
  * (one FMA per product, terms in order, k ascending); beta 0 or 1.  GBD_ERR_ARG for sizes below 1, other flags or beta, or NULL. */
 int gbd_gemm_f64(gbd_ctx *ctx, int32_t M, int32_t N, int32_t K, int32_t nterms, int32_t flags, double alpha,
                  int32_t beta, const double *A, const double *B, double *C);
+/* Plans of results whose split operands, partial sums and marks would take more
+ * than `bytes` of device memory run on FMAs, as they do when the device has
+ * no room (no limit: INT64_MAX, the default).  GBD_ERR_ARG for bytes < 0. */
+int gbd_set_split_limit(gbd_ctx *ctx, int64_t bytes);
 /* Failure detection without a fault: one bounded mbarrier wait (the helper
  * every role of the tensor-core kernel uses).  arrive = 0: nothing completes
  * the barrier, the wait runs out after its poll limit (2^22 polls, a few

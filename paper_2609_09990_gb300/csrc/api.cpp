@@ -524,6 +524,15 @@ int gbd_set_tc_min_two_site(gbd_ctx* ctx, int64_t n) {
   });
 }
 
+int gbd_set_split_limit(gbd_ctx* ctx, int64_t bytes) {
+  return guarded(ctx, [&]() {
+    if (bytes < 0) return fail(ctx, GBD_ERR_ARG, "bytes < 0");
+    if (!ctx->eng) ctx->eng.reset(new gbd::Engine(ctx->device));
+    ctx->eng->split_limit = bytes;
+    return GBD_OK;
+  });
+}
+
 int gbd_probe_step(gbd_ctx* ctx, int32_t k, int32_t precision, int32_t fp64_refine, double tol, double* theta,
                    double* e64, double* r64) {
   return guarded(ctx, [&]() {

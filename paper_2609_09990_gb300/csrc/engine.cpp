@@ -587,26 +587,35 @@ void Engine::upload(GemmPlan& p) {
   // for small outputs.  A K step of it takes about as long for 8 x 8 outputs
   // as for 64 x 64, so it needs work to pay: at least 4096 products per step,
   // or a large output in all (everything on it: CAS(13,11) M=200 orbital RDMs
-  // 10.1 ms instead of 7.5 ms).
+  // 10.1 ms instead of 7.5 ms).  Where the device has no room for the digits
+  // (14 bytes an operand element), everything goes to the FMA kernel, which
+  // needs none.
   p.tiles.clear();
   std::vector<std::pair<int64_t, int>> fma;   // chain length and output
   int64_t fma_elems = 0;
   std::vector<std::pair<int64_t, int>> split;   // K steps and output
-  for (int o = 0; o < (int)p.outs.size(); ++o) {
-    const GemmOut& g = p.outs[o];
-    const int64_t elems = (int64_t)g.M * g.N;
-    if (elems == 0) continue;
-    int64_t ksum = 0, steps = 0;
-    for (int t = g.t0; t < g.t1; ++t) {
-      ksum += p.terms[t].K;
-      steps += (p.terms[t].K + kSplitChunk - 1) / kSplitChunk;
+  for (bool digits = p.result;; digits = false) {
+    fma.clear();
+    split.clear();
+    fma_elems = 0;
+    for (int o = 0; o < (int)p.outs.size(); ++o) {
+      const GemmOut& g = p.outs[o];
+      const int64_t elems = (int64_t)g.M * g.N;
+      if (elems == 0) continue;
+      int64_t ksum = 0, steps = 0;
+      for (int t = g.t0; t < g.t1; ++t) {
+        ksum += p.terms[t].K;
+        steps += (p.terms[t].K + kSplitChunk - 1) / kSplitChunk;
+      }
+      if (digits && elems * ksum >= std::min<int64_t>(4096 * std::max<int64_t>(steps, 1), 1 << 20)) {
+        split.push_back({steps, o});
+        continue;
+      }
+      fma.push_back({ksum, o});
+      fma_elems += elems;
     }
-    if (p.result && elems * ksum >= std::min<int64_t>(4096 * std::max<int64_t>(steps, 1), 1 << 20)) {
-      split.push_back({steps, o});
-      continue;
-    }
-    fma.push_back({ksum, o});
-    fma_elems += elems;
+    plan_split(p, split);
+    if (split.empty() || split_buffers(p)) break;
   }
   // The others: FMA tiles, the largest that still give every SM about eight
   // (fewer outputs a tile read more operands per product, fewer tiles leave
@@ -635,12 +644,6 @@ void Engine::upload(GemmPlan& p) {
       for (int n = 0; n < g.N; n += c.second)
         p.tiles.push_back({out, m, n, std::min(c.first, g.M - m) << 16 | std::min(c.second, g.N - n)});
   }
-  plan_split(p, split);
-  if (!p.swork.empty()) {
-    p.d_digits = dalloc<uint8_t>(p.digit_bytes);
-    p.d_part = dalloc<double>(p.part_slots * kSplitTile * kSplitTile);
-    if (!p.summed) p.d_weak = dalloc<uint2>(p.marks + 1);
-  }
   uint8_t* at[7];
   p.d_lists = upload_lists<7>({{p.terms.data(), p.terms.size() * sizeof(GemmTerm)},
                                {p.outs.data(), p.outs.size() * sizeof(GemmOut)},
@@ -656,6 +659,32 @@ void Engine::upload(GemmPlan& p) {
   p.d_sterms = (SplitTerm*)at[4];
   p.d_swork = (SplitWork*)at[5];
   p.d_ssums = (SplitSum*)at[6];
+}
+
+// The split kernel's buffers; false when the device has no room for them.  What
+// the call allocates after them has to fit as well: large ones leave a GiB.
+bool Engine::split_buffers(GemmPlan& p) {
+  const int64_t part = p.part_slots * kSplitTile * kSplitTile * (int64_t)sizeof(double);
+  const int64_t marks = p.summed ? 0 : (p.marks + 1) * (int64_t)sizeof(uint2), bytes = p.digit_bytes + part + marks;
+  if (bytes > split_limit || p.swork.size() >= (size_t)UINT32_MAX / kWeakPlaces) return false;
+  if (bytes > ((int64_t)256 << 20)) {
+    size_t room = 0, total = 0;
+    CK(cudaMemGetInfo(&room, &total));
+    cudaMemPool_t pool;
+    uint64_t reserved = 0, used = 0;
+    CK(cudaDeviceGetDefaultMemPool(&pool, device));
+    CK(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved));
+    CK(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
+    if ((int64_t)(room + reserved - used) < bytes + ((int64_t)1 << 30)) return false;
+  }
+  p.d_digits = try_alloc<uint8_t>(p.digit_bytes);
+  if (p.d_digits) p.d_part = try_alloc<double>(part / sizeof(double));
+  if (p.d_part && marks) p.d_weak = try_alloc<uint2>(p.marks + 1);
+  if (p.d_part && (p.d_weak || !marks)) return true;
+  for (void* q : {(void*)p.d_digits, (void*)p.d_part}) dfree(q);
+  p.d_digits = nullptr;
+  p.d_part = nullptr;
+  return false;
 }
 
 // The split kernel's lists for the outputs `list` (chunks per tile, output):

@@ -266,6 +266,7 @@ class Engine {
   // any level
   double tier2_floor_mult = 1.0;
   int hard_stag_iters = 8;
+  int64_t split_limit = INT64_MAX;  // plans of results whose split buffers take more bytes use the FMA kernel
   int64_t tc_min_two_site = 4096;   // smaller two-site states: reduced-precision schedules use FP64
   // tier-1 (BF16/TF32) Davidson iterations and steps of the current and the
   // previous sweep: a warm sweep whose predecessor averaged < 2 tier-1
@@ -329,13 +330,21 @@ class Engine {
   mutable size_t chk_size = 0;
   int num_sms = 152;
   template <class T>
-  T* dalloc(size_t n) {
+  T* try_alloc(size_t n) {   // nullptr when the device has no room
     void* p = nullptr;
     if (n == 0) n = 1;
     cudaError_t e = cudaMallocAsync(&p, n * sizeof(T), stream);
+    if (e != cudaSuccess) cudaGetLastError();   // reported here; the next launch's check must not find it
+    if (e == cudaErrorMemoryAllocation) return nullptr;
     if (e != cudaSuccess) throw Error(-2, std::string("device allocation failed: ") + cudaGetErrorString(e));
     allocs[(uintptr_t)p] = n * sizeof(T);
     return (T*)p;
+  }
+  template <class T>
+  T* dalloc(size_t n) {
+    T* p = try_alloc<T>(n);
+    if (!p) throw Error(-2, std::string("device allocation failed: ") + cudaGetErrorString(cudaErrorMemoryAllocation));
+    return p;
   }
   void check_range(const void* p, int64_t rows, int64_t cols, int64_t ld, const char* what) const;
   // the same test without the shared cache (safe on several host threads
@@ -352,6 +361,7 @@ class Engine {
   void dfree(void* p);
   void upload(GemmPlan& p);
   void plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>& list) const;
+  bool split_buffers(GemmPlan& p);
   void release(GemmPlan& p);
   void upload(AxpyPlan& p);
   void release(AxpyPlan& p);

@@ -104,6 +104,7 @@ def lib():
         "gbd_set_env_precision": (C.c_int, [vp, C.c_int32]),
         "gbd_gemm_tc_selftest": (C.c_int, [vp, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32,
                                            C.c_uint64, _dp, _dp]),
+        "gbd_set_split_limit": (C.c_int, [vp, C.c_int64]),
         "gbd_wait_flag_selftest": (C.c_int, [vp, C.c_int32]),
         "gbd_gemm_f64": (C.c_int, [vp, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_double, C.c_int32,
                                    _dp, _dp, _dp]),
@@ -390,6 +391,9 @@ class Context:
         self._check(self.L.gbd_gemm_tc_selftest(self.ptr, M, N, K, nterms, flags, prec, seed, C.byref(e),
                                                 C.byref(r)), "gbd_gemm_tc_selftest")
         return e.value, r.value
+
+    def set_split_limit(self, nbytes):
+        self._check(self.L.gbd_set_split_limit(self.ptr, int(nbytes)), "gbd_set_split_limit")
 
     def wait_flag_selftest(self, sigma):
         self._check(self.L.gbd_wait_flag_selftest(self.ptr, int(sigma)), "gbd_wait_flag_selftest")
