@@ -318,7 +318,7 @@ int gbd_gemm_f64(gbd_ctx *ctx, int32_t M, int32_t N, int32_t K, int32_t nterms, 
  * no room (no limit: INT64_MAX, the default).  GBD_ERR_ARG for bytes < 0. */
 int gbd_set_split_limit(gbd_ctx *ctx, int64_t bytes);
 /* Failure detection without a fault: one bounded mbarrier wait (the helper
- * every role of the tensor-core kernel uses).  arrive = 0: nothing completes
+ * every role of the tensor-core kernels uses).  arrive = 0: nothing completes
  * the barrier, the wait runs out after its poll limit (2^22 polls, a few
  * seconds) and
  * returns with *err_flag = 1, *waited_ok = 0; arrive = 1: *err_flag = 0,

@@ -70,6 +70,7 @@
 #include <cuda_fp16.h>
 
 #include "gbd_internal.h"
+#include "mbarrier.h"
 #include "smem_limit.h"
 
 namespace gbd {
@@ -90,38 +91,7 @@ constexpr uint32_t kMagicBits = 0x4B400000u;
 constexpr int kBadExp = 1 << 28;                // exponent of a row that the digits cannot hold
 constexpr int kStrong = 14;                     // the line of a weak output, in powers of two of digit units
 constexpr uint32_t kNoScale = 0x80008000u;      // no chunk yet
-constexpr uint32_t kWaitLimit = 1u << 22;
 
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(b)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_addr(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded wait; false (and *err raised) when the limit runs out or another role already failed
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err) {
-  for (uint32_t it = 0; it < kWaitLimit; ++it) {
-    if (mbar_try(b, parity)) return true;
-    if ((it & 1023u) == 1023u && *(volatile int*)err) return false;
-  }
-  atomicExch(err, 1);
-  return false;
-}
 __device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_addr(dst)),
@@ -380,7 +350,7 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         uint8_t* st = sm + s * 2 * kRec;
         if (lane == 0) {
           heads[s] = h;
-          mbar_expect(&full[s], (uint32_t)((ra + rb) * row_bytes));
+          mbar_expect_tx(&full[s], (uint32_t)((ra + rb) * row_bytes));
         }
         __syncwarp();
         if (lane < 16) {

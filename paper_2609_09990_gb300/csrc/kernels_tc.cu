@@ -30,6 +30,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "mbarrier.h"
 #include "smem_limit.h"
 #include "tc_gemm.h"
 
@@ -38,48 +39,14 @@ namespace gbd {
 namespace {
 
 constexpr int kThreads = 192;
-constexpr uint32_t kWaitLimit = 1u << 22;
 constexpr int kStageA = 128 * 128;          // bytes of one A box (128 rows x 128 B)
 constexpr int kSmemBudget = 232448;         // dynamic shared memory per CTA
 constexpr int kMaxStages = 8;
 
-__device__ __forceinline__ uint32_t saddr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(b)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(saddr(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded wait; false (and *err raised) when the limit runs out or another
-// role already failed
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err) {
-  for (uint32_t it = 0; it < kWaitLimit; ++it) {
-    if (mbar_try(b, parity)) return true;
-    if ((it & 1023u) == 1023u && *(volatile int*)err) return false;
-  }
-  atomicExch(err, 1);
-  return false;
-}
-
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(saddr(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(saddr(bar))
+      ::"r"(smem_addr(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar))
       : "memory");
 }
 
@@ -111,7 +78,7 @@ __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t
         : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(saddr(bar))
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
                : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -194,7 +161,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(saddr(tslot)) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_addr(tslot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
@@ -280,7 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         for (int k0 = 0; k0 < tm.k; k0 += kc) {
           if (!mbar_wait(&full[stage], ph, L.err)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t sa = saddr(base + stage * stage_bytes);
+          const uint32_t sa = smem_addr(base + stage * stage_bytes);
           const uint32_t sb = sa + kStageA;
           const int nk = min(kc, tm.k - k0) / kstep;
           const uint64_t ad = smem_desc(sa), bd = smem_desc(sb);
@@ -402,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
 }
 
 // ---------------------------------------------------------------- bounded waits
-// The failure path of every mbarrier wait above, on its own: one thread
+// The failure path of every mbarrier wait, on its own: one thread
 // waits (with the same bounded helper) on a barrier that is completed only
 // when `arrive` is set.  Without the arrival the wait runs out, raises
 // *err and the kernel returns; nothing hangs and no memory is touched
