@@ -30,6 +30,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "convert_bits.h"
 #include "mbarrier.h"
 #include "smem_limit.h"
 #include "tc_gemm.h"
@@ -94,12 +95,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ float to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
 }
 
 // true in one lane of a converged warp.  The issuing roles run in the elected
@@ -402,17 +397,6 @@ __device__ __forceinline__ int warp_find(int n, int64_t e, Key key) {
   return lo;
 }
 
-// x as FP64 by integer instructions (the conversion instruction would take the
-// FP64 pipe as long as the addition that follows)
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
-  const int sh = m < 0x00800000u ? __clz(m) - 8 : 0;   // subnormal: to the leading one
-  const uint32_t mm = m << sh;
-  uint32_t hi = (mm >> 3) + ((896u - sh) << 20);
-  hi += m >= 0x7F800000u ? 0x38000000u : 0u;            // infinities, NaN
-  return __hiloint2double((int)((m ? hi : 0u) | (u & 0x80000000u)), (int)(mm << 29));
-}
-
 // ---------------------------------------------------------------- split-K sum
 // one thread per output element; the slots are summed in FP64 with eight
 // interleaved partial sums combined in a fixed order (deterministic).  The
@@ -421,9 +405,7 @@ __device__ __forceinline__ double widen(float x) {
 // element together.  Bound by the FP64 pipe, one addition a value: a conversion
 // costs it as much, and one that is predicated off does too, hence widen and
 // the loop exits.  CAS(20,20) M=1024, 227 slots of 1.1 M elements at most: 573
-// -> 310 us; CAS(16,16) M=512, 137 of 0.29 M: 108 -> 71 us.  (One block per
-// column with a warp for every eighth slot: 660 us, lanes past the tile's rows
-// take the pipe too.)
+// -> 310 us; CAS(16,16) M=512, 137 of 0.29 M: 108 -> 71 us.
 __global__ void tc_reduce_kernel(const TcRed* __restrict__ tasks, int ntasks, int64_t total,
                                  const float* __restrict__ part, double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
@@ -467,34 +449,6 @@ __device__ __forceinline__ void store_conv(double x, int prec, void* hi, void* l
     reinterpret_cast<float*>(hi)[idx] = h;
     if (prec == kTF32x3) reinterpret_cast<float*>(lo)[idx] = to_tf32((float)(x - (double)h));
   }
-}
-
-// The same for TF32x3 and a finite value of ordinary size without the FP64
-// pipe, which takes 64 clocks for a warp's conversion or addition: x rounded
-// to FP32 and to TF32, and the rest x - hi (an integer of at most 43 bits in
-// units of x's last place) likewise.  Bit for bit what store_conv gives.
-__device__ __forceinline__ bool split_tf32(uint32_t xh, uint32_t xl, float* h, float* l) {
-  const int e = (int)((xh >> 20) & 0x7FFu) - 896;          // exponent field of the FP32 value
-  if (e < 80 || e > 250) return false;
-  const uint32_t m23 = (xh & 0xFFFFFu) << 3 | xl >> 29, rest = xl << 3;
-  uint32_t f = ((uint32_t)e << 23) + m23;
-  f += (rest > 0x80000000u || (rest == 0x80000000u && (m23 & 1u))) ? 1u : 0u;   // to nearest even
-  f = (f + 0x1000u) & 0xFFFFE000u;                          // to nearest, ties away
-  const int64_t mx = (int64_t)((uint64_t)((xh & 0xFFFFFu) | 0x100000u) << 32 | xl);
-  const int64_t mh = (int64_t)(f - ((uint32_t)e << 23) + 0x800000u) << 29;   // a carry into the exponent counts 2^23
-  const uint32_t sg = xh & 0x80000000u;
-  *h = __uint_as_float(f | sg);
-  *l = to_tf32(__ll2float_rn(sg ? mh - mx : mx - mh) * __uint_as_float((uint32_t)(e - 52) << 23));
-  return true;
-}
-
-// Likewise BF16, to nearest even from the FP64 bits.
-__device__ __forceinline__ bool round_bf16(uint32_t xh, uint32_t xl, uint16_t* b) {
-  const int e = (int)((xh >> 20) & 0x7FFu) - 896;
-  if (e < 1 || e > 253) return false;
-  const uint32_t v = (uint32_t)e << 7 | ((xh >> 13) & 0x7Fu), rest = xh << 19 | (xl ? 1u : 0u);
-  *b = (uint16_t)((xh >> 31 << 15) | (v + ((rest > 0x80000000u || (rest == 0x80000000u && (v & 1u))) ? 1u : 0u)));
-  return true;
 }
 
 // A block per sub-block.  Positions advance by additions (256 elements a step),
