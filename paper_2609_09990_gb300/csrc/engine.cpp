@@ -327,6 +327,7 @@ Engine::Engine(int dev) : device(dev) {
 
 Engine::~Engine() {
   cudaSetDevice(device);
+  if (stream) cudaStreamSynchronize(stream);   // kernels of a call that threw may still write the pinned sums
   if (tc_err_host) cudaFreeHost(tc_err_host);
   if (dav_host) cudaFreeHost(dav_host);
   for (auto& e : Lenv) free_env(e);
