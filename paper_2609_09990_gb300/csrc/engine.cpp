@@ -588,7 +588,10 @@ void Engine::upload(GemmPlan& p) {
   // for small outputs.  A K step of it takes about as long for 8 x 8 outputs
   // as for 64 x 64, so it needs work to pay: at least 4096 products per step,
   // or a large output in all (everything on it: CAS(13,11) M=200 orbital RDMs
-  // 10.1 ms instead of 7.5 ms).  Where the device has no room for the digits
+  // 10.1 ms instead of 7.5 ms).  The second bound is for long chains of few
+  // outputs: without it the 3-RDM of CAS(9,9), whose first operators have 1 x 81
+  // outputs over 15,876 columns, takes 5.3 ms instead of 3.9; at 2^18 the H_eff
+  // product of CAS(9,9) takes 2.28 instead of 2.15.  Where the device has no room for the digits
   // (14 bytes an operand element), everything goes to the FMA kernel, which
   // needs none.
   p.tiles.clear();
@@ -692,7 +695,9 @@ bool Engine::split_buffers(GemmPlan& p) {
 // every distinct operand block once (blocks that are the first rows of another
 // are part of it), the chunks of every 64 x 64 tile, long chains cut into
 // pieces of about a sixth of an SM's share of all chunks (at least 16: a piece
-// costs a partial tile written and read).  The cuts depend
+// costs a partial tile written and read).  With a third the 3-RDM of CAS(9,9)
+// takes 4.05 ms instead of 3.9, with a twelfth the 1-/2-RDM of CAS(16,16) 68.4
+// instead of 67.2; H_eff products differ by less than their runs.  The cuts depend
 // on the plan alone, so results do not depend on the device's load.
 void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>& list) const {
   p.operands.clear();

@@ -188,9 +188,10 @@ struct AxpyPlan {
 };
 constexpr int kAxpyChunk = 1024;   // output elements per work chunk of the block axpy
 
-// side of an output tile of the split kernel, and K columns per step
-// largest side of an FMA tile (shared memory: 3 steps of 32 columns of both sides, at most 51 KB)
+// Largest side of an FMA tile.  Its shared memory is 3 steps of 32 columns of
+// both sides: at most 32 KB, since a tile has at most 256 outputs (32 x 8).
 constexpr int kFmaSide = 32;
+// side of an output tile of the split kernel, and K columns per step
 constexpr int kSplitTile = 64, kSplitChunk = 32;
 constexpr int kSplitTail = 8;      // bytes behind a row's digits: exponent, mask of nonzero elements
 constexpr int kWeakPlaces = 128;   // places of a mark of weak outputs in a 64 x 64 tile

@@ -451,7 +451,11 @@ davidson_kernel(const double* __restrict__ V, const double* __restrict__ S, cons
     s = warp_tree(s);
     if (lane == 0) part[(int64_t)j * nunits + unit] = s;
   }
-  if (nblk > 64) return;   // davidson_finish_kernel adds the parts
+  // Long vectors: davidson_finish_kernel adds the parts.  Up to 64 blocks the
+  // last CTA to finish does, two loads a lane, and saves a launch; with 0 or 32
+  // the solves of CAS(6,6) and CAS(10,10) differ by less than their runs
+  // (41-44 and 160-206 ms), so the line is where the loads still fit.
+  if (nblk > 64) return;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) last = atomicAdd(count, 1) == (int)gridDim.x - 1;

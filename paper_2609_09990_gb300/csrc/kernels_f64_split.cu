@@ -25,44 +25,44 @@
 // products in 70), next to the largest scale 2^e of a b that any chunk brought
 // (chunks in which no nonzero element meets another do not count).  An output
 // with (columns + 4) sum |A||B| below 2^14 digit units, less the square root
-// of the number of chunks, whose errors are independent, is formed again
+// of the number of its chunks, whose errors are independent, is formed again
 // by FP64 FMAs (split_redo).  Outputs then are within (K + 4) 2^-53 |A||B| by
-// element, as the FMA loop's are by its a priori bound; measured on Gaussian,
+// element, as the FMA loop's are by its a priori bound.  Measured on Gaussian,
 // graded (both ways, 0.5 to 8 decades), near-diagonal, sparse and 6-decade
-// random operands, K = 3 to 3000: at most 0.55 of that bound, root mean
-// square 0.1 to 2 of 2^-53 |A||B| where the FMA loop has 0.4 to 23 (and up to
-// 6 times the loop's where products graded apart stay just above the line).
-// The line is measured, H_eff of CAS(16,16) M=512: 2^13 without the root 0.6 %
-// of the outputs again, 2^14 without it 1.4 % and 7.4 ms, with it 0.6 ms;
-// 2^15 1.7 ms and errors halved; the check itself takes 0.8 ms of 8.5.  Plans whose
-// products are only summed into one number (an energy) leave it out: their
-// error counts against the norm, where the digits' is 0.4 to 0.9 of the FMA loop's.
+// random operands, K = 3 to 3000: at most about half of that bound; root mean
+// square 0.05 to 7 times 2^-53 |A||B| where the FMA loop has 0.4 to 23, and at
+// most 6 times the loop's, where products graded apart stay just above the
+// line.  The line is measured, repeated outputs of the H_eff product of
+// CAS(16,16) M=512 (9.8 ms in all): without the root 2^12 0.9 ms, 2^13 2.3 and
+// 2^14 7.4 (1.4 % of the outputs), with it 0.5; the check itself takes 1.0.
+// Plans whose products are only summed into one number (an energy) leave it
+// out: their error counts against the norm, where the digits' is 0.4 to 0.9
+// of the FMA loop's on operands like a state's.
 //
 // Rows whose largest magnitude is not finite or outside 2^-323 .. 2^277
 // (all-zero rows are fine) and coefficients outside 2^-73 .. 2^77 send
 // their chunk through plain FMAs instead, so infinities, NaN and extreme
 // scales give what the FMA loop gives.
 //
-// Two kernels.  split_operands cuts every operand block of a plan once (a
+// Four kernels.  split_operands cuts every operand block of a plan once (a
 // block of the sigma build serves up to hundreds of products) into records
 // that the second one copies as they are: per 32-column chunk and 64 rows, the
-// seven digit planes, swizzled for ldmatrix, and the rows' exponents, all
-// contiguous.  gemm_f64_split multiplies 64 x 64 output tiles: one thread
-// streams the records of all chunks of all terms of all tiles of its CTA
-// through a ring of three stages by bulk copies, sixteen warps multiply.  Long
-// chains are cut into pieces with partial sums, added in a fixed order.
+// seven digit planes, swizzled for ldmatrix, and the rows' exponents and masks
+// of nonzero elements, all contiguous.  gemm_f64_split multiplies 64 x 64
+// output tiles: one warp streams the records of all chunks of all terms of all
+// tiles of its CTA through a ring of three stages by bulk copies, sixteen
+// warps multiply.  Long chains are cut into pieces with partial sums;
+// split_redo repeats weak outputs, split_sum adds the pieces in a fixed order.
 // What bounds it: a 64 x 64 x 32 chunk takes 4350 clocks of mma.sync (34
 // pairs) and 2048 clocks of FP64 FMAs, but the sub-blocks are small (35 % of
 // a chunk's products are real in CAS(16,16) M=512, 58 % in CAS(20,20)
 // M=1024), so that a warp has one 16 x 8 block per chunk and its latencies
 // count: loading fragments, putting the weights together, the barriers.
-// Four consumer warps a sub-core hide them best: with 96 registers a thread,
-// the B digits of a block and two planes of A in registers, the header left
-// in shared memory and no division in a chunk, the H_eff product of
-// CAS(16,16) M=512 (39 GFLOP) takes 8.4 ms (operands 0.8) and the one of
-// CAS(20,20) M=1024 (432 GFLOP) 53 ms; twelve warps with all A digits in
-// registers took 9.15 and 56 ms, eight 12 ms, a first kernel that split its
-// operands itself, tile by tile, 21 ms, and FP64 FMAs 79 and 562 ms.
+// Four consumer warps a sub-core hide them best: 96 registers a thread, the B
+// digits of a block and two planes of A in registers, the header left in
+// shared memory and no division in a chunk.  The H_eff product of CAS(16,16)
+// M=512 (39 GFLOP) takes 8.4 ms without the check by element (operands 0.8)
+// and the one of CAS(20,20) M=1024 (432 GFLOP) 53 ms, FP64 FMAs 79 and 562 ms.
 #include <algorithm>
 
 #include <cuda_runtime.h>
@@ -278,7 +278,7 @@ struct Head {          // what the consumers need of one chunk, 64 bytes
   double alpha;
   int32_t ldc, mr, nr, flags;   // kFirst | kLast | kBeta | kEnd
   int32_t nh, kc, term, k0;     // 16-column halves; columns, GemmTerm and first column of the chunk
-  int32_t m0, n0, work, slack;
+  int32_t m0, n0, work, slack;  // work, slack: its SplitWork and that one's slack
 };
 static_assert(sizeof(Head) == kHead, "stage header");
 enum { kFirst = 1, kLast = 2, kBeta = 4, kEnd = 8 };
@@ -517,11 +517,11 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
 // takes a mark (a place of a consumer warp, 32 lanes) four outputs at a time,
 // a lane every 32nd product of a term, its partial sums added as a tree.
 // Bound by the latency of the terms' chains (a term has one or two rounds of
-// 32 products), hence four outputs at once and the next term's record asked for early:
-// one output a warp at a time took twice as long, marks found by
-// scanning a bit map (uneven shares of them) five times as long on small plans.
-// H_eff of CAS(16,16) M=512: 0.6 ms for both stages, its 1-/2-RDM 2.5 ms in
-// 48 launches behind the host's planning.
+// 32 products), hence four outputs at once and the next term's record asked
+// for early: one at a time, from a bit map of marks, took 2.3 times as long on
+// the H_eff product of CAS(16,16) and 5.7 times on the small plans of
+// CAS(13,11) orbital RDMs.  Now 0.5 ms of that product's two stages; 2.5 ms in
+// the 48 launches of the 1-/2-RDM there, behind the host's planning.
 __global__ void __launch_bounds__(256, 3)
 split_redo_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
                   const SplitTerm* __restrict__ sterms, const SplitWork* __restrict__ work, double* __restrict__ part,
