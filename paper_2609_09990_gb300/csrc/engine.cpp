@@ -769,14 +769,13 @@ void Engine::plan_split(GemmPlan& p, const std::vector<std::pair<int64_t, int>>&
     const int64_t steps = kstep.back();
     const int slack = (63 - __builtin_clzll((uint64_t)std::max<int64_t>(steps, 1))) / 2;
     const int pieces = 2 * steps > 3 * piece ? (int)((steps + piece - 1) / piece) : 1;
+    p.marks += (int64_t)pieces * 4 * ((o.M + 15) / 16) * ((o.N + 7) / 8);   // four per 16 x 8 block
     for (int tm = 0; tm * kSplitTile < o.M; ++tm)
       for (int tn = 0; tn * kSplitTile < o.N; ++tn) {
         if (pieces > 1) {
           p.ssums.push_back({l.second, tm, tn, (int)p.part_slots, pieces});
           p.part_slots += pieces;
         }
-        p.marks += (int64_t)pieces * 4 * ((std::min(kSplitTile, o.M - tm * kSplitTile) + 15) / 16) *
-                   ((std::min(kSplitTile, o.N - tn * kSplitTile) + 7) / 8);   // four per 16 x 8 block
         for (int i = 0; i < pieces; ++i) {
           const int64_t s0 = steps * i / pieces, s1 = steps * (i + 1) / pieces;
           const int t = (int)(std::upper_bound(kstep.begin(), kstep.end(), s0) - kstep.begin()) - 1;

@@ -33,8 +33,8 @@
 // square 0.05 to 7 times 2^-53 |A||B| where the FMA loop has 0.4 to 23, and at
 // most 6 times the loop's, where products graded apart stay just above the
 // line.  The line is measured, repeated outputs of the H_eff product of
-// CAS(16,16) M=512 (9.8 ms in all): without the root 2^12 0.9 ms, 2^13 2.3 and
-// 2^14 7.4 (1.4 % of the outputs), with it 0.5; the check itself takes 1.0.
+// CAS(16,16) M=512 (9.2 ms in all): without the root 2^12 0.9 ms, 2^13 2.3 and
+// 2^14 7.4 (1.4 % of the outputs), with it 0.5; the check itself takes 0.3.
 // Plans whose products are only summed into one number (an energy) leave it
 // out: their error counts against the norm, where the digits' is 0.4 to 0.9
 // of the FMA loop's on operands like a state's.
@@ -435,13 +435,19 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
         // of A leave room for four warps a sub-core
         float f[8][4];
         const int brow = c8 + (lane & 7), bc = (lane >> 3) & 1;
-        weights<true>(f, ad0, smem_addr(rb + piece(brow, bc, nh)));
-        if (nh == 2) weights<false>(f, ad1, smem_addr(rb + piece(brow, 2 + bc, 2)));
-        float mag[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        // exponents of the four outputs' (columns + 4) sum |A||B|, a byte each:
+        // before the products, whose sums leave no registers for it (after
+        // them the two stages of CAS(16,16) M=512 took 8.6 ms instead of 7.9)
+        uint32_t strong = 0;
         if (kGuard) {
+          float mag[4] = {0.0f, 0.0f, 0.0f, 0.0f};
           magnitudes(mag, ad0, smem_addr(rb + piece(brow, bc, nh)));
           if (nh == 2) magnitudes(mag, ad1, smem_addr(rb + piece(brow, 2 + bc, 2)));
+#pragma unroll
+          for (int j = 0; j < 4; ++j) strong |= __float_as_uint(mag[j] * columns) >> 23 << (8 * j);
         }
+        weights<true>(f, ad0, smem_addr(rb + piece(brow, bc, nh)));
+        if (nh == 2) weights<false>(f, ad1, smem_addr(rb + piece(brow, 2 + bc, 2)));
         // asked for only now, so that the exponents arrive during the products
         if (__any_sync(0xffffffffu, badA || y0 == kBadExp || y1 == kBadExp)) {
           // the chunk of these 16 x 8 outputs by FP64 FMAs from the operands themselves
@@ -471,7 +477,7 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
           const int e = (j < 2 ? x0 : x1) + ((j & 1) ? y1 : y0) - 2100;
           if (kGuard && ((j < 2 ? xa.y : xb.y) & ((j & 1) ? yb.y : ya.y)) != 0)
             scale[i][j] = __vmaxs2(scale[i][j], (uint32_t)(e + aexp) * 0x10001u +
-                                                    ((__float_as_uint(mag[j] * columns) >> 7) & 0x00FF0000u) + 127 + kStrong);
+                                                    __byte_perm(strong, 0, 0x4044 | j << 8) + 127 + kStrong);
           acc[i][j] = fma(__ll2double_rn(v), __hiloint2double(ahi + (int)((uint32_t)e << 20), alo), acc[i][j]);
         }
       }
