@@ -42,7 +42,11 @@ extern "C" {
  * tensor-core tiers -- the named precision while ||r|| is large, then TF32x3
  * (split TF32 hi/lo, FP32 accumulation) -- then optional FP64 refinement.
  * Environments, H_eff diagonal, Davidson orthogonalisation, Rayleigh-Ritz,
- * decimation and the final energy are FP64 in every mode. */
+ * decimation and the final energy are FP64 in every mode.  Large products of
+ * results run on the tensor cores with operands split into digits: every
+ * element of a density matrix or an H_eff product keeps the a priori error
+ * bound of FP64 multiply-adds, energies keep their rounding error relative
+ * to the norm of H. */
 #define GBD_FP64 0
 #define GBD_TF32 1
 #define GBD_BF16 2

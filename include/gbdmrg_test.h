@@ -309,8 +309,11 @@ int gbd_gemm_tc_selftest(gbd_ctx *ctx, int32_t M, int32_t N, int32_t K, int32_t 
  * op(A_t) op(B_t), nterms terms of K columns, each block dense row-major and
  * back to back; flags 1 = A_t stored transposed (K x M), 2 = B_t stored
  * transposed (N x K), 4 = the product is a result (large ones run on the
- * tensor cores with exactly split operands) and not the input of an iteration
- * (one FMA per product, terms in order, k ascending); beta 0 or 1.  GBD_ERR_ARG for sizes below 1, other flags or beta, or NULL. */
+ * tensor cores with operands split into digits; an output whose digits would
+ * not keep FP64 accuracy is formed by FMAs, so that every element is within
+ * (K nterms + 4) 2^-53 sum |A||B||alpha|) and not the input of an iteration
+ * (one FMA per product, terms in order, k ascending); beta 0 or 1.
+ * GBD_ERR_ARG for sizes below 1, other flags or beta, or NULL. */
 int gbd_gemm_f64(gbd_ctx *ctx, int32_t M, int32_t N, int32_t K, int32_t nterms, int32_t flags, double alpha,
                  int32_t beta, const double *A, const double *B, double *C);
 /* Plans of results whose split operands, partial sums and marks would take more

@@ -522,11 +522,12 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
 // The outputs marked weak, by FP64 FMAs from the operands themselves: a warp
 // takes a mark (a place of a consumer warp, 32 lanes) four outputs at a time,
 // a lane every 32nd product of a term, its partial sums added as a tree.
-// Bound by the latency of the terms' chains (a term has one or two rounds of
-// 32 products), hence four outputs at once and the next term's record asked
-// for early: one at a time, from a bit map of marks, took 2.3 times as long on
-// the H_eff product of CAS(16,16) and 5.7 times on the small plans of
-// CAS(13,11) orbital RDMs.  Now 0.5 ms of that product's two stages; 2.5 ms in
+// Bound by the FP64 pipe where the chains are short (stage A of the H_eff
+// product of CAS(16,16): 80 % busy, with the trees) and by the latency of the
+// terms' records and loads where they are long, hence four outputs at once and
+// the next term's record asked for early: one at a time, from a bit map of
+// marks, took 2.3 times as long there and 5.7 times on the small plans of
+// CAS(13,11) orbital RDMs.  Now 0.5 ms of that product's two stages; 2.4 ms in
 // the 48 launches of the 1-/2-RDM there, behind the host's planning.
 __global__ void __launch_bounds__(256, 3)
 split_redo_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
