@@ -527,8 +527,8 @@ gemm_f64_split_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restr
 // terms' records and loads where they are long, hence four outputs at once and
 // the next term's record asked for early: one at a time, from a bit map of
 // marks, took 2.3 times as long there and 5.7 times on the small plans of
-// CAS(13,11) orbital RDMs.  Now 0.5 ms of that product's two stages; 2.4 ms in
-// the 48 launches of the 1-/2-RDM there, behind the host's planning.
+// CAS(13,11) orbital RDMs.  Now 0.5 ms of that product's two stages, and 2.4 ms
+// in the 48 launches of the 1-/2-RDM there (the call 65-66 -> 67 ms).
 __global__ void __launch_bounds__(256, 3)
 split_redo_kernel(const GemmTerm* __restrict__ terms, const GemmOut* __restrict__ outs,
                   const SplitTerm* __restrict__ sterms, const SplitWork* __restrict__ work, double* __restrict__ part,
